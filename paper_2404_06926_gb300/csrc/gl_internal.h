@@ -102,6 +102,10 @@ struct AllocFreeze {
 };
 bool alloc_frozen();
 
+// Floats per row of screen-space gradient sums: ten sums, padded so that rows
+// are 16-byte aligned (vector atomics and float4 loads).
+constexpr int kGradStride = 12;
+
 constexpr int kMaxViews = 64;   // views in one step (a keyframe window)
 constexpr int kDescRing = 8;    // pinned upload slots for view descriptors
 
@@ -149,7 +153,7 @@ struct View {
     DevBuf dkey2, gidx2;      // sort ping-pong
     DevBuf dup_off;           // u32 offset of the Gaussian's first instance
     DevBuf kmask;             // u64 kept-tile mask of the rectangle (all ones if it is not culled)
-    DevBuf g2d;               // float[10] screen-space gradient accumulators
+    DevBuf g2d;               // screen-space gradient accumulators (rows of kGradStride floats)
     // scan
     DevBuf bsum;              // u64 per scan block: instance offset, then duplication-part offset
     DevBuf count;             // u64[16]: I (0 after an overflow), overflow flag, N (depth
@@ -183,9 +187,9 @@ struct View {
     bool persistent = false;
     DevBuf work;              // int[2] unit counters (forward, backward)
     // deterministic backward: per (instance, pixel block) sums, reduced per
-    // (view, Gaussian) in a fixed order (floats: instances x blocks x 10)
+    // (view, Gaussian) in a fixed order (floats: instances x blocks x kGradStride)
     bool det = false;
-    DevBuf gpart;
+    DevBuf gpart, gmask;
     // segmented raster: tiles whose list holds >= 2 seg records are split
     // into segments of seg records (seg a power of two; 0: never split)
     int seg = 0;

@@ -370,8 +370,10 @@ k_params_bwd(GParams p, const ViewDesc* __restrict__ views, int V, const int* __
         geometry(mu, ls, q, sLg[r], cam, G);
 
         // screen-space gradients of this Gaussian, accumulated by the raster backward
-        float s[kNG];
-        for (int k = 0; k < kNG; k++) s[k] = g2d[(size_t)tv * kNG + k];
+        const float4* gr = reinterpret_cast<const float4*>(g2d + (size_t)tv * kGradStride);
+        const float4 s03 = gr[0], s47 = gr[1];
+        const float2 s89 = *reinterpret_cast<const float2*>(gr + 2);
+        const float s[kNG] = {s03.x, s03.y, s03.z, s03.w, s47.x, s47.y, s47.z, s47.w, s89.x, s89.y};
         const float du = -G.A * s[4] - G.B * s[5];
         const float dv = -G.C * s[5] - G.B * s[4];
         const float dA = -0.5f * s[6], dB = -s[7], dC = -0.5f * s[8];

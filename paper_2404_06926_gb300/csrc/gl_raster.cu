@@ -42,11 +42,12 @@
 // differ from a single running product by float rounding.
 //
 // Backward: every item walked back to front from its starting state (the
-// final transmittance and R = 0 for a whole tile); per hit, each lane sums
-// its D pixels' ten partial sums (colour 3, dL/dpower moments 6, depth 1),
-// the warp folds the 32 lanes with a transposed butterfly and ten lanes add
-// the totals to the Gaussian's accumulator (or, deterministic, store them
-// per instance and pixel block).
+// final transmittance and R = 0 for a whole tile).  Per hit a lane leaves two
+// numbers per pixel in shared memory, the blend weight and dL/d(exponent);
+// every 16 / D hits the warp turns over: lanes own hits instead of pixels and
+// form each hit's ten sums (colour 3, dL/dpower moments 6, depth 1) from
+// those rows, then add them to the Gaussian's accumulator with two vector
+// atomics (or, deterministic, store them per instance and pixel block).
 //
 // Scheduling: either one unit per warp of a grid that covers the bound on
 // units, or a persistent grid (sized to the resident warps) whose warps take
@@ -71,11 +72,10 @@ constexpr int wpb() { return NB <= 2 ? kWarpsPerBlock : 16 / NB; }
 template <int NB>
 constexpr int pf_slots() { return NB <= 2 ? NB : 1; }
 // resident CTAs per SM the kernels are compiled for: the forward passes fit
-// 64 registers (4 CTAs); the backward is faster with 76 registers (3 CTAs)
-// than squeezed into 64
+// 64 registers (4 CTAs)
 constexpr int kMinBlocks = 4;
-constexpr int kMinBlocksBwd = 3;
-constexpr int kNG = 10;   // screen-space gradient slots per Gaussian
+constexpr int kMinBlocksPg = 3;   // per-Gaussian backward
+constexpr int kNG = 10;           // screen-space gradient sums per Gaussian (rows of kGradStride floats)
 constexpr int kSegFields = 16;  // per (segment item, pixel): see below
 constexpr int kSegBatch = 4;    // segments whose state one load round trip brings (prefix, finish)
 
@@ -120,6 +120,7 @@ struct RasterGrad {
     // instance's emission index (sinst of its sorted position)
     float* part;
     const uint32_t* sinst;
+    uint32_t* pmask;             // per instance: the pixel blocks whose sums are in `part`
 };
 
 struct Unit {
@@ -618,83 +619,160 @@ __device__ __forceinline__ float warp_transpose_reduce16(float (&v)[16])
     return v[0] + __shfl_xor_sync(kFull, v[0], 1);
 }
 
-// Sum 9 per-lane values over the warp: values 0..7 by a transposed butterfly
-// (on return lane l holds the total of value l >> 2), value 8 by a plain one
-// (*t8 in every lane) -- 14 shuffles where the 16-slot fold takes 16.
-__device__ __forceinline__ float warp_transpose_reduce8(const float (&v)[16], float* t8)
+// Warps per CTA of the per-pixel backward: its staging takes 6.5 KB a warp at
+// the default shape, and CTAs of 4 warps (2 with 256-record batches) keep
+// every variant's within 48 KB of static shared memory.
+template <int NB>
+constexpr int wpb_bwd() { return NB <= 4 ? 4 : 2; }
+// registers: 96 a thread (20 warps per SM) at the default shape
+template <int NB, int D>
+constexpr int minb_bwd() { return (D > 1 ? 12 : (NB <= 2 ? 20 : 16)) / wpb_bwd<NB>(); }
+
+constexpr uint32_t kNoOwner = 0xffffffffu;
+
+// The per-pixel backward.  Bound by instruction issue (the deepest tiles'
+// latency in small frames).  Folding every hit's nine sums across the warp
+// took 37 of its ~100 instructions and the moments behind them ten more; the
+// turn-over replaces both by one 8-byte store per hit and about ten
+// instructions.  Two hits are evaluated together because a warp's chain, not
+// its throughput, ends the kernel on a single frame; the registers that takes
+// are worth more than warps: 64 / 80 / 96 / 128 a thread (32 / 24 / 20 / 16
+// warps per SM) gave 107 / 85 / 79 / 79 us on the 250k-Gaussian street at
+// 640x512 and 264 / 237 / 233 / 258 us on the 1M one at 1280x1024 (before: 126
+// and 306 us, and 1,218 -> 650 us with unsplit lists and depth gradients).
+// Staging of one warp: `sv` holds a row per
+// pending hit: (blend weight, dL/d(exponent)) of each of the block's 32 D
+// pixels.  The turn-over reads a row in parts of 16 pixels (two pixel rows),
+// one part per lane: the row stride S and the part stride PS (in float2) put
+// the 16 lanes of each half-warp phase of the 8-byte loads on different banks
+// (2 S mod 32 and 2 PS mod 32 are (2, -), (4, 2) and (8, 2) words for D = 1,
+// 2, 4).
+template <int NB, int D>
+struct BwdWarp {
+    static constexpr int H = 16 / D;                  // pending hits per turn-over
+    static constexpr int PARTS = 2 * D;               // lanes per hit, 16 pixels each
+    static constexpr int PS = D == 1 ? 16 : 17;
+    static constexpr int S = D == 1 ? 33 : (D == 2 ? 82 : 148);
+    static_assert(H * PARTS == 32 && S >= PARTS * PS, "one lane per (hit, part)");
+    // hit records from index 1, r1.w owner, r2.w list position (bits); entry 0
+    // is a record that reaches no pixel, the partner of an odd last hit
+    float4 r0[32 * NB + 1], r1[32 * NB + 1], r2[32 * NB + 1];
+    float4 pix[32 * D];                               // per pixel: dL/dC, dL/dD
+    float4 info[H];                                   // pending hits: tile-relative mean, owner (bits; kNoOwner: none)
+    float2 sv[H * S];
+};
+
+// The n pending hits' sums: lane (h, part) adds up hit h over the part's two
+// pixel rows, the parts are folded across the warp, and the lower half-warp
+// emits slots 0-3 and 8-9, the upper one slots 4-7.  The moments take dx, dy
+// per pixel (no expansion about the block), so they round as per-pixel sums.
+template <bool EXTRA, int NB, int D, bool DET>
+__device__ __forceinline__ void bwd_turn_over(const RasterArgs& A, const RasterGrad& G, const BwdWarp<NB, D>& W,
+                                              int n, float bx, float by, int wb, int lane)
 {
-    const unsigned lane = threadIdx.x & 31u;
-    float w[4];
-    {
-        const bool up = lane & 16u;
+    using BW = BwdWarp<NB, D>;
+    constexpr int H = BW::H;
+    const int h = lane % H, part = lane / H;
+    const float4 in = W.info[h];
+    const float2* row = W.sv + h * BW::S + part * BW::PS;
+    const float4* pc = W.pix + part * 16;
+    const float dya = in.y - (by + (float)(2 * part)), dyb = in.y - (by + (float)(2 * part + 1));
+    float c0 = 0.f, c1 = 0.f, c2 = 0.f, cD = 0.f;
+    float m0a = 0.f, m0b = 0.f, mxa = 0.f, mxb = 0.f, mxx = 0.f;
+#pragma unroll
+    for (int x = 0; x < 8; x++) {
+        const float2 va = row[x], vb = row[8 + x];
+        const float4 ga = pc[x], gb = pc[8 + x];
+        const float dx = in.x - (bx + (float)x), dx2 = dx * dx;
+        c0 = fmaf(va.x, ga.x, c0); c1 = fmaf(va.x, ga.y, c1); c2 = fmaf(va.x, ga.z, c2);
+        c0 = fmaf(vb.x, gb.x, c0); c1 = fmaf(vb.x, gb.y, c1); c2 = fmaf(vb.x, gb.z, c2);
+        if (EXTRA) cD = fmaf(vb.x, gb.w, fmaf(va.x, ga.w, cD));
+        m0a += va.y; m0b += vb.y;
+        mxa = fmaf(va.y, dx, mxa); mxb = fmaf(vb.y, dx, mxb);
+        mxx = fmaf(vb.y, dx2, fmaf(va.y, dx2, mxx));
+    }
+    // slots 0-3 (lo), 4-7 (hi), 8-9
+    float lo[4] = {c0, c1, c2, m0a + m0b};
+    float hi[4] = {mxa + mxb, fmaf(dya, m0a, dyb * m0b), mxx, fmaf(dya, mxa, dyb * mxb)};
+    float s8 = fmaf(dya * dya, m0a, dyb * dyb * m0b), s9 = cD;
+#pragma unroll
+    for (int off = H; off < 16; off <<= 1) {
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            const float send = up ? v[k] : v[k + 4];
-            const float keep = up ? v[k + 4] : v[k];
-            w[k] = keep + __shfl_xor_sync(kFull, send, 16);
+            lo[k] += __shfl_xor_sync(kFull, lo[k], off);
+            hi[k] += __shfl_xor_sync(kFull, hi[k], off);
+        }
+        s8 += __shfl_xor_sync(kFull, s8, off);
+        if (EXTRA) s9 += __shfl_xor_sync(kFull, s9, off);
+    }
+    const bool up = lane & 16;
+    float4 r;
+    float* rp = &r.x;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const float send = up ? lo[k] : hi[k], keep = up ? hi[k] : lo[k];
+        rp[k] = keep + __shfl_xor_sync(kFull, send, 16);
+    }
+    s8 += __shfl_xor_sync(kFull, s8, 16);
+    if (EXTRA) s9 += __shfl_xor_sync(kFull, s9, 16);
+    const uint32_t id = __float_as_uint(in.z);
+    if (h < n && (lane & 15) < H && id != kNoOwner) {
+        float* dst = DET ? G.part + ((size_t)id * A.nblk + wb) * kGradStride : G.g2d + (size_t)id * kGradStride;
+        if (DET) {
+            *reinterpret_cast<float4*>(dst + (up ? 4 : 0)) = r;
+            if (!up) {
+                *reinterpret_cast<float2*>(dst + 8) = make_float2(s8, EXTRA ? s9 : 0.0f);
+                atomicOr(G.pmask + id, 1u << wb);
+            }
+        } else {
+            atomicAdd(reinterpret_cast<float4*>(dst + (up ? 4 : 0)), r);
+            if (!up) {
+                if (EXTRA) atomicAdd(reinterpret_cast<float2*>(dst + 8), make_float2(s8, s9));
+                else atomicAdd(dst + 8, s8);
+            }
         }
     }
-    {
-        const bool up = lane & 8u;
-#pragma unroll
-        for (int k = 0; k < 2; k++) {
-            const float send = up ? w[k] : w[k + 2];
-            const float keep = up ? w[k + 2] : w[k];
-            w[k] = keep + __shfl_xor_sync(kFull, send, 8);
-        }
-    }
-    {
-        const bool up = lane & 4u;
-        const float send = up ? w[0] : w[1];
-        const float keep = up ? w[1] : w[0];
-        w[0] = keep + __shfl_xor_sync(kFull, send, 4);
-    }
-    w[0] += __shfl_xor_sync(kFull, w[0], 2);
-    w[0] += __shfl_xor_sync(kFull, w[0], 1);
-    float x = v[8];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(kFull, x, off);
-    *t8 = x;
-    return w[0];
 }
 
 template <bool EXTRA, int NB, int D, bool DET>
-__device__ __forceinline__ void bwd_item(int u, const RasterArgs& A, const RasterGrad& G, float4* sr0,
-                                         float4* sr1, float4* sr2, uint32_t* spos, uint32_t* sg, int lane)
+__device__ __forceinline__ void bwd_item(int u, const RasterArgs& A, const RasterGrad& G, BwdWarp<NB, D>& W, int lane)
 {
+    using BW = BwdWarp<NB, D>;
     Unit U;
     unit_of<D>(u, A, U);
     const LanePix<D> L(U, A.TS, lane);
     const unsigned lt = (1u << lane) - 1u;
-    float T[D], R0[D], R1[D], R2[D], RD[D], RO[D], g0[D], g1[D], g2[D], gD[D], gO[D];
+    // per pixel: transmittance, what is blended behind (colour; EXTRA: depth,
+    // opacity), the gradients of the pixel's outputs
+    float T[D], R[D][5], g0[D], g1[D], g2[D], gD[D], gO[D];
     uint32_t last[D];
     uint32_t wmax = 0;
 #pragma unroll
     for (int j = 0; j < D; j++) {
-        T[j] = 1.0f; R0[j] = R1[j] = R2[j] = RD[j] = RO[j] = 0.0f;
+        T[j] = 1.0f;
         g0[j] = g1[j] = g2[j] = gD[j] = gO[j] = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 5; k++) R[j][k] = 0.0f;
         last[j] = 0;
         if (L.inside[j]) {
             const size_t p = L.pix(U, j);
             last[j] = G.ncon[p];
-            if (U.nseg == 1) {
-                T[j] = G.Tfin[p];
-            } else {
-                const float* S = A.segstate;
-                const int q = L.p[j];
-                T[j] = S[seg_at(U.w, 0, q, A.TS)];
-                R0[j] = S[seg_at(U.w, 1, q, A.TS)];
-                R1[j] = S[seg_at(U.w, 2, q, A.TS)];
-                R2[j] = S[seg_at(U.w, 3, q, A.TS)];
-                RD[j] = S[seg_at(U.w, 4, q, A.TS)];
-                RO[j] = S[seg_at(U.w, 5, q, A.TS)];
-            }
             g0[j] = G.dL_drgb[3 * p]; g1[j] = G.dL_drgb[3 * p + 1]; g2[j] = G.dL_drgb[3 * p + 2];
             if (EXTRA) {
                 gD[j] = G.dL_ddepth ? G.dL_ddepth[p] : 0.0f;
                 gO[j] = G.dL_dopac ? G.dL_dopac[p] : 0.0f;
             }
+            if (U.nseg == 1) {
+                T[j] = G.Tfin[p];
+            } else {
+                const float* S = A.segstate;
+                const int i = L.p[j];
+                T[j] = S[seg_at(U.w, 0, i, A.TS)];
+#pragma unroll
+                for (int k = 0; k < (EXTRA ? 5 : 3); k++) R[j][k] = S[seg_at(U.w, 1 + k, i, A.TS)];
+            }
         }
+        W.pix[j * 32 + lane] = make_float4(g0[j], g1[j], g2[j], gD[j]);
         wmax = max(wmax, last[j]);
     }
 #pragma unroll
@@ -702,6 +780,13 @@ __device__ __forceinline__ void bwd_item(int u, const RasterArgs& A, const Raste
     // positions at or beyond the last contributor reach no pixel of the block
     const uint32_t end = min(U.re, U.trs + wmax);
     if (end <= U.rs) return;
+    const float bx = (float)U.lx0, by = (float)U.ly0;
+    int slot = 0;   // pending hits
+    if (lane == 0) {
+        W.r0[0] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        W.r1[0] = make_float4(0.0f, -3.0e38f, 0.0f, __uint_as_float(kNoOwner));
+        W.r2[0] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
     // batches from the back: [bstart, bstart + 32 NB) with bstart = end - 32 NB k, clipped at rs
     constexpr int BS = 32 * NB;
     constexpr int PF = pf_slots<NB>();
@@ -722,8 +807,9 @@ __device__ __forceinline__ void bwd_item(int u, const RasterArgs& A, const Raste
 #pragma unroll
         for (int b = 0; b < NB; b++) {
             const int sl = PF == NB ? b : 0;
-            const float4 c0 = n0[sl], c1 = n1[sl], c2 = n2[sl], c3 = n3[sl];
-            const uint32_t cg = ng[sl];
+            const float4 c0 = n0[sl], c3 = n3[sl];
+            float4 c1 = n1[sl], c2 = n2[sl];
+            c1.w = __uint_as_float(ng[sl]);
             const int64_t i = bstart + b * 32 + lane;
             // next: the same sub-batch of the batch before (whole-batch
             // prefetch), else the next sub-batch of this one, or the first
@@ -736,96 +822,88 @@ __device__ __forceinline__ void bwd_item(int u, const RasterArgs& A, const Raste
             const bool hit = i >= (int64_t)U.rs && box_hit(c3, L.bx0, L.bx1, L.by0, L.by1);
             const unsigned mask = __ballot_sync(kFull, hit);
             if (hit) {
-                const int k = nh + __popc(mask & lt);
-                sr0[k] = c0; sr1[k] = c1; sr2[k] = c2;
-                spos[k] = (uint32_t)(i - U.trs);
-                sg[k] = cg;
+                const int k = 1 + nh + __popc(mask & lt);
+                c2.w = __uint_as_float((uint32_t)(i - U.trs));
+                W.r0[k] = c0; W.r1[k] = c1; W.r2[k] = c2;
             }
             nh += __popc(mask);
         }
         __syncwarp();
-        for (int k = nh - 1; k >= 0; k--) {
-            const float4 a = sr0[k], b = sr1[k], c = sr2[k];
-            const uint32_t pos = spos[k];
-            // Branch-free: a pixel the hit does not reach takes alpha = 0,
-            // which leaves its R exactly unchanged (0 c + 1 R) and zeroes its
-            // sums; only T needs a select.  No per-hit zeroing of the sums and
-            // no divergent branch around the update.
-            float v[16];
-            bool any = false;
+        // Two hits at a time: their alphas are independent, only T and what is
+        // behind form a chain.  Branch-free, without selects where arithmetic
+        // does: a pixel a hit does not reach takes alpha = 0, which leaves T
+        // (T / 1) and the state behind exactly unchanged and zeroes its sums.
+        // (Hits that reach no pixel at all are too few to be worth a vote.)
+        for (int k = nh; k >= 1; k -= 2) {
+            float4 a[2], b[2], c[2];
 #pragma unroll
-            for (int j = 0; j < D; j++) {
-                float dx, dy, alpha;
-                bool capped;
-                const bool live = pair_eval_nb(a, b, L.px, L.py[j], dx, dy, alpha, capped) && pos < last[j];
-                const float al = live ? alpha : 0.0f;
-                T[j] = live ? __fdividef(T[j], 1.0f - al) : T[j];
-                const float wgt = al * T[j];
-                const float d0 = c.x - R0[j], d1 = c.y - R1[j], d2 = c.z - R2[j];
-                float dot = g0[j] * d0 + g1[j] * d1 + g2[j] * d2;
-                float dD = 0.0f, dO = 0.0f;
-                if (EXTRA) {
-                    dD = b.z - RD[j];
-                    dO = 1.0f - RO[j];
-                    dot += gD[j] * dD + gO[j] * dO;
-                }
-                // what is blended behind moves toward this Gaussian by alpha:
-                // R + alpha (c - R) = alpha c + (1 - alpha) R
-                R0[j] = fmaf(al, d0, R0[j]);
-                R1[j] = fmaf(al, d1, R1[j]);
-                R2[j] = fmaf(al, d2, R2[j]);
-                if (EXTRA) {
-                    RD[j] = fmaf(al, dD, RD[j]);
-                    RO[j] = fmaf(al, dO, RO[j]);
-                }
-                // dL/d(exponent) = alpha dL/dalpha = alpha T g . (c - R)
-                const float gp = capped ? 0.0f : wgt * dot;
-                const float gx = gp * dx, gy = gp * dy;
-                const float t[10] = {wgt * g0[j], wgt * g1[j], wgt * g2[j], gp, gx, gy, gx * dx, gx * dy, gy * dy,
-                                     EXTRA ? wgt * gD[j] : 0.0f};
+            for (int i = 0; i < 2; i++) { a[i] = W.r0[k - i]; b[i] = W.r1[k - i]; c[i] = W.r2[k - i]; }
+            float al[2][D];
 #pragma unroll
-                for (int q = 0; q < 10; q++) v[q] = j == 0 ? t[q] : v[q] + t[q];
-                any = any || live;
+            for (int i = 0; i < 2; i++) {
+                const uint32_t pos = __float_as_uint(c[i].w);
+#pragma unroll
+                for (int j = 0; j < D; j++) {
+                    float dx, dy, alpha;
+                    bool capped;
+                    const bool live = pair_eval_nb(a[i], b[i], L.px, L.py[j], dx, dy, alpha, capped) && pos < last[j];
+                    al[i][j] = live ? alpha : 0.0f;
+                }
             }
 #pragma unroll
-            for (int q = 10; q < 16; q++) v[q] = 0.0f;
-            if (__any_sync(kFull, any)) {
-                if (EXTRA) {
-                    const float r = warp_transpose_reduce16(v);
-                    const int q = lane >> 1;
-                    if ((lane & 1) == 0 && q < kNG) {
-                        if (DET) G.part[((size_t)sg[k] * A.nblk + U.wb) * kNG + q] = r;
-                        else atomicAdd(G.g2d + (size_t)sg[k] * kNG + q, r);
+            for (int i = 0; i < 2; i++) {
+                float2* sv = W.sv + (slot + i) * BW::S;
+#pragma unroll
+                for (int j = 0; j < D; j++) {
+                    const float al_ = al[i][j];
+                    T[j] = __fdividef(T[j], 1.0f - al_);
+                    const float wgt = al_ * T[j];
+                    // dL/dalpha = T g . (c - R); what is blended behind moves
+                    // toward this Gaussian by alpha.  (Keeping only g . R of
+                    // the colour behind saves four instructions and loses
+                    // digits of the pose gradient: c is close to R.)
+                    const float d0 = c[i].x - R[j][0], d1 = c[i].y - R[j][1], d2 = c[i].z - R[j][2];
+                    float dot = g0[j] * d0 + g1[j] * d1 + g2[j] * d2;
+                    R[j][0] = fmaf(al_, d0, R[j][0]);
+                    R[j][1] = fmaf(al_, d1, R[j][1]);
+                    R[j][2] = fmaf(al_, d2, R[j][2]);
+                    if (EXTRA) {
+                        const float dD = b[i].z - R[j][3], dO = 1.0f - R[j][4];
+                        dot += gD[j] * dD + gO[j] * dO;
+                        R[j][3] = fmaf(al_, dD, R[j][3]);
+                        R[j][4] = fmaf(al_, dO, R[j][4]);
                     }
-                } else {
-                    // nine live slots (no depth or opacity gradient)
-                    float r8;
-                    const float r = warp_transpose_reduce8(v, &r8);
-                    const int q = (lane & 3) == 0 ? (int)(lane >> 2) : (lane == 1 ? 8 : -1);
-                    if (q >= 0) {
-                        const float val = q == 8 ? r8 : r;
-                        if (DET) G.part[((size_t)sg[k] * A.nblk + U.wb) * kNG + q] = val;
-                        else atomicAdd(G.g2d + (size_t)sg[k] * kNG + q, val);
-                    }
+                    // dL/d(exponent) = alpha dL/dalpha, none at the cap
+                    const float gp = al_ < kAlphaMax ? wgt * dot : 0.0f;
+                    const int p = j * 32 + lane;
+                    sv[p + (p >> 4) * (BW::PS - 16)] = make_float2(wgt, gp);
                 }
+                if (lane == 0) W.info[slot + i] = make_float4(a[i].x, a[i].y, b[i].w, 0.0f);
+            }
+            slot += 2;
+            if (slot == BW::H) {
+                __syncwarp();
+                bwd_turn_over<EXTRA, NB, D, DET>(A, G, W, BW::H, bx, by, U.wb, lane);
+                slot = 0;
+                __syncwarp();
             }
         }
         __syncwarp();
     }
+    if (slot > 0) bwd_turn_over<EXTRA, NB, D, DET>(A, G, W, slot, bx, by, U.wb, lane);
+    __syncwarp();
 }
 
 template <bool EXTRA, int NB, int D, bool DET>
-__global__ void __launch_bounds__(32 * wpb<NB>(), kMinBlocksBwd * kWarpsPerBlock / wpb<NB>())
-k_raster_bwd(RasterArgs A, RasterGrad G)
+__global__ void __launch_bounds__(32 * wpb_bwd<NB>(), minb_bwd<NB, D>()) k_raster_bwd(RasterArgs A, RasterGrad G)
 {
-    constexpr int WPB = wpb<NB>();
-    __shared__ float4 sr0[WPB][32 * NB], sr1[WPB][32 * NB], sr2[WPB][32 * NB];
-    __shared__ uint32_t spos[WPB][32 * NB], sg[WPB][32 * NB];
+    constexpr int WPB = wpb_bwd<NB>();
+    __shared__ BwdWarp<NB, D> sw[WPB];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int nunits = units_of(A, false);
     int u = A.work ? next_unit(A.work, lane) : blockIdx.x * WPB + w;
     while (u < nunits) {
-        bwd_item<EXTRA, NB, D, DET>(u, A, G, sr0[w], sr1[w], sr2[w], spos[w], sg[w], lane);
+        bwd_item<EXTRA, NB, D, DET>(u, A, G, sw[w], lane);
         if (!A.work) break;
         u = next_unit(A.work, lane);
     }
@@ -871,11 +949,12 @@ template <bool EXTRA, bool DET>
 __device__ __forceinline__ void pg_flush(const RasterArgs& A, const RasterGrad& G, int wb, uint32_t g,
                                          const float (&acc)[kNG])
 {
-    constexpr int NQ = EXTRA ? kNG : kNG - 1;
+    constexpr int NQ = EXTRA || DET ? kNG : kNG - 1;   // deterministic rows are stored whole
+    if (DET) atomicOr(G.pmask + g, 1u << wb);
 #pragma unroll
     for (int q = 0; q < NQ; q++) {
-        if (DET) G.part[((size_t)g * A.nblk + wb) * kNG + q] = acc[q];
-        else atomicAdd(G.g2d + (size_t)g * kNG + q, acc[q]);
+        if (DET) G.part[((size_t)g * A.nblk + wb) * kGradStride + q] = acc[q];
+        else atomicAdd(G.g2d + (size_t)g * kGradStride + q, acc[q]);
     }
 }
 
@@ -1024,10 +1103,11 @@ __device__ __forceinline__ void bwd_item_pg(int u, const RasterArgs& A, const Ra
                 if (__any_sync(kFull, on)) {
                     const float r = warp_transpose_reduce16(v);
                     const int q = lane >> 1;
-                    if ((lane & 1) == 0 && q < (EXTRA ? kNG : kNG - 1)) {
+                    if ((lane & 1) == 0 && q < (EXTRA || DET ? kNG : kNG - 1)) {
                         const uint32_t g = W.qg[k];
-                        if (DET) G.part[((size_t)g * A.nblk + U.wb) * kNG + q] = r;
-                        else atomicAdd(G.g2d + (size_t)g * kNG + q, r);
+                        if (DET && lane == 0) atomicOr(G.pmask + g, 1u << U.wb);
+                        if (DET) G.part[((size_t)g * A.nblk + U.wb) * kGradStride + q] = r;
+                        else atomicAdd(G.g2d + (size_t)g * kGradStride + q, r);
                     }
                 }
             }
@@ -1105,7 +1185,7 @@ __device__ __forceinline__ void bwd_item_pg(int u, const RasterArgs& A, const Ra
 }
 
 template <bool EXTRA, bool DET>
-__global__ void __launch_bounds__(32 * kWarpsPerBlock, kMinBlocksBwd)
+__global__ void __launch_bounds__(32 * kWarpsPerBlock, kMinBlocksPg)
 k_raster_bwd_pg(RasterArgs A, RasterGrad G)
 {
     __shared__ PgWarp sw[kWarpsPerBlock];
@@ -1119,29 +1199,92 @@ k_raster_bwd_pg(RasterArgs A, RasterGrad G)
     }
 }
 
-// Deterministic gradient sums: for each (view, Gaussian) pair, its instances
-// (emission indices dup_off .. dup_off + touched) and each instance's pixel
-// blocks in ascending order.
-__global__ void k_part_reduce(const float* __restrict__ part, const uint32_t* __restrict__ touched,
-                              const uint32_t* __restrict__ dup_off, int nblk, int64_t pairs,
-                              const uint64_t* __restrict__ ctl, uint64_t cap, float* __restrict__ g2d)
+// Deterministic gradient sums: each (view, Gaussian) pair's instances
+// (emission indices dup_off .. dup_off + touched), of each the pixel blocks
+// its mask names.  Four lanes share a row (three of them hold its float4s)
+// and a pair's instances are dealt to row streams: two of them for a pair of
+// up to kHeavyPair instances (four pairs per warp), eight -- the warp -- for
+// the others, one pair after the other.  The streams' sums are then added in
+// a fixed order.  Only written rows are read, so neither the rows nor the
+// blocks without a hit need clearing.  Bound by the latency of the pairs with
+// hundreds of instances: 32 masks come in one load, the four pairs of a warp
+// lie a quarter of all pairs apart (near Gaussians are neighbours in the
+// map).  A thread per pair over every row, 173 us and a memset of the rows
+// (115 MB, 18 us) -> 66 us (250k Gaussians, street, 640x512).
+constexpr uint32_t kHeavyPair = 8;
+
+// acc += the rows of one instance that its mask m names (this lane's float4).
+__device__ __forceinline__ void part_rows(const float* __restrict__ part, uint64_t e, uint32_t m, int nblk, int f,
+                                          float4& acc)
+{
+    const float4* row = reinterpret_cast<const float4*>(part + (size_t)e * nblk * kGradStride) + f;
+    for (int b0 = 0; b0 < nblk; b0 += 8) {
+        const uint32_t mb = f < 3 ? m >> b0 : 0u;
+        float4 v[8];
+#pragma unroll
+        for (int b = 0; b < 8; b++)
+            if ((mb >> b) & 1u) v[b] = row[(b0 + b) * (kGradStride / 4)];
+#pragma unroll
+        for (int b = 0; b < 8; b++)
+            if ((mb >> b) & 1u) { acc.x += v[b].x; acc.y += v[b].y; acc.z += v[b].z; acc.w += v[b].w; }
+    }
+}
+
+__device__ __forceinline__ void fold_streams(float4& a, int off)
+{
+    a.x += __shfl_xor_sync(kFull, a.x, off);
+    a.y += __shfl_xor_sync(kFull, a.y, off);
+    a.z += __shfl_xor_sync(kFull, a.z, off);
+    a.w += __shfl_xor_sync(kFull, a.w, off);
+}
+
+__global__ void __launch_bounds__(256)
+k_part_reduce(const float* __restrict__ part, const uint32_t* __restrict__ pmask,
+              const uint32_t* __restrict__ touched, const uint32_t* __restrict__ dup_off, int nblk, int64_t pairs,
+              const uint64_t* __restrict__ ctl, uint64_t cap, float* __restrict__ g2d)
 {
     const bool overflow = ctl[1] != 0;   // the step's instances did not fit: nothing was written
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < pairs;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        float acc[kNG];
+    const int lane = threadIdx.x & 31, f = lane & 3;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5), quarter = (pairs + 3) / 4;
+    for (int64_t t0 = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t0 < quarter; t0 += warps) {
+        const int64_t t = t0 + (lane >> 3) * quarter;
+        uint32_t cnt = t < pairs ? touched[t] : 0u;
+        const uint64_t first = cnt ? dup_off[t] : 0u;
+        if (overflow || first + cnt > cap) cnt = 0;
+        const bool heavy = cnt > kHeavyPair;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        const uint32_t light = heavy ? 0u : cnt;
+        // lane k of a pair's eight holds the mask of its instance k
+        const uint32_t lm = (uint32_t)(lane & 7) < light ? pmask[first + (lane & 7)] : 0u;
+        const int s = (lane >> 2) & 1;
 #pragma unroll
-        for (int q = 0; q < kNG; q++) acc[q] = 0.0f;
-        const uint32_t cnt = touched[t];
-        if (cnt && !overflow && (uint64_t)dup_off[t] + cnt <= cap) {
-            const float* p = part + (size_t)dup_off[t] * nblk * kNG;
-            for (uint32_t e = 0; e < cnt * (uint32_t)nblk; e++, p += kNG) {
-#pragma unroll
-                for (int q = 0; q < kNG; q++) acc[q] += p[q];
-            }
+        for (int i = 0; i < (int)kHeavyPair; i += 2) {
+            const uint32_t m = __shfl_sync(kFull, lm, (lane & ~7) + i + s);
+            if (m) part_rows(part, first + i + s, m, nblk, f, acc);
         }
+        fold_streams(acc, 4);
+        for (unsigned left = __ballot_sync(kFull, heavy && (lane & 7) == 0); left; left &= left - 1) {
+            const int src = __ffs(left) - 1;
+            const uint64_t hf = __shfl_sync(kFull, first, src);
+            const uint32_t hc = __shfl_sync(kFull, cnt, src);
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+            uint32_t hm = (uint32_t)lane < hc ? pmask[hf + lane] : 0u;
+            for (uint32_t e0 = 0; e0 < hc; e0 += 32) {
+                const uint32_t cur = hm;
+                hm = e0 + 32 + lane < hc ? pmask[hf + e0 + 32 + lane] : 0u;
 #pragma unroll
-        for (int q = 0; q < kNG; q++) g2d[(size_t)t * kNG + q] = acc[q];
+                for (int i = 0; i < 4; i++) {
+                    const int k = i * 8 + (lane >> 2);
+                    const uint32_t m = __shfl_sync(kFull, cur, k);
+                    if (m) part_rows(part, hf + e0 + k, m, nblk, f, a);
+                }
+            }
+            fold_streams(a, 4);
+            fold_streams(a, 8);
+            fold_streams(a, 16);
+            if ((lane >> 3) == (src >> 3)) acc = a;
+        }
+        if (t < pairs && (lane & 7) < 3) reinterpret_cast<float4*>(g2d + (size_t)t * kGradStride)[f] = acc;
     }
 }
 
@@ -1284,8 +1427,8 @@ void fwd_launch(const RasterArgs& A, const RasterOut& O, int64_t units, int64_t 
 template <bool EXTRA, int NB, int D, bool DET>
 void bwd_launch(const RasterArgs& A, const RasterGrad& G, int64_t units, bool persistent, cudaStream_t s)
 {
-    const int grid = grid_for(k_raster_bwd<EXTRA, NB, D, DET>, units, persistent, wpb<NB>());
-    k_raster_bwd<EXTRA, NB, D, DET><<<grid, 32 * wpb<NB>(), 0, s>>>(A, G);
+    const int grid = grid_for(k_raster_bwd<EXTRA, NB, D, DET>, units, persistent, wpb_bwd<NB>());
+    k_raster_bwd<EXTRA, NB, D, DET><<<grid, 32 * wpb_bwd<NB>(), 0, s>>>(A, G);
 }
 
 template <bool EXTRA, bool DET>
@@ -1397,7 +1540,7 @@ gl_status raster_backward(View& v, const float* dL_drgb, const float* dL_ddepth,
                           const float* dL_dopac, cudaStream_t s)
 {
     const size_t pairs = (size_t)v.n * v.V;
-    GL_TRY(v.g2d.reserve(sizeof(float) * kNG * std::max<size_t>(pairs, 1)));
+    GL_TRY(v.g2d.reserve(sizeof(float) * kGradStride * std::max<size_t>(pairs, 1)));
     GL_TRY(check_exec(v));
     GL_TRY(v.work.reserve(32));
     PhaseScope ps(v.prof, PH_RASTER_BWD, s);
@@ -1405,7 +1548,7 @@ gl_status raster_backward(View& v, const float* dL_drgb, const float* dL_ddepth,
     // the per-Gaussian backward works on 8x4 pixel blocks whatever the
     // forward's pixels per lane
     const int nblk = v.pg ? v.Ts * v.Ts / 32 : blocks_per_tile(v);
-    if (!det) GL_CUDA_TRY(cudaMemsetAsync(v.g2d.p, 0, sizeof(float) * kNG * pairs, s));
+    if (!det) GL_CUDA_TRY(cudaMemsetAsync(v.g2d.p, 0, sizeof(float) * kGradStride * pairs, s));
     if (v.ntiles == 0 || v.I == 0) return GL_OK;
     int* work = nullptr;
     if (v.persistent) {
@@ -1415,16 +1558,18 @@ gl_status raster_backward(View& v, const float* dL_drgb, const float* dL_ddepth,
     RasterArgs A = make_args(v, work);
     A.nblk = nblk;
     RasterGrad G{v.Tfin.as<float>(), v.ncon.as<uint32_t>(), dL_drgb, dL_ddepth, dL_dopac, v.g2d.as<float>(),
-                 nullptr, v.sorted_inst};
+                 nullptr, v.sorted_inst, nullptr};
     const size_t cap = v.itile.bytes / 4;
     if (det) {
-        // every instance's block sums, zero where a block has no hit; the
-        // instance count is bounded by the capacity when it is known on the
-        // device only
+        // every instance's block sums, and a mask of the blocks that have any;
+        // the instance count is bounded by the capacity when it is known on
+        // the device only
         const size_t inst = v.I > 0 ? (size_t)v.I : cap;
-        GL_TRY(v.gpart.reserve(sizeof(float) * kNG * (size_t)nblk * std::max<size_t>(cap, 1)));
-        GL_CUDA_TRY(cudaMemsetAsync(v.gpart.p, 0, sizeof(float) * kNG * (size_t)nblk * inst, s));
+        GL_TRY(v.gpart.reserve(sizeof(float) * kGradStride * (size_t)nblk * std::max<size_t>(cap, 1)));
+        GL_TRY(v.gmask.reserve(sizeof(uint32_t) * std::max<size_t>(cap, 1)));
+        GL_CUDA_TRY(cudaMemsetAsync(v.gmask.p, 0, sizeof(uint32_t) * inst, s));
         G.part = v.gpart.as<float>();
+        G.pmask = v.gmask.as<uint32_t>();
     }
     const int64_t units = work_items_bound(v) * nblk;
     if (dL_ddepth != nullptr || dL_dopac != nullptr)
@@ -1433,8 +1578,9 @@ gl_status raster_backward(View& v, const float* dL_drgb, const float* dL_ddepth,
         bwd_dispatch<false>(v.nb, v.pd, det, v.pg, A, G, units, v.persistent, s);
     count_launches(1);
     if (det) {
-        const int blocks = (int)std::min<size_t>(8 * (size_t)sm_count(), (pairs + 255) / 256);
-        k_part_reduce<<<std::max(blocks, 1), 256, 0, s>>>(v.gpart.as<float>(), v.touched.as<uint32_t>(),
+        const int blocks = (int)std::min<size_t>(8 * (size_t)sm_count(), (pairs + 31) / 32);
+        k_part_reduce<<<std::max(blocks, 1), 256, 0, s>>>(v.gpart.as<float>(), v.gmask.as<uint32_t>(),
+                                                          v.touched.as<uint32_t>(),
                                                           v.dup_off.as<uint32_t>(), nblk, (int64_t)pairs,
                                                           v.count.as<uint64_t>(), (uint64_t)cap, v.g2d.as<float>());
         count_launches(1);

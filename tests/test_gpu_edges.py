@@ -1,0 +1,71 @@
+"""Kernels at the sizes where their splits and tiles end: hit counts around the
+backward's groups of sixteen, lists around the runs, rounds and segments of a
+split tile, loss images around the 32 x 32 tile and its halo, Gaussian counts
+around a warp's, copies of odd length and alignment.  Against the oracle, with
+the tolerances of the parity tests (pixels 1e-5; gradients: median relative
+error 1e-3, 99th percentile 1e-2, floor 1e-4 of the largest)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2404_06926_gb300 import scenes
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+NAMES = ("means", "log_scales", "quats", "logits", "sh")
+
+
+def _dev(params):
+    return {k: torch.from_numpy(np.ascontiguousarray(v, np.float32)).cuda() for k, v in params.items()}
+
+
+def _stack(n, opacity, seed=0):
+    """n wide Gaussians behind one another, each covering the whole 20 x 13 image."""
+    rng = np.random.default_rng(seed)
+    cam = scenes.camera(20, 13, 100.0, 100.0, 10.0, 6.5)
+    z = rng.permutation(np.linspace(1.0, 3.0, n)) if n > 1 else np.array([2.0])
+    q = rng.normal(size=(n, 4))
+    return cam, dict(means=np.stack([rng.normal(0, 0.05, n), rng.normal(0, 0.05, n), z], 1).astype(np.float32),
+                     log_scales=rng.uniform(0.4, 0.8, (n, 3)).astype(np.float32),
+                     quats=(q / np.linalg.norm(q, axis=1, keepdims=True)).astype(np.float32),
+                     logits=np.full(n, np.log(opacity / (1 - opacity)), np.float32),
+                     sh=rng.normal(0, 0.5, (n, 1, 3)).astype(np.float32))
+
+
+def _check_stack(n, opacity, extra, tile=16, **knobs):
+    from paper_2404_06926_gb300 import binding
+    cam, params = _stack(n, opacity)
+    H, W = cam["height"], cam["width"]
+    pre, bins, img = oracle.forward(params, cam, tile)
+    rng = np.random.default_rng(n)
+    dC = (rng.normal(size=(H, W, 3)) * 1e-3).astype(np.float32)
+    dD = (rng.normal(size=(H, W)) * 1e-4).astype(np.float32) if extra else None
+    dO = (rng.normal(size=(H, W)) * 1e-3).astype(np.float32) if extra else None
+    g = oracle.backward(params, cam, pre, bins, dC.astype(np.float64), None if dD is None else dD.astype(np.float64),
+                        None if dO is None else dO.astype(np.float64))
+    ctx = binding.Ctx()
+    ctx.set_exec(**knobs)
+    p = _dev(params)
+    rgb, dep, opa = ctx.forward(p, cam, tile)
+    T, nc = ctx.pixel_state(H, W, "cuda")
+    ok = img["ambiguous"] == 0
+    assert ok.mean() > 0.9
+    assert np.abs(rgb.cpu().numpy() - img["color"])[ok].max() <= 1e-5
+    assert np.abs(opa.cpu().numpy() - img["opacity"])[ok].max() <= 1e-5
+    assert np.abs(T.cpu().numpy() - img["T_final"])[ok].max() <= 1e-5
+    assert np.abs(dep.cpu().numpy() - img["depth"])[ok].max() <= 3e-5
+    assert np.array_equal(nc.cpu().numpy()[ok], img["n_contrib"][ok])
+    tt = lambda a: None if a is None else torch.from_numpy(a).cuda()
+    gg, _ = ctx.backward(p, tt(dC), tt(dD), tt(dO))
+    for name in NAMES:
+        a, ref = gg[name].cpu().numpy().astype(np.float64).ravel(), np.asarray(g[name], np.float64).ravel()
+        rel = np.abs(a - ref) / np.maximum(np.abs(ref), 1e-4 * max(np.abs(ref).max(), 1e-30))
+        assert np.median(rel) < 1e-3 and np.percentile(rel, 99) < 1e-2, (name, np.median(rel), np.percentile(rel, 99))
+
+
+@pytest.mark.parametrize("n", [1, 2, 15, 16, 17, 32, 33, 65])
+@pytest.mark.parametrize("ppl,det,extra,pg", [(1, 0, False, 0), (1, 0, True, 0), (2, 0, True, 0), (4, 0, False, 0),
+                                              (1, 1, True, 0), (1, 1, False, 1)])
+def test_backward_hit_counts(n, ppl, det, extra, pg):
+    _check_stack(n, 0.05, extra, pixels_per_lane=ppl, deterministic=det, per_gaussian=pg)
