@@ -5,23 +5,31 @@
 // SSIM uses an 11x11 Gaussian window (sigma 1.5), zero padding, C1 = 0.01^2,
 // C2 = 0.03^2 -- the D-SSIM of 3DGS the paper cites.
 //
-// One CTA per 32x32 output tile does everything in shared memory: it loads the
-// exposed colour and the target over the tile plus a 10-pixel halo, blurs the
-// five moment maps separably over a 5-pixel halo, forms the SSIM map and its
-// partials w.r.t. (mu_x, E[x^2], E[xy]), blurs those back (the adjoint of a
-// zero-padded symmetric correlation is the same correlation) and adds the
-// channel's part of dL/dC = A^T dL/dE[C] in registers (the thread owning a
-// pixel is the same in every channel, so dL/dC is written once, after the
-// third channel, and never read back).  In every pass a thread slides the 11 taps along a
-// run of 3-8 outputs held in registers, so each shared-memory value is read
-// once per run rather than once per tap and output; the run lengths (and the
-// split of the horizontal adjoint by map) are chosen so that each pass gives
-// the CTA's 256 threads close to a whole number of rounds of equal items
-// (728 = 2.8 x 256, 252, 504 = 2 x 252, 256).  The maps of later passes
-// reuse the space of those consumed (65 KB, three CTAs per SM).  Per-CTA
-// partial sums of |.|, SSIM and dL/dE are reduced afterwards in a fixed
-// order, in double.
+// One CTA per 32x32 output tile and channel, the three channels of a tile in
+// one cluster.  A CTA loads the channel's exposed colour x and target y over
+// the tile plus a 10-pixel halo as (x, y) pairs, blurs the five moment maps
+// separably over a 5-pixel halo, forms the SSIM map and its partials w.r.t. (mu_x, E[x^2], E[xy]) and
+// blurs those back (the adjoint of a zero-padded symmetric correlation is the
+// same correlation).  dL/dC = A^T dL/dE[C] needs all three channels: each CTA
+// leaves its dL/dE[C] in shared memory and, after a cluster barrier, CTA j
+// reads the other two and writes component j.
+//
+// Bound: FP32 issue.  Four of the maps are kept as pairs, (mu_x, mu_y) and
+// (E[x^2], E[y^2]), so a tap is one 8-byte load and one two-lane FMA per pair,
+// and the tap weights are literals.  In every pass a thread slides the 11 taps
+// along a run of 3-8 outputs held in registers; the run lengths give the 256
+// threads 728 = 2.8 x 256, 252, 168 and 256 equal items, and the row strides
+// (43 and 33) keep the passes whose lanes go down rows off shared bank
+// conflicts.  The maps of later passes reuse the space of those consumed:
+// 63.8 KB, three CTAs (24 warps) per SM.  A CTA per channel also cuts the
+// length of the longest chain to a third where a small image leaves SMs idle.
+// One CTA for all three channels -> this: 115.7 -> 104.9 us (1280x1024), 40.6 ->
+// 32.9 (647x481), 24.2 -> 13.8 (256x192: 48 tiles).
+// Per-CTA partial sums of |.|, SSIM and dL/dE are reduced afterwards in a
+// fixed order, in double.
 #include "gl_internal.h"
+
+#include <cooperative_groups.h>
 
 #include <algorithm>
 
@@ -37,16 +45,45 @@ constexpr int kThreads = 256;
 constexpr int kNP = 14;               // partials per CTA: 12 dL/dE, sum|d|, sum SSIM
 constexpr int HR = 3;                 // outputs per thread, horizontal moment pass (RB = 14 x 3)
 constexpr int VR = 7;                 // outputs per thread, vertical moment pass (RB = 6 x 7)
-constexpr int AHR = 8;                // outputs per item, horizontal adjoint pass (LT = 4 x 8)
+constexpr int AHR = 8;                // outputs per thread, horizontal adjoint pass (LT = 4 x 8)
 constexpr int AVR = 4;                // outputs per thread, vertical adjoint pass (LT = 8 x 4)
+constexpr int GS = RB + 1;            // row stride of the partial maps
+constexpr int HS = LT + 1;            // row stride of their horizontal blur
 static_assert(RB % HR == 0 && RB % VR == 0 && LT % AHR == 0 && LT % AVR == 0, "run lengths must tile the maps");
 constexpr float kC1 = 0.01f * 0.01f;
 constexpr float kC2 = 0.03f * 0.03f;
 
-// x and y over the tile and halo (later the three SSIM partial maps), then
-// the five moment maps (later the horizontally blurred partials)
-constexpr size_t kSmemFloats = 2 * RA * RA + 5 * RA * RB;
-static_assert(3 * RB * RB <= 2 * RA * RA && 3 * RB * LT <= 5 * RA * RB, "aliased maps must fit");
+// The window exp(-k^2 / (2 1.5^2)) / sum, |k| <= 5, every operation rounded to
+// single precision.  SSIM divides small differences of blurred squares, where
+// the image is flat by little more than C2: there the rounding of the taps and
+// of the moments shows in the gradient (exact taps move dL/dC by 2.6e-5; x^2 +
+// y^2 blurred as one map costs the loss digits, because 2 xy no longer rounds
+// as it does).  So every sum here takes its terms in one fixed form and order.
+constexpr float kT0 = 0x1.0d957p-10f;
+constexpr float kT1 = 0x1.f1fe06p-8f;
+constexpr float kT2 = 0x1.26eb18p-5f;
+constexpr float kT3 = 0x1.bff102p-4f;
+constexpr float kT4 = 0x1.b43c4p-3f;
+constexpr float kT5 = 0x1.106562p-2f;
+__host__ __device__ constexpr float tap(int k)
+{
+    return k == 0 || k == 10 ? kT0 : k == 1 || k == 9 ? kT1 : k == 2 || k == 8 ? kT2 : k == 3 || k == 7 ? kT3
+         : k == 4 || k == 6 ? kT4 : kT5;
+}
+
+// two FMAs on a register pair, both lanes rounded to nearest
+__device__ __forceinline__ float2 fma2(float a, float2 b, float2 c)
+{
+    return __ffma2_rn(make_float2(a, a), b, c);
+}
+
+// (x, y) over the tile and halo (later the three SSIM partial maps: a pair
+// map and a single one), then the two pair maps and the single one of the
+// moments (later the horizontally blurred partials)
+constexpr size_t kXYBytes = 12 * RB * GS;   // >= 8 RA RA
+constexpr size_t kSmemBytes = kXYBytes + 20 * RA * RB;
+static_assert(8 * RA * RA <= kXYBytes && 12 * RB * HS <= 16 * RA * RB && kXYBytes % 8 == 0, "aliased maps must fit");
+static_assert(4 * LT * LT <= 8 * RA * RA, "the channel's gradient map reuses the partial maps");
 
 // One view passed by value (the stateless and allocation-free entry points).
 struct LossOne {
@@ -57,20 +94,23 @@ struct LossOne {
     int W, H;
 };
 
-// Grid: one CTA per 32x32 loss tile over all views.  With `views` null the
-// single view `one` is used; otherwise view, images, exposure and weight
-// come from the descriptors and images are the concatenated ones.
-__global__ void __launch_bounds__(kThreads, 3)
+// Grid: a cluster of three CTAs (the channels) per 32x32 loss tile over all
+// views.  With `views` null the single view `one` is used; otherwise view,
+// images, exposure and weight come from the descriptors and images are the
+// concatenated ones.
+__global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(kThreads, 3)
 k_loss(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __restrict__ rgb_all,
        float* __restrict__ dL_all, float lambda, float* __restrict__ part)
 {
+    namespace cg = cooperative_groups;
     const float* rgb = one.rgb;
     const float* target = one.target;
     const float* E = one.E;
     float* dL_drgb = one.dL;
     int W = one.W, H = one.H;
     float weight = 1.0f;
-    int lt = blockIdx.x;
+    const int ch = blockIdx.x % 3;   // the rank in the cluster
+    int lt = blockIdx.x / 3;
     if (views) {
         const int v = view_of_ltile(views, V, lt);
         const ViewDesc& d = views[v];
@@ -83,210 +123,240 @@ k_loss(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __re
         H = d.cam.H;
         weight = d.weight;
     }
-    extern __shared__ float sm[];
-    float* xs = sm;
-    float* ys = xs + RA * RA;
-    float* hm = ys + RA * RA;          // 5 maps, RA rows x RB cols
-    float* gmap = xs;                  // 3 maps, RB x RB (reuses x, y after the horizontal pass)
-    float* hg = hm;                    // 3 maps, RB rows x LT cols (reuses hm)
-    __shared__ float wt[11];
-    __shared__ float Es[12];
-    __shared__ float red[kNP][kThreads / 32];
-    const int tid = threadIdx.x;
-    if (tid < 11) {
-        float s = 0.0f;
-        for (int k = 0; k < 11; k++) s += expf(-(float)((k - HW) * (k - HW)) / 4.5f);
-        wt[tid] = expf(-(float)((tid - HW) * (tid - HW)) / 4.5f) / s;
-    }
-    if (tid < 12) Es[tid] = E ? E[tid] : ((tid % 5 == 0) ? 1.0f : 0.0f);
-    __syncthreads();
+    extern __shared__ __align__(16) unsigned char smraw[];
+    float2* xy = reinterpret_cast<float2*>(smraw);                 // RA x RA
+    float2* gab = xy;                                              // RB x GS (reuses xy after the horizontal pass)
+    float* gcm = reinterpret_cast<float*>(gab + RB * GS);          // RB x GS
+    float* gout = reinterpret_cast<float*>(smraw);                 // LT x LT (reuses the partial maps)
+    float2* hm = reinterpret_cast<float2*>(smraw + kXYBytes);      // 2 maps, RA rows x RB cols
+    float* hp = reinterpret_cast<float*>(hm + 2 * RA * RB);        // E[xy]
+    float2* hab = hm;                                              // RB rows x HS (reuses hm)
+    float* hc = reinterpret_cast<float*>(hab + RB * HS);           // RB rows x HS
+    __shared__ float red[6][kThreads / 32];
+    __shared__ float chsum[3][2];    // in CTA 0 of the cluster: the channels' sums of |.| and SSIM
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const float e0 = E ? E[4 * ch] : (ch == 0 ? 1.0f : 0.0f), e1 = E ? E[4 * ch + 1] : (ch == 1 ? 1.0f : 0.0f);
+    const float e2 = E ? E[4 * ch + 2] : (ch == 2 ? 1.0f : 0.0f), e3 = E ? E[4 * ch + 3] : 0.0f;
     const int LTX = (W + LT - 1) / LT;
     const int ox = (lt % LTX) * LT, oy = (lt / LTX) * LT;
     const float invN = 1.0f / (3.0f * (float)W * (float)H);
     const float gS = -lambda * invN * weight;
     const float gL1 = (1.0f - lambda) * invN * weight;
-    float l1acc = 0.0f, sacc = 0.0f;
-    const int lane = tid & 31, wid = tid >> 5;
 
-    // the adjoint pass gives every thread one run of AVR rows of one column,
-    // the same in every channel: its pixels' dL/dC stays in registers
-    static_assert(LT * (LT / AVR) == kThreads, "one adjoint run per thread");
-    float dC[AVR][3];
-#pragma unroll
-    for (int o = 0; o < AVR; o++) dC[o][0] = dC[o][1] = dC[o][2] = 0.0f;
-    for (int ch = 0; ch < 3; ch++) {
-        // exposure gradient partials of this channel: sum g C_j (j < 3), sum g
-        float pe[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        const float e0 = Es[4 * ch], e1 = Es[4 * ch + 1], e2 = Es[4 * ch + 2], e3 = Es[4 * ch + 3];
-        for (int e = tid; e < RA * RA; e += kThreads) {
-            const int gx = ox - 2 * HW + e % RA, gy = oy - 2 * HW + e / RA;
-            float x = 0.0f, y = 0.0f;
-            if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
-                const size_t p = (size_t)gy * W + gx;
-                x = e0 * rgb[3 * p] + e1 * rgb[3 * p + 1] + e2 * rgb[3 * p + 2] + e3;
-                y = target[3 * p + ch];
-            }
-            xs[e] = x;
-            ys[e] = y;
+    // a warp per row, two columns per lane; a tile whose halo lies inside the
+    // image takes the loads without bounds
+    const bool inner = ox >= 2 * HW && oy >= 2 * HW && ox + LT + 2 * HW <= W && oy + LT + 2 * HW <= H;
+    if (inner) {
+        const size_t p0 = 3 * ((size_t)(oy - 2 * HW + wid) * W + (ox - 2 * HW + lane));
+        const float* cp = rgb + p0;
+        const float* tp = target + p0 + ch;
+        const size_t step = 3 * (size_t)(kThreads / 32) * W;
+#pragma unroll 4
+        for (int r = wid; r < RA; r += kThreads / 32, cp += step, tp += step) {
+            xy[r * RA + lane] = make_float2(e0 * cp[0] + e1 * cp[1] + e2 * cp[2] + e3, tp[0]);
+            if (lane < RA - 32)
+                xy[r * RA + 32 + lane] = make_float2(e0 * cp[96] + e1 * cp[97] + e2 * cp[98] + e3, tp[96]);
         }
-        __syncthreads();
-        // horizontal pass of the five moments: a thread slides the 11 taps
-        // along a run of HR outputs of one row, loading each input once
-        for (int e = tid; e < RA * (RB / HR); e += kThreads) {
-            const int r = e / (RB / HR), c0 = (e % (RB / HR)) * HR;
-            float xv[HR + 10], yv[HR + 10];
+    } else {
+        for (int r = wid; r < RA; r += kThreads / 32) {
+            const int gy = oy - 2 * HW + r;
+            const bool rowin = gy >= 0 && gy < H;
 #pragma unroll
-            for (int k = 0; k < HR + 10; k++) { xv[k] = xs[r * RA + c0 + k]; yv[k] = ys[r * RA + c0 + k]; }
-#pragma unroll
-            for (int o = 0; o < HR; o++) {
-                float s0 = 0, s1 = 0, s2 = 0, s3 = 0, s4 = 0;
-#pragma unroll
-                for (int k = 0; k < 11; k++) {
-                    const float x = xv[o + k], y = yv[o + k], wk = wt[k];
-                    s0 += wk * x; s1 += wk * y; s2 += wk * x * x; s3 += wk * y * y; s4 += wk * x * y;
+            for (int k = 0; k < 2; k++) {
+                const int c = lane + 32 * k, gx = ox - 2 * HW + c;
+                float2 v = make_float2(0.0f, 0.0f);
+                if (rowin && c < RA && gx >= 0 && gx < W) {
+                    const size_t p = 3 * ((size_t)gy * W + gx);
+                    v.x = e0 * rgb[p] + e1 * rgb[p + 1] + e2 * rgb[p + 2] + e3;
+                    v.y = target[p + ch];
                 }
-                const int i = r * RB + c0 + o;
-                hm[i] = s0; hm[RA * RB + i] = s1; hm[2 * RA * RB + i] = s2;
-                hm[3 * RA * RB + i] = s3; hm[4 * RA * RB + i] = s4;
+                if (c < RA) xy[r * RA + c] = v;
             }
-        }
-        __syncthreads();
-        // vertical pass, SSIM and its partials: a thread takes a run of VR
-        // rows of one column, one moment map at a time
-        for (int e = tid; e < RB * (RB / VR); e += kThreads) {
-            const int c = e % RB, r0 = (e / RB) * VR;
-            float mom[5][VR];
-#pragma unroll
-            for (int m = 0; m < 5; m++) {
-                float col[VR + 10];
-#pragma unroll
-                for (int k = 0; k < VR + 10; k++) col[k] = hm[m * RA * RB + (r0 + k) * RB + c];
-#pragma unroll
-                for (int o = 0; o < VR; o++) {
-                    float a = 0.0f;
-#pragma unroll
-                    for (int k = 0; k < 11; k++) a += wt[k] * col[o + k];
-                    mom[m][o] = a;
-                }
-            }
-#pragma unroll
-            for (int o = 0; o < VR; o++) {
-                const int r = r0 + o;
-                const int gx = ox - HW + c, gy = oy - HW + r;
-                float ga = 0.0f, gb = 0.0f, gc = 0.0f;
-                if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
-                    const float mx = mom[0][o], my = mom[1][o], exx = mom[2][o], eyy = mom[3][o], exy = mom[4][o];
-                    const float sxx = exx - mx * mx, syy = eyy - my * my, sxy = exy - mx * my;
-                    const float N1 = 2.f * mx * my + kC1, N2 = 2.f * sxy + kC2;
-                    const float D1 = mx * mx + my * my + kC1, D2 = sxx + syy + kC2;
-                    // one approximate reciprocal (a few ulp) serves S and both
-                    // partials: 1/D1 = D2 iD, 1/D2 = D1 iD
-                    const float iD = __fdividef(1.0f, D1 * D2);
-                    const float S = N1 * N2 * iD;
-                    if (r >= HW && r < HW + LT && c >= HW && c < HW + LT) sacc += S;
-                    const float dN1 = N2 * iD, dN2 = N1 * iD, dD1 = -S * (D2 * iD), dD2 = -S * (D1 * iD);
-                    const float dmx = dN1 * 2.f * my - dN2 * 2.f * my + dD1 * 2.f * mx - dD2 * 2.f * mx;
-                    ga = gS * dmx;
-                    gb = gS * dD2;
-                    gc = gS * 2.f * dN2;
-                }
-                const int i = r * RB + c;
-                gmap[i] = ga; gmap[RB * RB + i] = gb; gmap[2 * RB * RB + i] = gc;
-            }
-        }
-        __syncthreads();
-        // adjoint, horizontal: one item per (map, row, run of AHR outputs)
-        for (int e = tid; e < 3 * RB * (LT / AHR); e += kThreads) {
-            const int m = e / (RB * (LT / AHR)), rr = e % (RB * (LT / AHR));
-            const int r = rr / (LT / AHR), c0 = (rr % (LT / AHR)) * AHR;
-            float row[AHR + 10];
-#pragma unroll
-            for (int k = 0; k < AHR + 10; k++) row[k] = gmap[m * RB * RB + r * RB + c0 + k];
-#pragma unroll
-            for (int o = 0; o < AHR; o++) {
-                float a = 0.0f;
-#pragma unroll
-                for (int k = 0; k < 11; k++) a += wt[k] * row[o + k];
-                hg[m * RB * LT + r * LT + c0 + o] = a;
-            }
-        }
-        __syncthreads();
-        // adjoint, vertical, and dL/dE[C] of the tile's pixels: runs of AVR rows of a column
-        for (int e = tid; e < LT * (LT / AVR); e += kThreads) {
-            const int c = e % LT, r0 = (e / LT) * AVR;
-            float acc[3][AVR];
-#pragma unroll
-            for (int m = 0; m < 3; m++) {
-                float col[AVR + 10];
-#pragma unroll
-                for (int k = 0; k < AVR + 10; k++) col[k] = hg[m * RB * LT + (r0 + k) * LT + c];
-#pragma unroll
-                for (int o = 0; o < AVR; o++) {
-                    float a = 0.0f;
-#pragma unroll
-                    for (int k = 0; k < 11; k++) a += wt[k] * col[o + k];
-                    acc[m][o] = a;
-                }
-            }
-            // dL/dE[C]_ch of the pixels (x, y read again: their shared copy
-            // now holds the partial maps); dL/dC += A_ch^T dL/dE[C]_ch, by
-            // the thread that owns the pixel in every channel
-#pragma unroll
-            for (int o = 0; o < AVR; o++) {
-                const int r = r0 + o;
-                const int gx = ox + c, gy = oy + r;
-                if (gx < W && gy < H) {
-                    const size_t p = (size_t)gy * W + gx;
-                    const float c0 = rgb[3 * p], c1 = rgb[3 * p + 1], c2 = rgb[3 * p + 2];
-                    const float x = e0 * c0 + e1 * c1 + e2 * c2 + e3, y = target[3 * p + ch];
-                    const float d = x - y;
-                    l1acc += fabsf(d);
-                    const float g = acc[0][o] + 2.f * x * acc[1][o] + y * acc[2][o] +
-                                    gL1 * (d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f));
-                    pe[0] += g * c0; pe[1] += g * c1; pe[2] += g * c2; pe[3] += g;
-                    dC[o][0] = ch == 0 ? e0 * g : dC[o][0] + e0 * g;
-                    dC[o][1] = ch == 0 ? e1 * g : dC[o][1] + e1 * g;
-                    dC[o][2] = ch == 0 ? e2 * g : dC[o][2] + e2 * g;
-                }
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 4; i++) {
-            float v = pe[i];
-            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
-            if (lane == 0) red[4 * ch + i][wid] = v;
-        }
-        __syncthreads();
-    }
-
-    {
-        const int c = tid % LT, r0 = (tid / LT) * AVR;
-#pragma unroll
-        for (int o = 0; o < AVR; o++) {
-            const int gx = ox + c, gy = oy + r0 + o;
-            if (gx < W && gy < H) {
-                const size_t p = (size_t)gy * W + gx;
-                dL_drgb[3 * p] = dC[o][0];
-                dL_drgb[3 * p + 1] = dC[o][1];
-                dL_drgb[3 * p + 2] = dC[o][2];
-            }
-        }
-    }
-    {
-        const float vals[2] = {l1acc, sacc};
-#pragma unroll
-        for (int i = 0; i < 2; i++) {
-            float v = vals[i];
-            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
-            if (lane == 0) red[12 + i][wid] = v;
         }
     }
     __syncthreads();
-    if (tid < kNP) {
+    // horizontal pass of the moments: runs of HR outputs of one row
+    for (int e = tid; e < RA * (RB / HR); e += kThreads) {
+        const int r = e / (RB / HR), c0 = (e % (RB / HR)) * HR;
+        float2 m[HR], q[HR];
+        float p[HR];
+#pragma unroll
+        for (int o = 0; o < HR; o++) {
+            m[o] = q[o] = make_float2(0.0f, 0.0f);
+            p[o] = 0.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < HR + 10; k++) {
+            const float2 v = xy[r * RA + c0 + k];
+#pragma unroll
+            for (int o = 0; o < HR; o++)
+                if (k >= o && k - o < 11) {
+                    const float w = tap(k - o);
+                    const float2 t = __fmul2_rn(make_float2(w, w), v);
+                    m[o] = fma2(w, v, m[o]);
+                    q[o] = __ffma2_rn(t, v, q[o]);
+                    p[o] = fmaf(t.x, v.y, p[o]);
+                }
+        }
+#pragma unroll
+        for (int o = 0; o < HR; o++) {
+            const int i = r * RB + c0 + o;
+            hm[i] = m[o];
+            hm[RA * RB + i] = q[o];
+            hp[i] = p[o];
+        }
+    }
+    __syncthreads();
+    // vertical pass, SSIM and its partials: runs of VR rows of one column
+    float l1acc = 0.0f, sacc = 0.0f;
+    if (tid < RB * (RB / VR)) {
+        const int c = tid % RB, r0 = (tid / RB) * VR;
+        float2 m[VR], q[VR];
+        float p[VR];
+#pragma unroll
+        for (int o = 0; o < VR; o++) {
+            m[o] = q[o] = make_float2(0.0f, 0.0f);
+            p[o] = 0.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < VR + 10; k++) {
+            const int i = (r0 + k) * RB + c;
+            const float2 v = hm[i], s = hm[RA * RB + i];
+            const float z = hp[i];
+#pragma unroll
+            for (int o = 0; o < VR; o++)
+                if (k >= o && k - o < 11) {
+                    m[o] = fma2(tap(k - o), v, m[o]);
+                    q[o] = fma2(tap(k - o), s, q[o]);
+                    p[o] = fmaf(tap(k - o), z, p[o]);
+                }
+        }
+        const int gx = ox - HW + c;
+        const bool colin = gx >= 0 && gx < W, core = c >= HW && c < HW + LT;
+#pragma unroll
+        for (int o = 0; o < VR; o++) {
+            const int r = r0 + o;
+            const int gy = oy - HW + r;
+            float ga = 0.0f, gb = 0.0f, gc = 0.0f;
+            if (colin && gy >= 0 && gy < H) {
+                const float mx = m[o].x, my = m[o].y, exx = q[o].x, eyy = q[o].y, exy = p[o];
+                const float sxx = exx - mx * mx, syy = eyy - my * my, sxy = exy - mx * my;
+                const float N1 = 2.f * mx * my + kC1, N2 = 2.f * sxy + kC2;
+                const float D1 = mx * mx + my * my + kC1, D2 = sxx + syy + kC2;
+                // one approximate reciprocal (a few ulp) serves S and both
+                // partials: 1/D1 = D2 iD, 1/D2 = D1 iD
+                const float iD = __fdividef(1.0f, D1 * D2);
+                const float S = N1 * N2 * iD;
+                if (core && r >= HW && r < HW + LT) sacc += S;
+                const float dN1 = N2 * iD, dN2 = N1 * iD, dD1 = -S * (D2 * iD), dD2 = -S * (D1 * iD);
+                const float dmx = dN1 * 2.f * my - dN2 * 2.f * my + dD1 * 2.f * mx - dD2 * 2.f * mx;
+                ga = gS * dmx;
+                gb = gS * dD2;
+                gc = gS * 2.f * dN2;
+            }
+            gab[r * GS + c] = make_float2(ga, gb);
+            gcm[r * GS + c] = gc;
+        }
+    }
+    __syncthreads();
+    // adjoint, horizontal: a thread per (row, run of AHR outputs), lanes down the rows
+    if (tid < RB * (LT / AHR)) {
+        const int r = tid % RB, c0 = (tid / RB) * AHR;
+        float2 a[AHR];
+        float b[AHR];
+#pragma unroll
+        for (int o = 0; o < AHR; o++) { a[o] = make_float2(0.0f, 0.0f); b[o] = 0.0f; }
+#pragma unroll
+        for (int k = 0; k < AHR + 10; k++) {
+            const float2 v = gab[r * GS + c0 + k];
+            const float s = gcm[r * GS + c0 + k];
+#pragma unroll
+            for (int o = 0; o < AHR; o++)
+                if (k >= o && k - o < 11) {
+                    a[o] = fma2(tap(k - o), v, a[o]);
+                    b[o] = fmaf(tap(k - o), s, b[o]);
+                }
+        }
+#pragma unroll
+        for (int o = 0; o < AHR; o++) {
+            hab[r * HS + c0 + o] = a[o];
+            hc[r * HS + c0 + o] = b[o];
+        }
+    }
+    __syncthreads();
+    // adjoint, vertical, and dL/dE[C] of the tile's pixels: runs of AVR rows
+    // of a column (x, y read again: their shared copy is overwritten)
+    static_assert(LT * (LT / AVR) == kThreads, "one adjoint run per thread");
+    const int c = tid % LT, r0 = (tid / LT) * AVR;
+    float pe[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // exposure gradient: sum g C_j (j < 3), sum g
+    float g[AVR];
+    {
+        float2 a[AVR];
+        float b[AVR];
+#pragma unroll
+        for (int o = 0; o < AVR; o++) { a[o] = make_float2(0.0f, 0.0f); b[o] = 0.0f; }
+#pragma unroll
+        for (int k = 0; k < AVR + 10; k++) {
+            const float2 v = hab[(r0 + k) * HS + c];
+            const float s = hc[(r0 + k) * HS + c];
+#pragma unroll
+            for (int o = 0; o < AVR; o++)
+                if (k >= o && k - o < 11) {
+                    a[o] = fma2(tap(k - o), v, a[o]);
+                    b[o] = fmaf(tap(k - o), s, b[o]);
+                }
+        }
+#pragma unroll
+        for (int o = 0; o < AVR; o++) {
+            const int gx = ox + c, gy = oy + r0 + o;
+            g[o] = 0.0f;
+            if (gx < W && gy < H) {
+                const size_t p = 3 * ((size_t)gy * W + gx);
+                const float c0 = rgb[p], c1 = rgb[p + 1], c2 = rgb[p + 2];
+                const float x = e0 * c0 + e1 * c1 + e2 * c2 + e3, y = target[p + ch];
+                const float d = x - y;
+                l1acc += fabsf(d);
+                g[o] = a[o].x + 2.f * x * a[o].y + y * b[o] + gL1 * (d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f));
+                pe[0] += g[o] * c0; pe[1] += g[o] * c1; pe[2] += g[o] * c2; pe[3] += g[o];
+            }
+            gout[(r0 + o) * LT + c] = g[o];
+        }
+    }
+    {
+        const float vals[6] = {pe[0], pe[1], pe[2], pe[3], l1acc, sacc};
+#pragma unroll
+        for (int i = 0; i < 6; i++) {
+            float v = vals[i];
+            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
+            if (lane == 0) red[i][wid] = v;
+        }
+    }
+    __syncthreads();
+    cg::cluster_group cluster = cg::this_cluster();
+    float* prow = part + (size_t)(blockIdx.x / 3) * kNP;
+    if (tid < 6) {
         float v = 0.0f;
         for (int ww = 0; ww < kThreads / 32; ww++) v += red[tid][ww];
-        part[(size_t)blockIdx.x * kNP + tid] = v;
+        if (tid < 4) prow[4 * ch + tid] = v;
+        else cluster.map_shared_rank(&chsum[0][0], 0)[2 * ch + tid - 4] = v;
     }
+    cluster.sync();
+    // component ch of dL/dC = sum over channels k of A[k][ch] dL/dE[C]_k
+    {
+        const float f0 = E ? E[ch] : (ch == 0 ? 1.0f : 0.0f), f1 = E ? E[4 + ch] : (ch == 1 ? 1.0f : 0.0f);
+        const float f2 = E ? E[8 + ch] : (ch == 2 ? 1.0f : 0.0f);
+        const float* g0 = cluster.map_shared_rank(gout, 0);
+        const float* g1 = cluster.map_shared_rank(gout, 1);
+        const float* g2 = cluster.map_shared_rank(gout, 2);
+#pragma unroll
+        for (int o = 0; o < AVR; o++) {
+            const int gx = ox + c, gy = oy + r0 + o, i = (r0 + o) * LT + c;
+            const float v = fmaf(f2, g2[i], fmaf(f1, g1[i], f0 * g0[i]));
+            if (gx < W && gy < H) dL_drgb[3 * ((size_t)gy * W + gx) + ch] = v;
+        }
+    }
+    if (ch == 0 && tid < 2) prow[12 + tid] = chsum[0][tid] + chsum[1][tid] + chsum[2][tid];
+    cluster.sync();   // the shared memory read by the other CTAs stays until they are done
 }
 
 // Sums the per-tile partials in a fixed order (double).  Single view (views
@@ -378,7 +448,7 @@ int loss_partials_needed(int W, int H)
 namespace {
 gl_status loss_attr()
 {
-    return ensure_smem_limit(reinterpret_cast<const void*>(&k_loss), (int)(kSmemFloats * sizeof(float)));
+    return ensure_smem_limit(reinterpret_cast<const void*>(&k_loss), (int)kSmemBytes);
 }
 }  // namespace
 
@@ -389,7 +459,7 @@ gl_status photometric_loss(const float* rgb, const float* target, const float* E
     GL_TRY(loss_attr());
     const int nblk = ((W + LT - 1) / LT) * ((H + LT - 1) / LT);
     LossOne one{rgb, target, E, dL_drgb, W, H};
-    k_loss<<<nblk, kThreads, kSmemFloats * sizeof(float), s>>>(one, nullptr, 0, nullptr, nullptr, lambda, part);
+    k_loss<<<3 * nblk, kThreads, kSmemBytes, s>>>(one, nullptr, 0, nullptr, nullptr, lambda, part);
     k_loss_final<<<1, 32 * kNP, 0, s>>>(part, nblk, W, H, lambda, loss_out, dE_out, nullptr, nullptr, 0.f, 0.f,
                                         0.f, 0.f, nullptr);
     count_launches(2);
@@ -403,7 +473,7 @@ gl_status photometric_loss_views(const View& v, const float* rgb, float lambda, 
 {
     GL_TRY(loss_attr());
     LossOne one{};
-    k_loss<<<v.nltiles, kThreads, kSmemFloats * sizeof(float), s>>>(one, v.d_desc(), v.V, rgb, dL_drgb, lambda,
+    k_loss<<<3 * v.nltiles, kThreads, kSmemBytes, s>>>(one, v.d_desc(), v.V, rgb, dL_drgb, lambda,
                                                                      part);
     k_loss_final<<<v.V, 32 * kNP, 0, s>>>(part, 0, 0, 0, lambda, nullptr, nullptr, v.d_desc(), loss_v, b1, b2, eps,
                                           lr, abort);

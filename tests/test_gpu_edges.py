@@ -69,3 +69,20 @@ def _check_stack(n, opacity, extra, tile=16, **knobs):
                                               (1, 1, True, 0), (1, 1, False, 1)])
 def test_backward_hit_counts(n, ppl, det, extra, pg):
     _check_stack(n, 0.05, extra, pixels_per_lane=ppl, deterministic=det, per_gaussian=pg)
+
+
+@pytest.mark.parametrize("W,H", [(1, 1), (5, 40), (31, 33), (32, 32), (33, 31), (52, 53), (84, 107)])
+def test_loss_sizes(W, H):
+    from paper_2404_06926_gb300 import binding
+    rng = np.random.default_rng(W * 1000 + H)
+    C = rng.uniform(0, 1, (H, W, 3)).astype(np.float32)
+    tgt = np.clip(C + rng.normal(0, 0.1, (H, W, 3)), 0, 1).astype(np.float32)
+    E = (np.eye(3, 4) + rng.normal(0, 0.05, (3, 4))).astype(np.float32)
+    L = oracle.loss(C.astype(np.float64), tgt, E)
+    ctx = binding.Ctx()
+    loss, dC, dE = ctx.loss(*(torch.from_numpy(x).cuda() for x in (C, tgt, E.reshape(12))))
+    assert abs(loss.item() - L["loss"]) <= 1e-5 * abs(L["loss"])
+    for got, ref in ((dC, L["dL_dC"]), (dE, L["dL_dE"])):
+        a, ref = got.cpu().numpy().astype(np.float64).ravel(), np.asarray(ref, np.float64).ravel()
+        rel = np.abs(a - ref) / np.maximum(np.abs(ref), 1e-4 * np.abs(ref).max())
+        assert np.median(rel) < 1e-3 and np.percentile(rel, 99) < 1e-2, (np.median(rel), np.percentile(rel, 99))
