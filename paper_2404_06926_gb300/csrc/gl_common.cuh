@@ -440,6 +440,24 @@ __device__ __forceinline__ void df_div(float ah, float al, float bh, float bl, f
     two_sum(q1, __fdiv_rn(r, bh), qh, ql);
 }
 
+// (h + l) += x, the sum of floats that the reductions of block partials keep:
+// as wide as their double sum was (about 2^-48 relative per addition) without
+// the few FP64 lanes of the chip, which made those sums the reductions' time
+__device__ __forceinline__ void df_acc(float& h, float& l, float x)
+{
+    float s, e;
+    two_sum(h, x, s, e);
+    h = s;
+    l = __fadd_rn(l, e);
+}
+
+// its value; an infinite or NaN sum keeps the plain sum's value (the error
+// terms of infinities are NaN)
+__device__ __forceinline__ double df_value(float h, float l)
+{
+    return fabsf(l) <= 3.0e38f ? (double)h + (double)l : (double)h;
+}
+
 // mu' as (u_hi + u_lo, v_hi + v_lo); z > 0 is known (the decision passed)
 __device__ __forceinline__ void mean2d_df(const float mu[3], const Cam& cam, float& uh, float& ul, float& vh,
                                           float& vl)
