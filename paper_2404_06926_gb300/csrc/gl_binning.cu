@@ -644,7 +644,8 @@ k_duplicate(const uint32_t* __restrict__ sorted_g, const uint32_t* __restrict__ 
 // for a tile whose list holds at least 2 seg records, one per segment of
 // seg records (seg a power of two, so such tiles sit in the log2 buckets
 // ahead of all others and their items come first).  item = (tile,
-// segment); count[6] = items, count[7] = items of split tiles.  One CTA of
+// segment); count[6] = items, count[7] = items of split tiles, count[11] =
+// split tiles, whose first items are listed in heads.  One CTA of
 // 1024 threads computes the tile launch order first, then the items.  With
 // SMEM the list lengths and the order stay in shared memory (8 bytes per
 // tile), so that the ranges are read once and nothing is read back.
@@ -652,17 +653,17 @@ constexpr int kOrderSmemTiles = 24576;   // 192 KB of shared memory
 template <bool SMEM>
 __global__ void __launch_bounds__(1024) k_order_items(const uint32_t* __restrict__ ranges, int ntiles, int seg,
                                                       uint32_t* __restrict__ order, uint2* __restrict__ items,
-                                                      uint64_t* __restrict__ count)
+                                                      uint32_t* __restrict__ heads, uint64_t* __restrict__ count)
 {
     extern __shared__ uint32_t dyn[];   // SMEM: list length [ntiles] | order [ntiles]
     __shared__ uint32_t cnt[33], off[33];
     __shared__ uint32_t sm[1024 / 32 + 1];
-    __shared__ uint32_t seg_end;
+    __shared__ uint32_t seg_end, split_end;
     uint32_t* slen = dyn;
     uint32_t* sord = dyn + ntiles;
     const uint2* r2 = reinterpret_cast<const uint2*>(ranges);
     if (threadIdx.x < 33) cnt[threadIdx.x] = 0;
-    if (threadIdx.x == 0) seg_end = 0;
+    if (threadIdx.x == 0) seg_end = split_end = 0;
     __syncthreads();
     // bucket b = clz(length): 0 for the longest lists, 32 for empty ones
     constexpr int U = 4;   // lengths loaded before any is counted
@@ -724,13 +725,19 @@ __global__ void __launch_bounds__(1024) k_order_items(const uint32_t* __restrict
         uint32_t tot;
         const uint32_t off0 = carry + block_exclusive_scan<uint32_t, 1024>(nseg, sm, &tot);
         for (uint32_t j = 0; j < nseg; j++) items[off0 + j] = make_uint2(t, j);
-        if (nseg > 1) atomicMax(&seg_end, off0 + nseg);
+        if (nseg > 1) {
+            // split tiles lead the order: k counts them
+            heads[k] = off0;
+            atomicMax(&seg_end, off0 + nseg);
+            atomicMax(&split_end, (uint32_t)k + 1u);
+        }
         carry += tot;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         count[6] = carry;
         count[7] = seg_end;
+        count[11] = split_end;
     }
 }
 
@@ -822,16 +829,17 @@ gl_status build_items(View& v, cudaStream_t s)
 {
     GL_TRY(v.items.reserve(sizeof(uint2) * (size_t)std::max<int64_t>(work_items_bound(v), 1)));
     GL_TRY(v.tile_order.reserve(4 * (size_t)std::max(v.ntiles, 1)));
+    GL_TRY(v.heads.reserve(4 * (size_t)std::max(v.ntiles, 1)));
     if (v.ntiles <= kOrderSmemTiles) {
         const int bytes = 8 * std::max(v.ntiles, 1);
         GL_TRY(ensure_smem_limit(reinterpret_cast<const void*>(&k_order_items<true>), bytes));
         k_order_items<true><<<1, 1024, bytes, s>>>(v.ranges.as<uint32_t>(), v.ntiles, v.seg,
                                                    v.tile_order.as<uint32_t>(), v.items.as<uint2>(),
-                                                   v.count.as<uint64_t>());
+                                                   v.heads.as<uint32_t>(), v.count.as<uint64_t>());
     } else {
         k_order_items<false><<<1, 1024, 0, s>>>(v.ranges.as<uint32_t>(), v.ntiles, v.seg,
                                                 v.tile_order.as<uint32_t>(), v.items.as<uint2>(),
-                                                v.count.as<uint64_t>());
+                                                v.heads.as<uint32_t>(), v.count.as<uint64_t>());
     }
     count_launches(1);
     GL_CUDA_TRY(cudaGetLastError());

@@ -233,7 +233,7 @@ gl_status View::upload_descs(cudaStream_t s)
 void View::release()
 {
     DevBuf* all[] = {&rec0, &rec1, &rec2, &rec3, &radius, &rect, &touched, &dkey, &gidx, &dkey2, &gidx2,
-                     &dup_off, &bsum, &count, &itile, &ival, &itile2, &ival2, &iowner, &srec0, &srec1, &srec2, &srec3, &sgid, &g2d, &gpart, &gmask, &work, &items, &segstate, &kmask,
+                     &dup_off, &bsum, &count, &itile, &ival, &itile2, &ival2, &iowner, &srec0, &srec1, &srec2, &srec3, &sgid, &g2d, &gpart, &gmask, &work, &items, &heads, &segstate, &kmask,
                      &hist, &ranges, &tile_order, &Tfin, &ncon, &rgb, &depth, &opac};
     for (DevBuf* b : all) b->release();
     desc.release();
@@ -1173,7 +1173,7 @@ std::vector<int64_t> graph_key(const gl_map* m, const StepPlan& sp)
                             &v.gidx, &v.dkey2, &v.gidx2, &v.dup_off, &v.g2d, &v.bsum, &v.count, &v.itile,
                             &v.ival, &v.itile2, &v.ival2, &v.iowner, &v.srec0, &v.srec1, &v.srec2, &v.srec3,
                             &v.sgid, &v.hist, &v.ranges, &v.tile_order, &v.Tfin, &v.ncon, &v.rgb, &v.work, &v.gpart, &v.gmask,
-                            &v.items, &v.segstate, &v.kmask,
+                            &v.items, &v.heads, &v.segstate, &v.kmask,
                             &v.desc, &m->dLdC, &m->ctx.loss_part, &m->loss_dev};
     for (const DevBuf* b : bufs) {
         k.push_back((int64_t)(uintptr_t)b->p);

@@ -533,6 +533,19 @@ __device__ __forceinline__ bool pair_eval_nb(const float4 r0, const float4 r1, f
     return e >= kLog2AlphaMin && !(e > r1.y);
 }
 
+// The forward's pair_eval_nb: alpha against a per-pixel log2 threshold (kNoAlpha:
+// no Gaussian reaches it).
+constexpr float kNoAlpha = 3.0e38f;
+__device__ __forceinline__ bool pair_alpha(const float4 r0, const float4 r1, float px, float py, float thr,
+                                           float& alpha)
+{
+    const float dx = __fsub_rn(r0.x, px), dy = __fsub_rn(r0.y, py);
+    const float e = __fmaf_rn(__fmul_rn(r0.z, dx), dx,
+                              __fmaf_rn(__fmul_rn(r0.w, dy), dy, __fmaf_rn(__fmul_rn(r1.x, dx), dy, r1.y)));
+    alpha = fminf(kAlphaMax, ex2_approx(e));
+    return e >= thr && !(e > r1.y);
+}
+
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 
 }  // namespace gl

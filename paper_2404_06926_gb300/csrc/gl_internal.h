@@ -163,7 +163,7 @@ struct View {
                               // bit 1: parameter staging; sticky until
                               // sort_wait_status reads it), Gaussians left after
                               // the depth sort drops the culled ones [9],
-                              // duplication parts [10]
+                              // duplication parts [10], split tiles [11]
     // per instance
     DevBuf itile, ival, itile2, ival2;  // u32 global tile id, u32 instance id (sort; input ids implied)
     DevBuf iowner;            // u32 owning (view, Gaussian) per instance id
@@ -199,6 +199,7 @@ struct View {
     // per-Gaussian backward: lanes own Gaussians, pixel states travel the warp
     bool pg = false;
     DevBuf items;             // uint2 per work item: (tile, segment), heaviest first
+    DevBuf heads;             // u32 first item of each split tile
     DevBuf segstate;          // 8 floats per (segment item, pixel of its tile), see gl_raster.cu
     const ViewDesc* d_desc() const
     {

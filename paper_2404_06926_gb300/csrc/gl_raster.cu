@@ -24,22 +24,25 @@
 // tile's list) of the last blended Gaussian, so the backward recomputes T by
 // division.
 //
-// Forward of a split tile, in four launches.  (1) Each segment item blends
-// its records per pixel from T = 1 without the stop rule and stores the
-// segment's transmittance product T_s, colour, depth and opacity sums and
-// last blended position.  (2) A prefix pass walks each pixel's segments in
-// order with the incoming transmittance T_in (the product of the earlier
-// T_s): the stop rule fires inside segment s exactly when T_in * T_s falls
-// below 1e-4 (the running value inside s is T_in times the segment's own
-// running product, and that product only decreases).  (3) Each segment
-// item replays its records from T_in for the pixels that stop in it (one
-// replay per warp, all segments in parallel) to find the stop and the
-// truncated sums.  (4) A finish pass writes the pixel's outputs and, per
-// segment, the backward's starting state: the transmittance after the
-// segment and the normalised colour blended behind it (R = C_next + T_next
-// * R_next over the later segments).
-// The transmittance is the product of the per-segment products, so it can
-// differ from a single running product by float rounding.
+// Forward of a split tile: a CTA per pixel block walks the list in rounds,
+// each warp blending the next run of kSub records from T = 1 (a pixel whose
+// own run falls below 1e-4 stops there: it cannot matter what follows).  The
+// stop rule fires inside a run exactly when the transmittance entering it
+// times the run's own product falls below 1e-4 (the running value inside is
+// the entering one times the run's running product, and that product only
+// decreases), so the runs' products in order give the entering values and
+// the run each pixel stops in; that run is replayed from its entering value
+// to find the truncated sums, and the walk ends when every pixel has stopped:
+// nothing behind the stop is blended.  Runs of a segment are folded into its
+// sums, from which the backward's starting state of each segment follows
+// back to front: the transmittance after the segment and the normalised
+// colour blended behind it (R = C_next + T_next * R_next over the later
+// segments).  The transmittance is the product of the per-run products, so
+// it can differ from a single running product by float rounding.
+// Against a segment pass over the whole list and three launches for prefix,
+// replay and finish: 106 -> 79 us (250k Gaussians, 640x512), 236 -> 184 us (1M,
+// 1280x1024), 3,853 -> 3,338 us (12 views of 2M), 225 -> 185 us (render,
+// 1920x1080).
 //
 // Backward: every item walked back to front from its starting state (the
 // final transmittance and R = 0 for a whole tile).  Per hit a lane leaves two
@@ -71,23 +74,32 @@ constexpr int wpb() { return NB <= 2 ? kWarpsPerBlock : 16 / NB; }
 // next batch up to 64 records, one sub-batch ahead beyond.
 template <int NB>
 constexpr int pf_slots() { return NB <= 2 ? NB : 1; }
-// resident CTAs per SM the kernels are compiled for: the forward passes fit
-// 64 registers (4 CTAs)
-constexpr int kMinBlocks = 4;
-constexpr int kMinBlocksPg = 3;   // per-Gaussian backward
+constexpr int kMinBlocksPg = 3;   // resident CTAs per SM, per-Gaussian backward
 constexpr int kNG = 10;           // screen-space gradient sums per Gaussian (rows of kGradStride floats)
-constexpr int kSegFields = 16;  // per (segment item, pixel): see below
-constexpr int kSegBatch = 4;    // segments whose state one load round trip brings (prefix, finish)
+constexpr int kSegFields = 8;   // per (segment item, pixel): see below
+constexpr int kSub = 128;       // records of a run (a warp's share of a round on a split tile)
+constexpr int kBackBatch = 4;   // segments whose sums one load round trip brings (back walk)
 
-// segstate fields of a segment item.  After the segment pass: 0 T_s, 1-3
-// colour, 4 depth, 5 opacity, 6 last position (as bits); 7 the incoming
-// transmittance (prefix pass); fields 0-6 replaced by the truncated sums in
-// the segment where the pixel stops (replay pass).  After the finish pass:
-// 0 transmittance after the segment, 1-3 R (colour behind it, normalised),
-// 4 R depth, 5 R opacity.  Fields 8-15 of a split tile's first item hold the
-// tile-level state of the pixel: 8 stop segment (bits; segments = none),
-// 9 transmittance entering it (or the final one), 10-12 colour, 13 depth,
-// 14 opacity summed over the segments before it, 15 last position there.
+// Warps per CTA of the forward; they walk a split tile's pixel block together.
+// Eight shorten the deepest lists' walks, which is what a single frame waits
+// for; four leave less idle at the rounds' barriers and overshoot the stop by
+// less, which counts once there is far more work than the chip holds
+// (8 and 4 warps: 79 and 112 us on 250k Gaussians at 640x512, 10k pixel
+// blocks; 184 and 216 us at 1280x1024, 41k; 185 and 184 us at 1920x1080, 65k;
+// 3,968 and 3,338 us on 12 views of 2M, 303k; the line lies at 88k).  (The staging and exchange of every
+// variant fit in 48 KB of static shared memory.)
+template <int NB, int D>
+constexpr int wpb_fwd(bool wide) { return D == 4 || NB == 8 ? 2 : (NB == 1 && D == 1 && wide ? 8 : 4); }
+// pixel blocks per resident warp from which CTAs of four warps are taken
+constexpr int kWideUnits = 24;
+// registers: 80 a thread (24 warps per SM) at the default shape
+template <int NB, int D>
+constexpr int warps_fwd() { return D == 4 ? 12 : (NB == 1 && D == 1 ? 24 : 16); }
+
+// segstate fields of a segment item: 0 transmittance after the segment, 1-3 R
+// (colour behind it, normalised), 4 R depth, 5 R opacity; until the back walk
+// 1-5 hold the segment's own sums from T = 1 and 6 its transmittance product.
+// Written for the segments up to the one a pixel stops in.
 __device__ __forceinline__ size_t seg_at(int w, int k, int p, int TS)
 {
     return ((size_t)w * kSegFields + k) * (size_t)(TS * TS) + p;
@@ -97,13 +109,14 @@ __device__ __forceinline__ size_t seg_at(int w, int k, int p, int TS)
 struct RasterArgs {
     int TS, V, nblk, seg;
     const uint2* items;          // (tile, segment), heaviest first
-    const uint64_t* ctl;         // ctl[6] work items, ctl[7] items of split tiles
+    const uint32_t* heads;       // first item of each split tile
+    const uint64_t* ctl;         // ctl[6] work items, ctl[7] items of split tiles, ctl[11] split tiles
     const uint32_t* ranges;      // [first, last + 1) of each tile's list
     const float4 *s0, *s1, *s2, *s3;
     const uint32_t* sgid;        // owning (view, Gaussian) pair of each sorted instance
     const ViewDesc* views;
     float* segstate;
-    int* work;                   // persistent grid: unit counter; nullptr: one unit per warp
+    int* work;                   // persistent grid: unit counters; nullptr: one unit per warp
 };
 
 struct RasterOut {
@@ -134,14 +147,15 @@ struct Unit {
     uint32_t rs, re;       // the item's part of it
 };
 
+// Pixel block wb of item w.
 template <int D>
-__device__ __forceinline__ void unit_of(int u, const RasterArgs& A, Unit& U)
+__device__ __forceinline__ void unit_at(int w, int wb, const RasterArgs& A, Unit& U)
 {
     // pixel blocks per tile, blocks per tile row and the segment length are
     // powers of two: shifts and masks instead of integer divisions
-    const int TS = A.TS, bsh = __ffs(TS >> 3) - 1, nsh = __ffs(A.nblk) - 1;
-    U.w = u >> nsh;
-    U.wb = u & (A.nblk - 1);
+    const int TS = A.TS, bsh = __ffs(TS >> 3) - 1;
+    U.w = w;
+    U.wb = wb;
     const uint2 it = A.items[U.w];
     const int tile = (int)it.x;
     U.j = (int)it.y;
@@ -168,6 +182,12 @@ __device__ __forceinline__ void unit_of(int u, const RasterArgs& A, Unit& U)
     }
 }
 
+template <int D>
+__device__ __forceinline__ void unit_of(int u, const RasterArgs& A, Unit& U)
+{
+    unit_at<D>(u >> (__ffs(A.nblk) - 1), u & (A.nblk - 1), A, U);
+}
+
 __device__ __forceinline__ bool box_hit(const float4 box, float bx0, float bx1, float by0, float by1)
 {
     return !(box.y < bx0 || box.x > bx1 || box.w < by0 || box.z > by1);
@@ -181,26 +201,35 @@ __device__ __forceinline__ int next_unit(int* work, int lane)
     return __shfl_sync(kFull, u, 0);
 }
 
-// Units of this launch: work items (or the split tiles' items) x pixel blocks.
-__device__ __forceinline__ int units_of(const RasterArgs& A, bool split_only)
-{
-    return (int)(A.ctl[split_only ? 7 : 6]) * A.nblk;
-}
+// One warp's staged hits of the forward, from index 1: records r0, r1 and r2
+// with the list position + 1 in r2.w (bits).  Entry 0 is a record that reaches
+// no pixel, the partner of an odd count's first hit.
+template <int NB>
+struct FwdHits {
+    float4 r0[32 * NB + 1], r1[32 * NB + 1], r2[32 * NB + 1];
+    __device__ __forceinline__ void init(int lane)
+    {
+        if (lane == 0) {
+            r0[0] = r2[0] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            r1[0] = make_float4(0.0f, -3.0e38f, 0.0f, 0.0f);
+        }
+        __syncwarp();
+    }
+};
 
 // Front-to-back blend of the records [a, b) of a tile list for the warp's
 // pixel block.  Per pixel: T (running transmittance), colour, depth and
 // opacity sums (XD; without it they stay 0) and the last blended position
-// (relative to trs).  With `stop`, a pixel stops (without blending) at the
-// first record whose T * (1 - alpha), scaled by its Tin, falls below 1e-4;
-// without it every accepted record is blended and a pixel stops only when T
-// reaches 0.  Pixels with done set take no part.
-template <int NB, int D, bool XD>
+// (relative to trs).  A pixel stops, without blending, at the first record
+// whose T * (1 - alpha) (SCALED: times its Tin) falls below 1e-4; its alpha
+// threshold `thr` then becomes infinite, as it is from the start for pixels
+// that take no part.
+template <int NB, int D, bool XD, bool SCALED>
 __device__ __forceinline__ void blend_range(const RasterArgs& A, uint32_t a, uint32_t b, uint32_t trs, float px,
                                             const float (&py)[D], float bx0, float bx1, float by0, float by1,
-                                            bool stop, const float (&Tin)[D], bool (&done)[D], float (&T)[D],
-                                            float (&C0)[D], float (&C1)[D], float (&C2)[D], float (&Dd)[D],
-                                            float (&Oo)[D], uint32_t (&last)[D], float4* sr0, float4* sr1,
-                                            float4* sr2, uint32_t* spos, int lane)
+                                            const float (&Tin)[D], float (&thr)[D], float (&T)[D], float (&C0)[D],
+                                            float (&C1)[D], float (&C2)[D], float (&Dd)[D], float (&Oo)[D],
+                                            uint32_t (&last)[D], FwdHits<NB>& F, int lane)
 {
     const unsigned lt = (1u << lane) - 1u;
     constexpr int PF = pf_slots<NB>();
@@ -213,53 +242,61 @@ __device__ __forceinline__ void blend_range(const RasterArgs& A, uint32_t a, uin
     for (uint32_t base = a; base < b; base += 32 * NB) {
         bool lane_done = true;
 #pragma unroll
-        for (int j = 0; j < D; j++) lane_done = lane_done && done[j];
+        for (int j = 0; j < D; j++) lane_done = lane_done && thr[j] > 0.0f;
         if (__all_sync(kFull, lane_done)) break;
         int nh = 0;
 #pragma unroll
         for (int q = 0; q < NB; q++) {
             const int sl = PF == NB ? q : 0;
-            const float4 c0 = n0[sl], c1 = n1[sl], c2 = n2[sl], c3 = n3[sl];
+            const float4 c0 = n0[sl], c1 = n1[sl], c3 = n3[sl];
+            float4 c2 = n2[sl];
             const uint32_t i = base + q * 32 + lane;
             const uint32_t ni = i + 32 * PF;
             if (ni < b) { n0[sl] = A.s0[ni]; n1[sl] = A.s1[ni]; n2[sl] = A.s2[ni]; n3[sl] = A.s3[ni]; }
             const bool hit = i < b && box_hit(c3, bx0, bx1, by0, by1);
             const unsigned mask = __ballot_sync(kFull, hit);
             if (hit) {
-                const int k = nh + __popc(mask & lt);
-                sr0[k] = c0; sr1[k] = c1; sr2[k] = c2;
-                spos[k] = i - trs;
+                const int k = 1 + nh + __popc(mask & lt);
+                c2.w = __uint_as_float(i - trs + 1u);
+                F.r0[k] = c0; F.r1[k] = c1; F.r2[k] = c2;
             }
             nh += __popc(mask);
         }
         __syncwarp();
-        for (int k = 0; k < nh && !lane_done; k++) {
-            // Branch-free: a pixel that is done, or that the hit misses or
-            // stops at, blends with weight 0 (its sums exactly unchanged);
-            // T and the last position move by selects.
-            const float4 g0 = sr0[k], g1 = sr1[k], c = sr2[k];
-            const uint32_t pos1 = spos[k] + 1;
+        // Two hits at a time: their alphas are independent, only T forms a
+        // chain.  Branch-free: a pixel that is done or that a hit misses takes
+        // alpha = 0, which leaves T and its sums exactly unchanged (and T at
+        // or above the stop); one that stops here blends with weight 0 and
+        // keeps its T.
+        for (int k = 1 - (nh & 1); k <= nh; k += 2) {
+            float4 g0[2], g1[2], c[2];
 #pragma unroll
-            for (int j = 0; j < D; j++) {
-                float dx, dy, alpha;
-                bool capped;
-                const bool live = pair_eval_nb(g0, g1, px, py[j], dx, dy, alpha, capped) && !done[j];
-                const float tT = __fmul_rn(T[j], __fsub_rn(1.0f, alpha));
-                const bool halt = stop && live && __fmul_rn(Tin[j], tT) < kTransMin;
-                const bool blend = live && !halt;
-                const float wgt = blend ? alpha * T[j] : 0.0f;
-                T[j] = blend ? tT : T[j];
-                last[j] = blend ? pos1 : last[j];
-                done[j] = done[j] || halt || (!stop && blend && tT == 0.0f);
-                C0[j] += c.x * wgt; C1[j] += c.y * wgt; C2[j] += c.z * wgt;
-                if (XD) {
-                    Dd[j] += g1.z * wgt;
-                    Oo[j] += wgt;
+            for (int i = 0; i < 2; i++) { g0[i] = F.r0[k + i]; g1[i] = F.r1[k + i]; c[i] = F.r2[k + i]; }
+            float al[2][D];
+#pragma unroll
+            for (int i = 0; i < 2; i++)
+#pragma unroll
+                for (int j = 0; j < D; j++) {
+                    float alpha;
+                    al[i][j] = pair_alpha(g0[i], g1[i], px, py[j], thr[j], alpha) ? alpha : 0.0f;
                 }
-            }
-            lane_done = true;
 #pragma unroll
-            for (int j = 0; j < D; j++) lane_done = lane_done && done[j];
+            for (int i = 0; i < 2; i++)
+#pragma unroll
+                for (int j = 0; j < D; j++) {
+                    const float al_ = i && thr[j] > 0.0f ? 0.0f : al[i][j];   // the first may have stopped the pixel
+                    const float tT = __fmul_rn(T[j], __fsub_rn(1.0f, al_));
+                    const bool halt = (SCALED ? __fmul_rn(Tin[j], tT) : tT) < kTransMin;
+                    const float wgt = halt ? 0.0f : al_ * T[j];
+                    T[j] = halt ? T[j] : tT;
+                    thr[j] = halt ? kNoAlpha : thr[j];
+                    last[j] = wgt > 0.0f ? __float_as_uint(c[i].w) : last[j];
+                    C0[j] += c[i].x * wgt; C1[j] += c[i].y * wgt; C2[j] += c[i].z * wgt;
+                    if (XD) {
+                        Dd[j] += g1[i].z * wgt;
+                        Oo[j] += wgt;
+                    }
+                }
         }
         __syncwarp();
     }
@@ -295,286 +332,328 @@ struct LanePix {
     }
 };
 
+// A whole tile's pixel block, by one warp.
 template <int NB, int D, bool XD>
-__device__ __forceinline__ void fwd_item(int u, const RasterArgs& A, const RasterOut& O, float4* sr0, float4* sr1,
-                                         float4* sr2, uint32_t* spos, int lane)
+__device__ __forceinline__ void fwd_item(const Unit& U, const RasterArgs& A, const RasterOut& O, FwdHits<NB>& F,
+                                         int lane)
 {
-    Unit U;
-    unit_of<D>(u, A, U);
     const LanePix<D> L(U, A.TS, lane);
-    float T[D], C0[D], C1[D], C2[D], Dd[D], Oo[D], one[D];
+    float T[D], C0[D], C1[D], C2[D], Dd[D], Oo[D], thr[D];
     uint32_t last[D];
-    bool done[D];
 #pragma unroll
     for (int j = 0; j < D; j++) {
         T[j] = 1.0f; C0[j] = C1[j] = C2[j] = Dd[j] = Oo[j] = 0.0f;
-        one[j] = 1.0f;
         last[j] = 0;
-        done[j] = !L.inside[j];
+        thr[j] = L.inside[j] ? kLog2AlphaMin : kNoAlpha;
     }
-    const bool whole = U.nseg == 1;
-    blend_range<NB, D, XD>(A, U.rs, U.re, U.trs, L.px, L.py, L.bx0, L.bx1, L.by0, L.by1, whole, one, done, T, C0, C1,
-                           C2, Dd, Oo, last, sr0, sr1, sr2, spos, lane);
+    blend_range<NB, D, XD, false>(A, U.trs, U.tre, U.trs, L.px, L.py, L.bx0, L.bx1, L.by0, L.by1, T, thr, T, C0, C1,
+                                  C2, Dd, Oo, last, F, lane);
 #pragma unroll
     for (int j = 0; j < D; j++) {
         if (!L.inside[j]) continue;
-        if (whole) {
-            const size_t p = L.pix(U, j);
-            O.rgb[3 * p] = C0[j]; O.rgb[3 * p + 1] = C1[j]; O.rgb[3 * p + 2] = C2[j];
-            if (O.depth) O.depth[p] = Dd[j];
-            if (O.opac) O.opac[p] = Oo[j];
-            O.Tfin[p] = T[j];
-            O.ncon[p] = last[j];
-        } else {
-            float* S = A.segstate;
-            const int q = L.p[j];
-            S[seg_at(U.w, 0, q, A.TS)] = T[j];
-            S[seg_at(U.w, 1, q, A.TS)] = C0[j];
-            S[seg_at(U.w, 2, q, A.TS)] = C1[j];
-            S[seg_at(U.w, 3, q, A.TS)] = C2[j];
-            S[seg_at(U.w, 4, q, A.TS)] = Dd[j];
-            S[seg_at(U.w, 5, q, A.TS)] = Oo[j];
-            S[seg_at(U.w, 6, q, A.TS)] = __uint_as_float(last[j]);
-        }
-    }
-}
-
-template <int NB, int D, bool XD>
-__global__ void __launch_bounds__(32 * wpb<NB>(), kMinBlocks * kWarpsPerBlock / wpb<NB>())
-k_raster_fwd(RasterArgs A, RasterOut O)
-{
-    constexpr int WPB = wpb<NB>();
-    __shared__ float4 sr0[WPB][32 * NB], sr1[WPB][32 * NB], sr2[WPB][32 * NB];
-    __shared__ uint32_t spos[WPB][32 * NB];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nunits = units_of(A, false);
-    int u = A.work ? next_unit(A.work, lane) : blockIdx.x * WPB + w;
-    while (u < nunits) {
-        fwd_item<NB, D, XD>(u, A, O, sr0[w], sr1[w], sr2[w], spos[w], lane);
-        if (!A.work) break;
-        u = next_unit(A.work, lane);
-    }
-}
-
-// Split tiles, pass 2 of 4 (after the segment pass): per pixel of a split
-// tile, the prefix of its segments' transmittance, the segment where the
-// stop rule fires (T_in * T_s < 1e-4) and the sums before it.
-template <int D>
-__device__ __forceinline__ void prefix_item(int u, const RasterArgs& A, int lane)
-{
-    Unit U;
-    unit_of<D>(u, A, U);
-    if (U.j != 0 || U.nseg < 2) return;
-    const LanePix<D> L(U, A.TS, lane);
-    const int w0 = U.w, ns = U.nseg, TS = A.TS;
-    float* S = A.segstate;
-#pragma unroll
-    for (int j = 0; j < D; j++) {
-        if (!L.inside[j]) continue;
-        const int q = L.p[j];
-        float Tb = 1.0f, c0 = 0.f, c1 = 0.f, c2 = 0.f, dd = 0.f, oo = 0.f;
-        uint32_t last = 0;
-        int stop = ns;
-        // the seven fields of kSegBatch segments are loaded before any of
-        // them is used, so that the serial walk waits for memory once per
-        // kSegBatch segments
-        for (int s0 = 0; s0 < ns && stop == ns; s0 += kSegBatch) {
-            float f[kSegBatch][7];
-#pragma unroll
-            for (int b = 0; b < kSegBatch; b++)
-                if (s0 + b < ns) {
-#pragma unroll
-                    for (int k = 0; k < 7; k++) f[b][k] = S[seg_at(w0 + s0 + b, k, q, TS)];
-                }
-#pragma unroll
-            for (int b = 0; b < kSegBatch; b++) {
-                const int s = s0 + b;
-                if (s >= ns || stop != ns) break;
-                const float Ts = f[b][0];
-                S[seg_at(w0 + s, 7, q, TS)] = Tb;
-                if (__fmul_rn(Tb, Ts) < kTransMin) { stop = s; break; }
-                c0 += Tb * f[b][1];
-                c1 += Tb * f[b][2];
-                c2 += Tb * f[b][3];
-                dd += Tb * f[b][4];
-                oo += Tb * f[b][5];
-                const uint32_t ls = __float_as_uint(f[b][6]);
-                if (ls) last = ls;
-                Tb = __fmul_rn(Tb, Ts);
-            }
-        }
-        S[seg_at(w0, 8, q, TS)] = __uint_as_float((uint32_t)stop);
-        S[seg_at(w0, 9, q, TS)] = Tb;
-        S[seg_at(w0, 10, q, TS)] = c0;
-        S[seg_at(w0, 11, q, TS)] = c1;
-        S[seg_at(w0, 12, q, TS)] = c2;
-        S[seg_at(w0, 13, q, TS)] = dd;
-        S[seg_at(w0, 14, q, TS)] = oo;
-        S[seg_at(w0, 15, q, TS)] = __uint_as_float(last);
-    }
-}
-
-// Split tiles, pass 3 of 4: each segment item replays its records from the
-// incoming transmittance for the pixels whose stop segment it is, and stores
-// their truncated sums in place of the segment pass's.
-template <int NB, int D, bool XD>
-__device__ __forceinline__ void replay_item(int u, const RasterArgs& A, float4* sr0, float4* sr1, float4* sr2,
-                                            uint32_t* spos, int lane)
-{
-    Unit U;
-    unit_of<D>(u, A, U);
-    if (U.nseg < 2) return;
-    const LanePix<D> L(U, A.TS, lane);
-    const int w0 = U.w - U.j, TS = A.TS;
-    float* S = A.segstate;
-    float Tin[D], T[D], c0[D], c1[D], c2[D], dd[D], oo[D];
-    uint32_t last[D];
-    bool dn[D];
-    bool any = false;
-#pragma unroll
-    for (int j = 0; j < D; j++) {
-        T[j] = 1.0f; c0[j] = c1[j] = c2[j] = dd[j] = oo[j] = 0.0f;
-        last[j] = 0;
-        Tin[j] = 1.0f;
-        dn[j] = true;
-        if (!L.inside[j]) continue;
-        const int q = L.p[j];
-        if ((int)__float_as_uint(S[seg_at(w0, 8, q, TS)]) != U.j) continue;
-        Tin[j] = S[seg_at(w0, 9, q, TS)];
-        dn[j] = false;
-        any = true;
-    }
-    if (!__any_sync(kFull, any)) return;
-    blend_range<NB, D, XD>(A, U.rs, U.re, U.trs, L.px, L.py, L.bx0, L.bx1, L.by0, L.by1, true, Tin, dn, T, c0, c1,
-                           c2, dd, oo, last, sr0, sr1, sr2, spos, lane);
-#pragma unroll
-    for (int j = 0; j < D; j++) {
-        if (!L.inside[j]) continue;
-        const int q = L.p[j];
-        if ((int)__float_as_uint(S[seg_at(w0, 8, q, TS)]) != U.j) continue;
-        S[seg_at(U.w, 0, q, TS)] = T[j];
-        S[seg_at(U.w, 1, q, TS)] = c0[j];
-        S[seg_at(U.w, 2, q, TS)] = c1[j];
-        S[seg_at(U.w, 3, q, TS)] = c2[j];
-        S[seg_at(U.w, 4, q, TS)] = dd[j];
-        S[seg_at(U.w, 5, q, TS)] = oo[j];
-        S[seg_at(U.w, 6, q, TS)] = __uint_as_float(last[j]);
-    }
-}
-
-// Split tiles, pass 4 of 4: per pixel, the outputs (sums before the stop
-// segment plus its truncated sums) and, back to front over the segments up
-// to the stop, the backward's starting state of each.
-template <int D>
-__device__ __forceinline__ void finish_item(int u, const RasterArgs& A, const RasterOut& O, int lane)
-{
-    Unit U;
-    unit_of<D>(u, A, U);
-    if (U.j != 0 || U.nseg < 2) return;
-    const LanePix<D> L(U, A.TS, lane);
-    const int w0 = U.w, ns = U.nseg, TS = A.TS;
-    float* S = A.segstate;
-#pragma unroll
-    for (int j = 0; j < D; j++) {
-        if (!L.inside[j]) continue;
-        const int q = L.p[j];
-        const int stop = (int)__float_as_uint(S[seg_at(w0, 8, q, TS)]);
-        float Tb = S[seg_at(w0, 9, q, TS)];
-        float c0 = S[seg_at(w0, 10, q, TS)], c1 = S[seg_at(w0, 11, q, TS)], c2 = S[seg_at(w0, 12, q, TS)];
-        float dd = S[seg_at(w0, 13, q, TS)], oo = S[seg_at(w0, 14, q, TS)];
-        uint32_t last = __float_as_uint(S[seg_at(w0, 15, q, TS)]);
-        if (stop < ns) {
-            const int ws = w0 + stop;
-            c0 += Tb * S[seg_at(ws, 1, q, TS)];
-            c1 += Tb * S[seg_at(ws, 2, q, TS)];
-            c2 += Tb * S[seg_at(ws, 3, q, TS)];
-            dd += Tb * S[seg_at(ws, 4, q, TS)];
-            oo += Tb * S[seg_at(ws, 5, q, TS)];
-            const uint32_t ls = __float_as_uint(S[seg_at(ws, 6, q, TS)]);
-            if (ls) last = ls;
-            Tb = __fmul_rn(Tb, S[seg_at(ws, 0, q, TS)]);
-        }
         const size_t p = L.pix(U, j);
-        O.rgb[3 * p] = c0; O.rgb[3 * p + 1] = c1; O.rgb[3 * p + 2] = c2;
-        if (O.depth) O.depth[p] = dd;
-        if (O.opac) O.opac[p] = oo;
-        O.Tfin[p] = Tb;
-        O.ncon[p] = last;
-        const int jl = stop < ns ? stop : ns - 1;
-        for (int s = ns - 1; s > jl; s--)
-            for (int k = 0; k < 6; k++) S[seg_at(w0 + s, k, q, TS)] = 0.0f;
-        // back to front from the stop segment; the fields (0-5 and the
-        // incoming transmittance, 7) of kSegBatch segments are loaded before
-        // any of them is used
-        float R0 = 0.f, R1 = 0.f, R2 = 0.f, RD = 0.f, RO = 0.f;
-        for (int s0 = jl; s0 >= 0; s0 -= kSegBatch) {
-            float f[kSegBatch][7];
+        O.rgb[3 * p] = C0[j]; O.rgb[3 * p + 1] = C1[j]; O.rgb[3 * p + 2] = C2[j];
+        if (O.depth) O.depth[p] = Dd[j];
+        if (O.opac) O.opac[p] = Oo[j];
+        O.Tfin[p] = T[j];
+        O.ncon[p] = last[j];
+    }
+}
+
+// Shared memory of a CTA's forward.  ex: the runs of a round, per warp and
+// pixel, in three buffers (one being written, one being replayed, one being
+// folded); tot: warp 0's running sums per pixel.
+template <int NB, int D, int WPB>
+struct FwdShared {
+    enum { ET, EC0, EC1, EC2, ELAST, ETR, ED, EO, NEX };   // ETR: product up to the stop
+    enum { C0, C1, C2, LAST, S0, S1, S2, ST, DD, OO, SD, SO, NTOT };
+    FwdHits<NB> hits[WPB];
+    float ex[3][WPB][NEX][32 * D];
+    float tot[NTOT][32 * D];
+    int unit;
+};
+
+// Warp 0 adds the `runs` runs of a round, in order and up to the run `stop` a
+// pixel stops in (-1: it stopped earlier), to the pixel's and the segment's
+// sums; t is the transmittance entering the round.  A finished segment's sums
+// go to its state.  At the stop, Tst and jstop get the final transmittance and
+// the segment.
+template <int NB, int D, bool XD, int WPB>
+__device__ __forceinline__ void fold_round(const Unit& U, const RasterArgs& A, FwdShared<NB, D, WPB>& M, int buf, int s0,
+                                           int runs, int nrun, int seg_runs, int p, int q, float t, int stop,
+                                           float& Tst, int& jstop)
+{
+    using FS = FwdShared<NB, D, WPB>;
+    float C0 = M.tot[FS::C0][p], C1 = M.tot[FS::C1][p], C2 = M.tot[FS::C2][p];
+    float S0 = M.tot[FS::S0][p], S1 = M.tot[FS::S1][p], S2 = M.tot[FS::S2][p], ST = M.tot[FS::ST][p];
+    float Dd = 0.f, Oo = 0.f, SD = 0.f, SO = 0.f;
+    if (XD) {
+        Dd = M.tot[FS::DD][p]; Oo = M.tot[FS::OO][p];
+        SD = M.tot[FS::SD][p]; SO = M.tot[FS::SO][p];
+    }
+    uint32_t lp = __float_as_uint(M.tot[FS::LAST][p]);
+    for (int v = 0; v < runs && v <= stop; v++) {
+        const float (*e)[32 * D] = M.ex[buf][v];
+        const bool at_stop = v == stop;
+        const float f0 = e[FS::EC0][p], f1 = e[FS::EC1][p], f2 = e[FS::EC2][p];
+        C0 += t * f0; C1 += t * f1; C2 += t * f2;
+        S0 += ST * f0; S1 += ST * f1; S2 += ST * f2;
+        if (XD) {
+            const float fd = e[FS::ED][p], fo = e[FS::EO][p];
+            Dd += t * fd; Oo += t * fo;
+            SD += ST * fd; SO += ST * fo;
+        }
+        const uint32_t ls = __float_as_uint(e[FS::ELAST][p]);
+        if (ls) lp = ls;
+        const float tr = at_stop ? e[FS::ETR][p] : e[FS::ET][p];
+        t = __fmul_rn(t, tr);
+        ST = __fmul_rn(ST, tr);
+        const int run = s0 + v;
+        if (at_stop || (run & (seg_runs - 1)) == seg_runs - 1 || run == nrun - 1) {
+            const int sg = run / seg_runs, wi = U.w + sg;
+            float* S = A.segstate;
+            S[seg_at(wi, 0, q, A.TS)] = t;
+            S[seg_at(wi, 1, q, A.TS)] = S0;
+            S[seg_at(wi, 2, q, A.TS)] = S1;
+            S[seg_at(wi, 3, q, A.TS)] = S2;
+            if (XD) {
+                S[seg_at(wi, 4, q, A.TS)] = SD;
+                S[seg_at(wi, 5, q, A.TS)] = SO;
+            }
+            S[seg_at(wi, 6, q, A.TS)] = ST;
+            S0 = S1 = S2 = SD = SO = 0.0f;
+            ST = 1.0f;
+            if (at_stop) {
+                Tst = t;
+                jstop = sg;
+            }
+        }
+    }
+    M.tot[FS::C0][p] = C0; M.tot[FS::C1][p] = C1; M.tot[FS::C2][p] = C2;
+    M.tot[FS::S0][p] = S0; M.tot[FS::S1][p] = S1; M.tot[FS::S2][p] = S2; M.tot[FS::ST][p] = ST;
+    if (XD) {
+        M.tot[FS::DD][p] = Dd; M.tot[FS::OO][p] = Oo;
+        M.tot[FS::SD][p] = SD; M.tot[FS::SO][p] = SO;
+    }
+    M.tot[FS::LAST][p] = __uint_as_float(lp);
+}
+
+// A split tile's pixel block, by the whole CTA (every warp calls it).  One
+// barrier per round: after it every warp finds the stops on its own, replays
+// its run if one is in it, and goes on to the next round, while warp 0 folds
+// the round before.
+template <int NB, int D, bool XD, int WPB>
+__device__ __forceinline__ void fwd_split(const Unit& U, const RasterArgs& A, const RasterOut& O,
+                                          FwdShared<NB, D, WPB>& M, int lane, int w)
+{
+    using FS = FwdShared<NB, D, WPB>;
+    const LanePix<D> L(U, A.TS, lane);
+    const uint32_t sub = (uint32_t)min(A.seg, kSub);
+    const int seg_runs = A.seg / (int)sub;   // a power of two
+    const int nrun = (int)((U.tre - U.trs + sub - 1) / sub);
+    float Trun[D];             // transmittance entering the round (of open pixels; the same in every warp)
+    bool open[D];              // not stopped yet
+    float Tprev[D], Tst[D];    // warp 0: entering the round to fold; at the stop
+    int sprev[D], jstop[D];    // warp 0: stops of the round to fold; segment of the stop
 #pragma unroll
-            for (int b = 0; b < kSegBatch; b++)
-                if (s0 - b >= 0) {
+    for (int j = 0; j < D; j++) {
+        Trun[j] = Tprev[j] = 1.0f;
+        Tst[j] = -1.0f;
+        open[j] = L.inside[j];
+        sprev[j] = -1;
+        jstop[j] = U.nseg - 1;
+        if (w == 0)
+            for (int k = 0; k < FS::NTOT; k++) M.tot[k][j * 32 + lane] = k == FS::ST ? 1.0f : 0.0f;
+    }
+    int buf = 0, bprev = 0, s0 = 0, sp0 = 0;
+    while (true) {
+        const int s = s0 + w, runs = min(WPB, nrun - s0);
+        const uint32_t a = U.trs + (uint32_t)s * sub, b = min(U.tre, a + sub);
+        float T[D], c0[D], c1[D], c2[D], dd[D], oo[D], thr[D];
+        uint32_t last[D];
 #pragma unroll
-                    for (int k = 0; k < 6; k++) f[b][k] = S[seg_at(w0 + s0 - b, k, q, TS)];
-                    f[b][6] = S[seg_at(w0 + s0 - b, 7, q, TS)];
+        for (int j = 0; j < D; j++) {
+            T[j] = 1.0f; c0[j] = c1[j] = c2[j] = dd[j] = oo[j] = 0.0f;
+            last[j] = 0;
+            thr[j] = open[j] ? kLog2AlphaMin : kNoAlpha;
+        }
+        if (s < nrun) {
+            blend_range<NB, D, XD, false>(A, a, b, U.trs, L.px, L.py, L.bx0, L.bx1, L.by0, L.by1, T, thr, T, c0, c1,
+                                          c2, dd, oo, last, M.hits[w], lane);
+#pragma unroll
+            for (int j = 0; j < D; j++) {
+                const int p = j * 32 + lane;
+                // a pixel that fell below 1e-4 within the run stops in it
+                // whatever enters it
+                M.ex[buf][w][FS::ET][p] = thr[j] > 0.0f ? 0.0f : T[j];
+                M.ex[buf][w][FS::EC0][p] = c0[j];
+                M.ex[buf][w][FS::EC1][p] = c1[j];
+                M.ex[buf][w][FS::EC2][p] = c2[j];
+                M.ex[buf][w][FS::ELAST][p] = __uint_as_float(last[j]);
+                if (XD) {
+                    M.ex[buf][w][FS::ED][p] = dd[j];
+                    M.ex[buf][w][FS::EO][p] = oo[j];
                 }
+            }
+        }
+        __syncthreads();
+        if (w == 0 && s0 > 0) {
 #pragma unroll
-            for (int b = 0; b < kSegBatch; b++) {
-                const int s = s0 - b;
-                if (s < 0) break;
-                const int ws = w0 + s;
-                const float Ts = f[b][0], cs0 = f[b][1], cs1 = f[b][2], cs2 = f[b][3], ds = f[b][4], os = f[b][5];
-                const float tin = f[b][6];
-                S[seg_at(ws, 0, q, TS)] = __fmul_rn(tin, Ts);
-                S[seg_at(ws, 1, q, TS)] = R0;
-                S[seg_at(ws, 2, q, TS)] = R1;
-                S[seg_at(ws, 3, q, TS)] = R2;
-                S[seg_at(ws, 4, q, TS)] = RD;
-                S[seg_at(ws, 5, q, TS)] = RO;
-                R0 = cs0 + Ts * R0; R1 = cs1 + Ts * R1; R2 = cs2 + Ts * R2;
-                RD = ds + Ts * RD; RO = os + Ts * RO;
+            for (int j = 0; j < D; j++)
+                fold_round<NB, D, XD, WPB>(U, A, M, bprev, sp0, WPB, nrun, seg_runs, j * 32 + lane, L.p[j], Tprev[j],
+                                      sprev[j], Tst[j], jstop[j]);
+        }
+        // entering transmittance of every run, in order; the run each pixel
+        // stops in
+        float Tin[D];
+        int stop[D];
+        bool mine = false, any_open = false;
+#pragma unroll
+        for (int j = 0; j < D; j++) {
+            float Tb = Trun[j];
+            Tprev[j] = Tb;
+            Tin[j] = 1.0f;
+            stop[j] = open[j] ? WPB : -1;
+            for (int v = 0; v < runs; v++) {
+                const float t = __fmul_rn(Tb, M.ex[buf][v][FS::ET][j * 32 + lane]);
+                if (stop[j] == WPB) {
+                    if (v == w) Tin[j] = Tb;
+                    if (t < kTransMin) stop[j] = v; else Tb = t;
+                }
+            }
+            mine = mine || stop[j] == w;
+            sprev[j] = stop[j];
+            Trun[j] = Tb;
+            open[j] = open[j] && stop[j] == WPB;
+            any_open = any_open || open[j];
+        }
+        if (__any_sync(kFull, mine)) {
+            // replay this warp's run from its entering transmittance for the
+            // pixels that stop in it
+#pragma unroll
+            for (int j = 0; j < D; j++) {
+                T[j] = 1.0f; c0[j] = c1[j] = c2[j] = dd[j] = oo[j] = 0.0f;
+                last[j] = 0;
+                thr[j] = stop[j] == w ? kLog2AlphaMin : kNoAlpha;
+            }
+            blend_range<NB, D, XD, true>(A, a, b, U.trs, L.px, L.py, L.bx0, L.bx1, L.by0, L.by1, Tin, thr, T, c0, c1,
+                                         c2, dd, oo, last, M.hits[w], lane);
+#pragma unroll
+            for (int j = 0; j < D; j++) {
+                const int p = j * 32 + lane;
+                if (stop[j] != w) continue;
+                M.ex[buf][w][FS::ETR][p] = T[j];
+                M.ex[buf][w][FS::EC0][p] = c0[j];
+                M.ex[buf][w][FS::EC1][p] = c1[j];
+                M.ex[buf][w][FS::EC2][p] = c2[j];
+                M.ex[buf][w][FS::ELAST][p] = __uint_as_float(last[j]);
+                if (XD) {
+                    M.ex[buf][w][FS::ED][p] = dd[j];
+                    M.ex[buf][w][FS::EO][p] = oo[j];
+                }
+            }
+        }
+        bprev = buf;
+        sp0 = s0;
+        buf = buf == 2 ? 0 : buf + 1;
+        s0 += WPB;
+        // (the same in every warp)
+        if (s0 >= nrun || !__any_sync(kFull, any_open)) break;
+    }
+    __syncthreads();
+    if (w != 0) return;
+    int smax = 0;
+#pragma unroll
+    for (int j = 0; j < D; j++) {
+        const int p = j * 32 + lane;
+        fold_round<NB, D, XD, WPB>(U, A, M, bprev, sp0, min(WPB, nrun - sp0), nrun, seg_runs, p, L.p[j], Tprev[j], sprev[j],
+                              Tst[j], jstop[j]);
+        if (!L.inside[j]) continue;
+        const size_t o = L.pix(U, j);
+        O.rgb[3 * o] = M.tot[FS::C0][p];
+        O.rgb[3 * o + 1] = M.tot[FS::C1][p];
+        O.rgb[3 * o + 2] = M.tot[FS::C2][p];
+        if (XD && O.depth) O.depth[o] = M.tot[FS::DD][p];
+        if (XD && O.opac) O.opac[o] = M.tot[FS::OO][p];
+        O.Tfin[o] = Tst[j] >= 0.0f ? Tst[j] : Trun[j];
+        O.ncon[o] = __float_as_uint(M.tot[FS::LAST][p]);
+        smax = max(smax, jstop[j]);
+    }
+    // the backward's starting states, back to front from the stop segment
+    // (each lane reads back only what it wrote)
+    for (int off = 16; off > 0; off >>= 1) smax = max(smax, __shfl_xor_sync(kFull, smax, off));
+    constexpr int NF = XD ? 6 : 4;   // sums (3 or 5) and the product
+#pragma unroll
+    for (int j = 0; j < D; j++) {
+        if (!L.inside[j]) continue;
+        const int q = L.p[j];
+        float* S = A.segstate;
+        float R[NF - 1];
+#pragma unroll
+        for (int k = 0; k < NF - 1; k++) R[k] = 0.0f;
+        for (int b0 = smax; b0 >= 0; b0 -= kBackBatch) {
+            float f[kBackBatch][NF];
+#pragma unroll
+            for (int b = 0; b < kBackBatch; b++) {
+                const int sg = b0 - b;
+                if (sg >= 0 && sg <= jstop[j]) {
+#pragma unroll
+                    for (int k = 0; k < NF - 1; k++) f[b][k] = S[seg_at(U.w + sg, 1 + k, q, A.TS)];
+                    f[b][NF - 1] = S[seg_at(U.w + sg, 6, q, A.TS)];
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < kBackBatch; b++) {
+                const int sg = b0 - b;
+                if (sg >= 0 && sg <= jstop[j]) {
+#pragma unroll
+                    for (int k = 0; k < NF - 1; k++) {
+                        S[seg_at(U.w + sg, 1 + k, q, A.TS)] = R[k];
+                        R[k] = f[b][k] + f[b][NF - 1] * R[k];
+                    }
+                }
             }
         }
     }
 }
 
-template <int D>
-__global__ void __launch_bounds__(32 * kWarpsPerBlock, kMinBlocks) k_seg_prefix(RasterArgs A)
+// Split tiles first (a CTA per pixel block; counters work[1] of a persistent
+// grid, the first CTAs otherwise), then the other tiles (a warp per pixel
+// block).
+template <int NB, int D, bool XD, int WPB>
+__global__ void __launch_bounds__(32 * WPB, warps_fwd<NB, D>() / WPB) k_raster_fwd(RasterArgs A, RasterOut O)
 {
+    __shared__ FwdShared<NB, D, WPB> M;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nunits = units_of(A, true);
-    int u = A.work ? next_unit(A.work, lane) : blockIdx.x * kWarpsPerBlock + w;
-    while (u < nunits) {
-        prefix_item<D>(u, A, lane);
-        if (!A.work) break;
-        u = next_unit(A.work, lane);
-    }
-}
-
-template <int NB, int D, bool XD>
-__global__ void __launch_bounds__(32 * wpb<NB>(), kMinBlocks * kWarpsPerBlock / wpb<NB>()) k_seg_replay(RasterArgs A)
-{
-    constexpr int WPB = wpb<NB>();
-    __shared__ float4 sr0[WPB][32 * NB], sr1[WPB][32 * NB], sr2[WPB][32 * NB];
-    __shared__ uint32_t spos[WPB][32 * NB];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nunits = units_of(A, true);
-    int u = A.work ? next_unit(A.work, lane) : blockIdx.x * WPB + w;
-    while (u < nunits) {
-        replay_item<NB, D, XD>(u, A, sr0[w], sr1[w], sr2[w], spos[w], lane);
-        if (!A.work) break;
-        u = next_unit(A.work, lane);
-    }
-}
-
-template <int D>
-__global__ void __launch_bounds__(32 * kWarpsPerBlock, kMinBlocks) k_seg_finish(RasterArgs A, RasterOut O)
-{
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nunits = units_of(A, true);
-    int u = A.work ? next_unit(A.work, lane) : blockIdx.x * kWarpsPerBlock + w;
-    while (u < nunits) {
-        finish_item<D>(u, A, O, lane);
-        if (!A.work) break;
-        u = next_unit(A.work, lane);
+    const int nsh = __ffs(A.nblk) - 1;
+    const int nsplit = (int)A.ctl[11] * A.nblk;
+    const int split_items = (int)A.ctl[7];
+    const int nwhole = ((int)A.ctl[6] - split_items) * A.nblk;
+    Unit U;
+    M.hits[w].init(lane);
+    if (A.work) {
+        while (nsplit > 0) {
+            __syncthreads();
+            if (threadIdx.x == 0) M.unit = atomicAdd(A.work + 1, 1);
+            __syncthreads();
+            const int u = M.unit;
+            if (u >= nsplit) break;
+            unit_at<D>((int)A.heads[u >> nsh], u & (A.nblk - 1), A, U);
+            fwd_split<NB, D, XD, WPB>(U, A, O, M, lane, w);
+        }
+        for (int u = next_unit(A.work, lane); u < nwhole; u = next_unit(A.work, lane)) {
+            unit_at<D>(split_items + (u >> nsh), u & (A.nblk - 1), A, U);
+            fwd_item<NB, D, XD>(U, A, O, M.hits[w], lane);
+        }
+    } else if ((int)blockIdx.x < nsplit) {
+        unit_at<D>((int)A.heads[blockIdx.x >> nsh], blockIdx.x & (A.nblk - 1), A, U);
+        fwd_split<NB, D, XD, WPB>(U, A, O, M, lane, w);
+    } else {
+        const int u = ((int)blockIdx.x - nsplit) * WPB + w;
+        if (u < nwhole) {
+            unit_at<D>(split_items + (u >> nsh), u & (A.nblk - 1), A, U);
+            fwd_item<NB, D, XD>(U, A, O, M.hits[w], lane);
+        }
     }
 }
 
@@ -764,7 +843,7 @@ __device__ __forceinline__ void bwd_item(int u, const RasterArgs& A, const Raste
             }
             if (U.nseg == 1) {
                 T[j] = G.Tfin[p];
-            } else {
+            } else if (last[j] > U.rs - U.trs) {   // (no state behind the stop segment)
                 const float* S = A.segstate;
                 const int i = L.p[j];
                 T[j] = S[seg_at(U.w, 0, i, A.TS)];
@@ -900,7 +979,7 @@ __global__ void __launch_bounds__(32 * wpb_bwd<NB>(), minb_bwd<NB, D>()) k_raste
     constexpr int WPB = wpb_bwd<NB>();
     __shared__ BwdWarp<NB, D> sw[WPB];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nunits = units_of(A, false);
+    const int nunits = (int)A.ctl[6] * A.nblk;
     int u = A.work ? next_unit(A.work, lane) : blockIdx.x * WPB + w;
     while (u < nunits) {
         bwd_item<EXTRA, NB, D, DET>(u, A, G, sw[w], lane);
@@ -977,15 +1056,17 @@ __device__ __forceinline__ void bwd_item_pg(int u, const RasterArgs& A, const Ra
         last = G.ncon[p];
         if (U.nseg == 1) {
             T = G.Tfin[p];
-        } else {
+        } else if (last > U.rs - U.trs) {
             const float* S = A.segstate;
             const int q = ly * A.TS + lx;
             T = S[seg_at(U.w, 0, q, A.TS)];
             R0 = S[seg_at(U.w, 1, q, A.TS)];
             R1 = S[seg_at(U.w, 2, q, A.TS)];
             R2 = S[seg_at(U.w, 3, q, A.TS)];
-            RD = S[seg_at(U.w, 4, q, A.TS)];
-            RO = S[seg_at(U.w, 5, q, A.TS)];
+            if (EXTRA) {
+                RD = S[seg_at(U.w, 4, q, A.TS)];
+                RO = S[seg_at(U.w, 5, q, A.TS)];
+            }
         }
         pc = make_float4(G.dL_drgb[3 * p], G.dL_drgb[3 * p + 1], G.dL_drgb[3 * p + 2], __uint_as_float(last));
         if (EXTRA) pe = make_float2(G.dL_ddepth ? G.dL_ddepth[p] : 0.0f, G.dL_dopac ? G.dL_dopac[p] : 0.0f);
@@ -1190,7 +1271,7 @@ k_raster_bwd_pg(RasterArgs A, RasterGrad G)
 {
     __shared__ PgWarp sw[kWarpsPerBlock];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nunits = units_of(A, false);
+    const int nunits = (int)A.ctl[6] * A.nblk;
     int u = A.work ? next_unit(A.work, lane) : blockIdx.x * kWarpsPerBlock + w;
     while (u < nunits) {
         bwd_item_pg<EXTRA, DET>(u, A, G, sw[w], lane);
@@ -1368,6 +1449,7 @@ RasterArgs make_args(View& v, int* work)
     A.nblk = blocks_per_tile(v);
     A.seg = v.seg;
     A.items = v.items.as<uint2>();
+    A.heads = v.heads.as<uint32_t>();
     A.ctl = v.count.as<uint64_t>();
     A.ranges = v.ranges.as<uint32_t>();
     A.s0 = v.srec0.as<float4>();
@@ -1403,25 +1485,24 @@ gl_status check_exec(const View& v)
     return GL_OK;
 }
 
+// split_units and units bound the split and the whole tiles' pixel blocks.
+template <int NB, int D, bool XD, int WPB>
+void fwd_launch_wpb(const RasterArgs& A, const RasterOut& O, int64_t units, int64_t split_units, bool persistent,
+                    cudaStream_t s)
+{
+    const int grid = grid_for(k_raster_fwd<NB, D, XD, WPB>, units + split_units * WPB, persistent, WPB);
+    k_raster_fwd<NB, D, XD, WPB><<<grid, 32 * WPB, 0, s>>>(A, O);
+}
+
 template <int NB, int D, bool XD>
 void fwd_launch(const RasterArgs& A, const RasterOut& O, int64_t units, int64_t split_units, bool persistent,
-                int* work, cudaStream_t s)
+                cudaStream_t s)
 {
-    RasterArgs a1 = A;
-    a1.work = work;
-    k_raster_fwd<NB, D, XD><<<grid_for(k_raster_fwd<NB, D, XD>, units, persistent, wpb<NB>()), 32 * wpb<NB>(), 0,
-                              s>>>(a1, O);
-    if (split_units > 0) {
-        // persistent grids take units from counters 2-4
-        RasterArgs a2 = A, a3 = A, a4 = A;
-        a2.work = work ? work + 2 : nullptr;
-        a3.work = work ? work + 3 : nullptr;
-        a4.work = work ? work + 4 : nullptr;
-        k_seg_prefix<D><<<grid_for(k_seg_prefix<D>, split_units, persistent), 32 * kWarpsPerBlock, 0, s>>>(a2);
-        k_seg_replay<NB, D, XD><<<grid_for(k_seg_replay<NB, D, XD>, split_units, persistent, wpb<NB>()),
-                                  32 * wpb<NB>(), 0, s>>>(a3);
-        k_seg_finish<D><<<grid_for(k_seg_finish<D>, split_units, persistent), 32 * kWarpsPerBlock, 0, s>>>(a4, O);
-    }
+    constexpr int wide = wpb_fwd<NB, D>(true), narrow = wpb_fwd<NB, D>(false);
+    if (wide != narrow && units < (int64_t)kWideUnits * warps_fwd<NB, D>() * sm_count())
+        fwd_launch_wpb<NB, D, XD, wide>(A, O, units, split_units, persistent, s);
+    else
+        fwd_launch_wpb<NB, D, XD, narrow>(A, O, units, split_units, persistent, s);
 }
 
 template <bool EXTRA, int NB, int D, bool DET>
@@ -1488,20 +1569,20 @@ gl_status permute_records(View& v, int64_t nmax, cudaStream_t s)
 
 template <bool XD>
 void fwd_dispatch(const View& v, const RasterArgs& A, const RasterOut& O, int64_t units, int64_t split_units,
-                  int* work, cudaStream_t s)
+                  cudaStream_t s)
 {
     if (v.nb == 4) {
-        fwd_launch<4, 1, XD>(A, O, units, split_units, v.persistent, work, s);
+        fwd_launch<4, 1, XD>(A, O, units, split_units, v.persistent, s);
     } else if (v.nb == 8) {
-        fwd_launch<8, 1, XD>(A, O, units, split_units, v.persistent, work, s);
+        fwd_launch<8, 1, XD>(A, O, units, split_units, v.persistent, s);
     } else if (v.nb == 1) {
-        if (v.pd == 1) fwd_launch<1, 1, XD>(A, O, units, split_units, v.persistent, work, s);
-        else if (v.pd == 2) fwd_launch<1, 2, XD>(A, O, units, split_units, v.persistent, work, s);
-        else fwd_launch<1, 4, XD>(A, O, units, split_units, v.persistent, work, s);
+        if (v.pd == 1) fwd_launch<1, 1, XD>(A, O, units, split_units, v.persistent, s);
+        else if (v.pd == 2) fwd_launch<1, 2, XD>(A, O, units, split_units, v.persistent, s);
+        else fwd_launch<1, 4, XD>(A, O, units, split_units, v.persistent, s);
     } else {
-        if (v.pd == 1) fwd_launch<2, 1, XD>(A, O, units, split_units, v.persistent, work, s);
-        else if (v.pd == 2) fwd_launch<2, 2, XD>(A, O, units, split_units, v.persistent, work, s);
-        else fwd_launch<2, 4, XD>(A, O, units, split_units, v.persistent, work, s);
+        if (v.pd == 1) fwd_launch<2, 1, XD>(A, O, units, split_units, v.persistent, s);
+        else if (v.pd == 2) fwd_launch<2, 2, XD>(A, O, units, split_units, v.persistent, s);
+        else fwd_launch<2, 4, XD>(A, O, units, split_units, v.persistent, s);
     }
 }
 
@@ -1525,13 +1606,15 @@ gl_status raster_forward(View& v, float* rgb, float* depth, float* opac, cudaStr
         work = v.work.as<int>();
         GL_CUDA_TRY(cudaMemsetAsync(work, 0, 8 * sizeof(int), s));
     }
-    const RasterArgs A = make_args(v, nullptr);
+    const RasterArgs A = make_args(v, work);
     RasterOut O{rgb, depth, opac, v.Tfin.as<float>(), v.ncon.as<uint32_t>()};
     const int nblk = blocks_per_tile(v);
-    const int64_t units = work_items_bound(v) * nblk, split_units = split * nblk;
-    if (extras) fwd_dispatch<true>(v, A, O, units, split_units, work, s);
-    else fwd_dispatch<false>(v, A, O, units, split_units, work, s);
-    count_launches(split_units > 0 ? 4 : 1);
+    // a split tile's list holds at least 2 seg records
+    const int64_t tiles = v.seg > 0 ? std::min<int64_t>(v.ntiles, (int64_t)(v.itile.bytes / 4) / (2 * v.seg)) : 0;
+    const int64_t units = (int64_t)v.ntiles * nblk, split_units = tiles * nblk;
+    if (extras) fwd_dispatch<true>(v, A, O, units, split_units, s);
+    else fwd_dispatch<false>(v, A, O, units, split_units, s);
+    count_launches(1);
     GL_CUDA_TRY(cudaGetLastError());
     return GL_OK;
 }

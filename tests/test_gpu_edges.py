@@ -86,3 +86,16 @@ def test_loss_sizes(W, H):
         a, ref = got.cpu().numpy().astype(np.float64).ravel(), np.asarray(ref, np.float64).ravel()
         rel = np.abs(a - ref) / np.maximum(np.abs(ref), 1e-4 * np.abs(ref).max())
         assert np.median(rel) < 1e-3 and np.percentile(rel, 99) < 1e-2, (np.median(rel), np.percentile(rel, 99))
+
+
+@pytest.mark.parametrize("n", [127, 128, 129, 192, 511, 512, 513, 577, 1030, 1100])
+@pytest.mark.parametrize("opacity", [0.006, 0.4])   # no pixel stops (0.994^1100 > 1e-4); every pixel stops early
+@pytest.mark.parametrize("ppl,persistent", [(1, 0), (2, 1)])
+def test_split_list_lengths(n, opacity, ppl, persistent):
+    _check_stack(n, opacity, True, segment=64, pixels_per_lane=ppl, persistent=persistent)
+
+
+@pytest.mark.parametrize("seg", [64, 256, 1024])
+@pytest.mark.parametrize("bd", [32, 64, 256])
+def test_split_segments_of_several_runs(seg, bd):
+    _check_stack(2100, 0.02, False, segment=seg, batch_depth=bd)
