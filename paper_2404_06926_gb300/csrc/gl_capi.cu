@@ -232,8 +232,8 @@ gl_status View::upload_descs(cudaStream_t s)
 
 void View::release()
 {
-    DevBuf* all[] = {&rec0, &rec1, &rec2, &rec3, &radius, &rect, &touched, &dkey, &gidx, &dkey2, &gidx2,
-                     &dup_off, &bsum, &count, &itile, &ival, &itile2, &ival2, &iowner, &srec0, &srec1, &srec2, &srec3, &sgid, &g2d, &gpart, &gmask, &work, &items, &heads, &segstate, &kmask,
+    DevBuf* all[] = {&rec, &radius, &brec, &touched, &dkey, &gidx, &dkey2, &gidx2,
+                     &dup_off, &bsum, &count, &itile, &ival, &itile2, &ival2, &iowner, &srec0, &srec1, &srec2, &srec3, &sgid, &g2d, &gpart, &gmask, &work, &items, &heads, &segstate,
                      &hist, &ranges, &tile_order, &Tfin, &ncon, &rgb, &depth, &opac};
     for (DevBuf* b : all) b->release();
     desc.release();
@@ -609,8 +609,7 @@ extern "C" gl_status gl_ctx_get_preprocess(gl_ctx* ctx, int32_t* radius, int32_t
     const size_t n = (size_t)v.n;
     if (n == 0) return GL_OK;
     if (radius) GL_CUDA_TRY(cudaMemcpyAsync(radius, v.radius.p, 4 * n, cudaMemcpyDeviceToDevice, s));
-    if (rect) GL_CUDA_TRY(cudaMemcpyAsync(rect, v.rect.p, 16 * n, cudaMemcpyDeviceToDevice, s));
-    return export_preprocess(v, mean2d, conic, opacity, rgb, depth, s);
+    return export_preprocess(v, rect, mean2d, conic, opacity, rgb, depth, s);
 }
 
 extern "C" gl_status gl_ctx_num_instances(gl_ctx* ctx, int64_t* I_out)
@@ -1169,11 +1168,11 @@ std::vector<int64_t> graph_key(const gl_map* m, const StepPlan& sp)
         k.push_back(sp.cams[i].H);
     }
     const View& v = m->ctx.view;
-    const DevBuf* bufs[] = {&v.rec0, &v.rec1, &v.rec2, &v.rec3, &v.radius, &v.rect, &v.touched, &v.dkey,
+    const DevBuf* bufs[] = {&v.rec, &v.radius, &v.brec, &v.touched, &v.dkey,
                             &v.gidx, &v.dkey2, &v.gidx2, &v.dup_off, &v.g2d, &v.bsum, &v.count, &v.itile,
                             &v.ival, &v.itile2, &v.ival2, &v.iowner, &v.srec0, &v.srec1, &v.srec2, &v.srec3,
                             &v.sgid, &v.hist, &v.ranges, &v.tile_order, &v.Tfin, &v.ncon, &v.rgb, &v.work, &v.gpart, &v.gmask,
-                            &v.items, &v.heads, &v.segstate, &v.kmask,
+                            &v.items, &v.heads, &v.segstate,
                             &v.desc, &m->dLdC, &m->ctx.loss_part, &m->loss_dev};
     for (const DevBuf* b : bufs) {
         k.push_back((int64_t)(uintptr_t)b->p);

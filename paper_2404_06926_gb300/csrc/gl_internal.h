@@ -145,14 +145,13 @@ struct View {
     bool pin_used[kDescRing] = {};
     int pin_slot = 0;
     // per (view, Gaussian)
-    DevBuf rec0, rec1, rec2, rec3;  // float4: (u,v,A',C'), (B',log2 o,z,o), (r,g,b,-), alpha box
+    DevBuf rec;               // 64 bytes: (u,v,A',C'), (B',log2 o,z,v_lo), (r,g,b,u_lo), alpha box
     DevBuf radius;            // int
-    DevBuf rect;              // int4 (x0,y0,x1,y1), tiles local to the view
+    DevBuf brec;              // uint4 kept-tile mask and tile rectangle (local to the view), see pack_bin
     DevBuf touched;           // u32
     DevBuf dkey, gidx;        // u32 depth key (sort input); u32 index (sort output buffer)
     DevBuf dkey2, gidx2;      // sort ping-pong
     DevBuf dup_off;           // u32 offset of the Gaussian's first instance
-    DevBuf kmask;             // u64 kept-tile mask of the rectangle (all ones if it is not culled)
     DevBuf g2d;               // screen-space gradient accumulators (rows of kGradStride floats)
     // scan
     DevBuf bsum;              // u64 per scan block: instance offset, then duplication-part offset
@@ -332,7 +331,7 @@ gl_status accumulate_view_counts(const View& v, uint64_t* acc, cudaStream_t s);
 gl_status view_counts(const View& v, int64_t* n_visible, int64_t* sum_contrib, cudaStream_t s);
 
 // Projected quantities of the last view in plain form (null outputs skipped).
-gl_status export_preprocess(const View& v, float* mean2d, float* conic, float* opacity, float* rgb,
+gl_status export_preprocess(const View& v, int32_t* rect, float* mean2d, float* conic, float* opacity, float* rgb,
                             float* depth, cudaStream_t s);
 
 // Sorted instances as (tile << 32 | depth bits) keys and owning Gaussians.

@@ -1379,9 +1379,8 @@ k_part_reduce(const float* __restrict__ part, const uint32_t* __restrict__ pmask
 __global__ void k_permute(const uint64_t* __restrict__ n_dev, uint32_t* __restrict__ ranges,
                           const uint32_t* __restrict__ sinst,
                           const uint32_t* __restrict__ stile, const ViewDesc* __restrict__ views, int V, int TS,
-                          const uint32_t* __restrict__ owner, const float4* __restrict__ r0,
-                          const float4* __restrict__ r1, const float4* __restrict__ r2,
-                          const float4* __restrict__ r3, float4* __restrict__ s0, float4* __restrict__ s1,
+                          const uint32_t* __restrict__ owner, const float4* __restrict__ rec,
+                          float4* __restrict__ s0, float4* __restrict__ s1,
                           float4* __restrict__ s2, float4* __restrict__ s3, uint32_t* __restrict__ sg)
 {
     const uint64_t I = *n_dev;
@@ -1393,11 +1392,12 @@ __global__ void k_permute(const uint64_t* __restrict__ n_dev, uint32_t* __restri
         const ViewDesc& d = views[view_of_tile(views, V, tile)];
         const int lt = tile - d.tile_base;
         const float x0 = (float)((lt % d.TX) * TS), y0 = (float)((lt / d.TX) * TS);
-        float4 a = r0[g];
-        const float4 b = r1[g], c = r2[g];
+        float4 a, b, c, box;
+        ld_sector(rec + 4 * (size_t)g, a, b);
+        ld_sector(rec + 4 * (size_t)g + 2, c, box);
         a.x = __fadd_rn(__fsub_rn(a.x, x0), c.w);
         a.y = __fadd_rn(__fsub_rn(a.y, y0), b.w);
-        s0[i] = a; s1[i] = b; s2[i] = c; s3[i] = r3[g];
+        s0[i] = a; s1[i] = b; s2[i] = c; s3[i] = box;
         sg[i] = g;
     }
 }
@@ -1559,8 +1559,7 @@ gl_status permute_records(View& v, int64_t nmax, cudaStream_t s)
     const int blocks = (int)std::min<size_t>(8 * (size_t)sm_count(), (I + 255) / 256);
     k_permute<<<blocks, 256, 0, s>>>(v.count.as<uint64_t>(), v.ranges.as<uint32_t>(), v.sorted_inst, v.sorted_tile, v.d_desc(), v.V, v.Ts,
                                      v.iowner.as<uint32_t>(),
-                                     v.rec0.as<float4>(), v.rec1.as<float4>(), v.rec2.as<float4>(),
-                                     v.rec3.as<float4>(), v.srec0.as<float4>(), v.srec1.as<float4>(),
+                                     v.rec.as<float4>(), v.srec0.as<float4>(), v.srec1.as<float4>(),
                                      v.srec2.as<float4>(), v.srec3.as<float4>(), v.sgid.as<uint32_t>());
     count_launches(1);
     GL_CUDA_TRY(cudaGetLastError());
