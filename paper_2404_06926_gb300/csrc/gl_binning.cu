@@ -68,17 +68,32 @@ __device__ __forceinline__ T block_sum(T x, T* sm)
 // ---------------------------------------------------------------------------
 // K1: projection, colour and tile rectangle of every Gaussian.
 // ---------------------------------------------------------------------------
+// What the first kernel of a step clears for the later ones (a memset of
+// each costs a launch and a gap of 2-5 us between graph nodes).
+struct PreClear {
+    uint32_t* ranges;    // nranges words: the tile lists
+    int64_t nranges;
+    uint32_t* sctl;      // 2 x kSortCountWords: both sorts' counts
+    float4* g2d;         // gradient rows of the visible pairs; nullptr: not wanted
+};
+
 template <int DEG>
 __global__ void __launch_bounds__(kPreThreads)
 k_preprocess(GParams p, const ViewDesc* __restrict__ views, int64_t total, int Ts, bool cull,
              float4* __restrict__ rec, int* __restrict__ radius, uint4* __restrict__ brec,
-             uint32_t* __restrict__ touched, uint32_t* __restrict__ dkey, uint64_t* __restrict__ ctl)
+             uint32_t* __restrict__ touched, uint32_t* __restrict__ dkey, uint64_t* __restrict__ ctl, PreClear clr)
 {
     // t indexes (view, Gaussian) pairs: t = view * n + g
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t == 0) {
         ctl[2] = (uint64_t)total;   // keys of the depth sort
         ctl[3] = 0;
+        ctl[9] = 0;
+    }
+    {
+        const int64_t all = (int64_t)gridDim.x * blockDim.x;
+        for (int64_t i = t; i < clr.nranges; i += all) clr.ranges[i] = 0u;
+        for (int64_t i = t; i < 2 * kSortCountWords; i += all) clr.sctl[i] = 0u;
     }
     if (t >= total) return;
     const int vw = (int)(t / p.n);
@@ -156,6 +171,11 @@ k_preprocess(GParams p, const ViewDesc* __restrict__ views, int64_t total, int T
     touched[t] = kept_tiles(D, Ts, cull, &km);
     dkey[t] = __float_as_uint(D.z);
     brec[t] = pack_bin(D, km);
+    if (clr.g2d) {
+        static_assert(kGradStride == 12, "three float4 a row");
+#pragma unroll
+        for (int k = 0; k < 3; k++) clr.g2d[3 * t + k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 }
 
 __global__ void k_set_u64(uint64_t* p, uint64_t v0, uint64_t v1)
@@ -179,8 +199,8 @@ __global__ void k_set_u64(uint64_t* p, uint64_t v0, uint64_t v1)
 // digit is the same for every key (one non-empty histogram bin, seen on the
 // device) copies its tiles through instead.
 //
-// Scratch (u32 words): global digit counts [pass][256] | tile counters
-// [pass] | look-back words [pass][tiles][256], each (flag << 30 | count):
+// Counts (u32 words): global digit counts [pass][256] | tile counters [pass].
+// Scratch: look-back words [pass][tiles][256], each (flag << 30 | count):
 // flag 1 = this tile's count, flag 2 = inclusive count of tiles 0..t.
 // A CTA only waits for tiles taken before its own, by CTAs already running,
 // so the waits end; they are still bounded (kOsSpin polls), after which the
@@ -192,7 +212,7 @@ constexpr int kOsItems = 15;
 constexpr int kOsTile = kOsThreads * kOsItems;   // 3840 keys per tile
 constexpr int kOsMaxPasses = 4;
 constexpr int kOsTicketOff = kOsMaxPasses * 256;
-constexpr int kOsStatusOff = kOsTicketOff + 64;
+static_assert(kOsTicketOff + 64 == kSortCountWords, "layout of the counts");
 constexpr uint32_t kOsAgg = 1u << 30, kOsIncl = 2u << 30, kOsValMask = kOsAgg - 1u;
 constexpr int kOsSpin = 1 << 20;   // polls of a tile not yet published before giving up
 constexpr int kOsWindow = 16;      // earlier tiles read per look-back round trip
@@ -209,7 +229,7 @@ __device__ __forceinline__ void st_relaxed_gpu(uint32_t* p, uint32_t v)
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Digit counts of all passes (scratch counts and counters zeroed before) and
+// Digit counts of all passes (counts and counters zeroed before) and
 // clearing of the look-back words of the tiles (tile_keys keys each) this
 // sort visits.  A thread loads kOsHistKeys keys before counting any of them.
 // With n_kept (zeroed before), keys 0xffffffff are left out of the counts and
@@ -219,7 +239,8 @@ __device__ __forceinline__ void st_relaxed_gpu(uint32_t* p, uint32_t v)
 constexpr int kOsHistKeys = 16;
 __global__ void __launch_bounds__(kOsThreads)
 k_os_hist(const uint32_t* __restrict__ kin, const uint64_t* n_dev, int passes, int tile_keys,
-          int64_t tiles_max, uint32_t* __restrict__ scratch, unsigned long long* __restrict__ n_kept)
+          int64_t tiles_max, uint32_t* __restrict__ counts, uint32_t* __restrict__ status,
+          unsigned long long* __restrict__ n_kept)
 {
     __shared__ uint32_t h[kOsMaxPasses * 256];
     __shared__ unsigned long long s_kept;
@@ -232,7 +253,6 @@ k_os_hist(const uint32_t* __restrict__ kin, const uint64_t* n_dev, int passes, i
     const uint64_t nt = (n + tile_keys - 1) / tile_keys;
     const uint64_t gsz = (uint64_t)gridDim.x * kOsThreads;
     const uint64_t gid = (uint64_t)blockIdx.x * kOsThreads + threadIdx.x;
-    uint32_t* status = scratch + kOsStatusOff;
     for (int p = 0; p < passes; p++)
         for (uint64_t i = gid; i < nt * 256; i += gsz) status[(uint64_t)p * tiles_max * 256 + i] = 0u;
     __syncthreads();
@@ -272,7 +292,7 @@ k_os_hist(const uint32_t* __restrict__ kin, const uint64_t* n_dev, int passes, i
     }
     __syncthreads();
     for (int i = threadIdx.x; i < passes * 256; i += kOsThreads)
-        if (h[i]) atomicAdd(&scratch[i], h[i]);
+        if (h[i]) atomicAdd(&counts[i], h[i]);
     if (drop && threadIdx.x == 0 && s_kept) atomicAdd(n_kept, s_kept);
 }
 
@@ -287,7 +307,8 @@ template <int NT, int ITEMS, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
 k_os_pass(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
           uint32_t* __restrict__ vout, const uint64_t* n_dev, int pass, int64_t tiles_max,
-          uint32_t* __restrict__ scratch, unsigned long long* __restrict__ err, bool drop)
+          uint32_t* __restrict__ counts, uint32_t* __restrict__ lookback, unsigned long long* __restrict__ err,
+          bool drop)
 {
     static_assert(NT >= 256 && NT % 32 == 0, "a thread per digit");
     constexpr int TILE = NT * ITEMS;
@@ -305,14 +326,14 @@ k_os_pass(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, ui
     const int shift = 8 * pass;
     const uint64_t n = *n_dev;
     const uint64_t nt = (n + TILE - 1) / TILE;
-    if (tid == 0) s_tile = atomicAdd(&scratch[kOsTicketOff + pass], 1u);
+    if (tid == 0) s_tile = atomicAdd(&counts[kOsTicketOff + pass], 1u);
     for (int d = lane; d < 256; d += 32) {
         wcnt[w][d] = 0u;
         wmask[w][d] = 0u;
     }
     // global digit offsets (while the tile counter answers)
     uint32_t tot;
-    const uint32_t dcount = owner ? scratch[pass * 256 + tid] : 0u;
+    const uint32_t dcount = owner ? counts[pass * 256 + tid] : 0u;
     const uint32_t gex = block_exclusive_scan<uint32_t, NT>(dcount, sm, &tot);
     // one digit holds every key: the stable pass keeps the order, so the
     // tile is copied through (no ranking, no look-back)
@@ -364,7 +385,7 @@ k_os_pass(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, ui
 
     // per digit: offsets of the warps, the tile's count, published at once
     uint32_t cnt = 0;
-    uint32_t* status = scratch + kOsStatusOff + (uint64_t)pass * tiles_max * 256;
+    uint32_t* status = lookback + (uint64_t)pass * tiles_max * 256;
     uint32_t* mine = status + (uint64_t)t * 256 + tid;
     if (owner) {
 #pragma unroll 8
@@ -652,7 +673,8 @@ constexpr int kOrderSmemTiles = 24576;   // 192 KB of shared memory
 template <bool SMEM>
 __global__ void __launch_bounds__(1024) k_order_items(const uint32_t* __restrict__ ranges, int ntiles, int seg,
                                                       uint32_t* __restrict__ order, uint2* __restrict__ items,
-                                                      uint32_t* __restrict__ heads, uint64_t* __restrict__ count)
+                                                      uint32_t* __restrict__ heads, int* __restrict__ work,
+                                                      uint64_t* __restrict__ count)
 {
     extern __shared__ uint32_t dyn[];   // SMEM: list length [ntiles] | order [ntiles]
     __shared__ uint32_t cnt[33], off[33];
@@ -663,6 +685,7 @@ __global__ void __launch_bounds__(1024) k_order_items(const uint32_t* __restrict
     const uint2* r2 = reinterpret_cast<const uint2*>(ranges);
     if (threadIdx.x < 33) cnt[threadIdx.x] = 0;
     if (threadIdx.x == 0) seg_end = split_end = 0;
+    if (threadIdx.x < 8) work[threadIdx.x] = 0;   // the raster kernels' unit counters
     __syncthreads();
     // bucket b = clz(length): 0 for the longest lists, 32 for empty ones
     constexpr int U = 4;   // lengths loaded before any is counted
@@ -838,16 +861,18 @@ gl_status build_items(View& v, cudaStream_t s)
     GL_TRY(v.items.reserve(sizeof(uint2) * (size_t)std::max<int64_t>(work_items_bound(v), 1)));
     GL_TRY(v.tile_order.reserve(4 * (size_t)std::max(v.ntiles, 1)));
     GL_TRY(v.heads.reserve(4 * (size_t)std::max(v.ntiles, 1)));
+    GL_TRY(v.work.reserve(8 * sizeof(int)));
+    v.work_clean = true;
     if (v.ntiles <= kOrderSmemTiles) {
         const int bytes = 8 * std::max(v.ntiles, 1);
         GL_TRY(ensure_smem_limit(reinterpret_cast<const void*>(&k_order_items<true>), bytes));
         k_order_items<true><<<1, 1024, bytes, s>>>(v.ranges.as<uint32_t>(), v.ntiles, v.seg,
                                                    v.tile_order.as<uint32_t>(), v.items.as<uint2>(),
-                                                   v.heads.as<uint32_t>(), v.count.as<uint64_t>());
+                                                   v.heads.as<uint32_t>(), v.work.as<int>(), v.count.as<uint64_t>());
     } else {
         k_order_items<false><<<1, 1024, 0, s>>>(v.ranges.as<uint32_t>(), v.ntiles, v.seg,
                                                 v.tile_order.as<uint32_t>(), v.items.as<uint2>(),
-                                                v.heads.as<uint32_t>(), v.count.as<uint64_t>());
+                                                v.heads.as<uint32_t>(), v.work.as<int>(), v.count.as<uint64_t>());
     }
     count_launches(1);
     GL_CUDA_TRY(cudaGetLastError());
@@ -855,8 +880,8 @@ gl_status build_items(View& v, cudaStream_t s)
 }
 
 gl_status radix_sort_u32(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
-                         const uint64_t* n_dev, int64_t n_max, int64_t n_reserve, int bits, DevBuf& scratch,
-                         uint64_t* ctl, uint32_t** out_k, uint32_t** out_v, cudaStream_t s, bool index_values,
+                         const uint64_t* n_dev, int64_t n_max, int64_t n_reserve, int bits, uint32_t* counts,
+                         DevBuf& scratch, uint64_t* ctl, uint32_t** out_k, uint32_t** out_v, cudaStream_t s, bool index_values,
                          uint64_t* n_kept)
 {
     const int passes = std::max(1, std::min(kOsMaxPasses, (bits + 7) / 8));
@@ -868,16 +893,14 @@ gl_status radix_sort_u32(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
         return GL_ERR_CAPACITY;
     }
     const int64_t tiles_max = (nbig + kOsTile - 1) / kOsTile;
-    GL_TRY(scratch.reserve(sizeof(uint32_t) * ((size_t)kOsStatusOff + (size_t)kOsMaxPasses * tiles_max * 256)));
+    GL_TRY(scratch.reserve(sizeof(uint32_t) * (size_t)kOsMaxPasses * tiles_max * 256));
     uint32_t* sc = scratch.as<uint32_t>();
-    GL_CUDA_TRY(cudaMemsetAsync(sc, 0, sizeof(uint32_t) * kOsStatusOff, s));
     const int tile_keys = kOsTile;
     const int64_t tiles = std::max<int64_t>(1, (n_max + tile_keys - 1) / tile_keys);
     const int hblocks = (int)std::min<int64_t>(
         4 * (int64_t)sm_count(), std::max<int64_t>(1, (n_max + kOsThreads * kOsHistKeys - 1) / (kOsThreads * kOsHistKeys)));
     unsigned long long* kept = reinterpret_cast<unsigned long long*>(n_kept);
-    if (kept) GL_CUDA_TRY(cudaMemsetAsync(kept, 0, sizeof(uint64_t), s));
-    k_os_hist<<<hblocks, kOsThreads, 0, s>>>(k0, n_dev, passes, tile_keys, tiles_max, sc, kept);
+    k_os_hist<<<hblocks, kOsThreads, 0, s>>>(k0, n_dev, passes, tile_keys, tiles_max, counts, sc, kept);
     uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
     unsigned long long* err = reinterpret_cast<unsigned long long*>(ctl + 8);
     for (int p = 0; p < passes; p++) {
@@ -885,7 +908,7 @@ gl_status radix_sort_u32(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
         // the first pass drops the 0xffffffff keys; the later ones sort the rest
         const uint64_t* np = (p > 0 && n_kept) ? n_kept : n_dev;
         k_os_pass<kOsThreads, kOsItems, 3><<<(unsigned)tiles, kOsThreads, 0, s>>>(ki, vsrc, ko, vo, np, p,
-                                                                                  tiles_max, sc, err,
+                                                                                  tiles_max, counts, sc, err,
                                                                                   p == 0 && n_kept);
         std::swap(ki, ko);
         std::swap(vi, vo);
@@ -903,7 +926,7 @@ gl_status sort_wait_selftest(int32_t* expired)
     // tile 1 and looks back at tile 0, whose look-back words stay zero
     const uint64_t n = 2 * (uint64_t)kOsTile;
     const int64_t tiles_max = 2;
-    const size_t words = (size_t)kOsStatusOff + (size_t)tiles_max * 256;
+    const size_t words = (size_t)kSortCountWords + (size_t)tiles_max * 256;   // counts, then look-back words
     struct Bufs {
         DevBuf keys, vals, kout, vout, scratch, ctl;
         ~Bufs()
@@ -928,6 +951,7 @@ gl_status sort_wait_selftest(int32_t* expired)
     GL_CUDA_TRY(cudaMemcpy(scratch.as<uint32_t>() + kOsTicketOff, &one, sizeof(one), cudaMemcpyHostToDevice));
     k_os_pass<kOsThreads, kOsItems, 3><<<1, kOsThreads>>>(keys.as<uint32_t>(), vals.as<uint32_t>(), kout.as<uint32_t>(),
                                                          vout.as<uint32_t>(), c, 0, tiles_max, scratch.as<uint32_t>(),
+                                                         scratch.as<uint32_t>() + kSortCountWords,
                                                          reinterpret_cast<unsigned long long*>(c + 8), false);
     count_launches(1);
     GL_CUDA_TRY(cudaGetLastError());
@@ -1044,7 +1068,7 @@ void View::set_views(const Cam* cams, const ViewExtra* extra, int nv, int ts)
 }
 
 gl_status bin_views(View& v, const GParams& p, const Cam* cams, const ViewExtra* extra, int V, int Ts,
-                    cudaStream_t s, bool sync_free)
+                    cudaStream_t s, bool sync_free, bool grad)
 {
     if (V < 1 || V > kMaxViews) { set_error("1..64 views per step"); return GL_ERR_INVALID; }
     v.n = p.n;
@@ -1071,11 +1095,15 @@ gl_status bin_views(View& v, const GParams& p, const Cam* cams, const ViewExtra*
     const int nb = (int)((n + kScanBlock - 1) / kScanBlock);
     GL_TRY(v.bsum.reserve(16 * (size_t)std::max(nb, 1)));   // block offsets, then their duplication parts
     GL_TRY(v.ranges.reserve(8 * (size_t)v.ntiles));
-    GL_CUDA_TRY(cudaMemsetAsync(v.ranges.p, 0, 8 * (size_t)v.ntiles, s));
+    GL_TRY(v.sctl.reserve(sizeof(uint32_t) * 2 * kSortCountWords));
+    // (a deterministic backward writes every row)
+    v.g2d_clean = grad && !v.det;
+    if (v.g2d_clean) GL_TRY(v.g2d.reserve(sizeof(float) * kGradStride * nn));
 
     uint64_t* count = v.count.as<uint64_t>();
     if (n == 0) {
         v.I = 0;
+        GL_CUDA_TRY(cudaMemsetAsync(v.ranges.p, 0, 8 * (size_t)v.ntiles, s));
         k_set_u64<<<1, 1, 0, s>>>(count, 0, 0);
         count_launches(1);
         GL_CUDA_TRY(cudaGetLastError());
@@ -1085,11 +1113,13 @@ gl_status bin_views(View& v, const GParams& p, const Cam* cams, const ViewExtra*
     {
     PhaseScope ps(v.prof, PH_PREPROCESS, s);
     count_launches(1);
+    const PreClear clr{v.ranges.as<uint32_t>(), 2 * (int64_t)v.ntiles, v.sctl.as<uint32_t>(),
+                       v.g2d_clean ? v.g2d.as<float4>() : nullptr};
     switch (p.deg) {
-        case 0: k_preprocess<0><<<grid, kPreThreads, 0, s>>>(p, dv, n, Ts, v.cull, v.rec.as<float4>(), v.radius.as<int>(), v.brec.as<uint4>(), v.touched.as<uint32_t>(), v.dkey.as<uint32_t>(), count); break;
-        case 1: k_preprocess<1><<<grid, kPreThreads, 0, s>>>(p, dv, n, Ts, v.cull, v.rec.as<float4>(), v.radius.as<int>(), v.brec.as<uint4>(), v.touched.as<uint32_t>(), v.dkey.as<uint32_t>(), count); break;
-        case 2: k_preprocess<2><<<grid, kPreThreads, 0, s>>>(p, dv, n, Ts, v.cull, v.rec.as<float4>(), v.radius.as<int>(), v.brec.as<uint4>(), v.touched.as<uint32_t>(), v.dkey.as<uint32_t>(), count); break;
-        case 3: k_preprocess<3><<<grid, kPreThreads, 0, s>>>(p, dv, n, Ts, v.cull, v.rec.as<float4>(), v.radius.as<int>(), v.brec.as<uint4>(), v.touched.as<uint32_t>(), v.dkey.as<uint32_t>(), count); break;
+        case 0: k_preprocess<0><<<grid, kPreThreads, 0, s>>>(p, dv, n, Ts, v.cull, v.rec.as<float4>(), v.radius.as<int>(), v.brec.as<uint4>(), v.touched.as<uint32_t>(), v.dkey.as<uint32_t>(), count, clr); break;
+        case 1: k_preprocess<1><<<grid, kPreThreads, 0, s>>>(p, dv, n, Ts, v.cull, v.rec.as<float4>(), v.radius.as<int>(), v.brec.as<uint4>(), v.touched.as<uint32_t>(), v.dkey.as<uint32_t>(), count, clr); break;
+        case 2: k_preprocess<2><<<grid, kPreThreads, 0, s>>>(p, dv, n, Ts, v.cull, v.rec.as<float4>(), v.radius.as<int>(), v.brec.as<uint4>(), v.touched.as<uint32_t>(), v.dkey.as<uint32_t>(), count, clr); break;
+        case 3: k_preprocess<3><<<grid, kPreThreads, 0, s>>>(p, dv, n, Ts, v.cull, v.rec.as<float4>(), v.radius.as<int>(), v.brec.as<uint4>(), v.touched.as<uint32_t>(), v.dkey.as<uint32_t>(), count, clr); break;
         default: set_error("sh_degree must be 0..3"); return GL_ERR_INVALID;
     }
     GL_CUDA_TRY(cudaGetLastError());
@@ -1101,7 +1131,7 @@ gl_status bin_views(View& v, const GParams& p, const Cam* cams, const ViewExtra*
     {
         PhaseScope ps(v.prof, PH_DEPTH_SORT, s);
         GL_TRY(radix_sort_u32(v.dkey.as<uint32_t>(), v.gidx.as<uint32_t>(), v.dkey2.as<uint32_t>(),
-                              v.gidx2.as<uint32_t>(), count + 2, n, n, 32, v.hist, count, &sk, &sv, s,
+                              v.gidx2.as<uint32_t>(), count + 2, n, n, 32, v.sctl.as<uint32_t>(), v.hist, count, &sk, &sv, s,
                               true, count + 9));
     }
     v.sorted_g = sv;
@@ -1167,8 +1197,8 @@ gl_status bin_views(View& v, const GParams& p, const Cam* cams, const ViewExtra*
     {
         PhaseScope ps(v.prof, PH_TILE_SORT, s);
         GL_TRY(radix_sort_u32(v.itile.as<uint32_t>(), v.ival.as<uint32_t>(), v.itile2.as<uint32_t>(),
-                              v.ival2.as<uint32_t>(), count, nmax, (int64_t)cap2, tbits, v.hist, count, &sk, &sv,
-                              s, true));
+                              v.ival2.as<uint32_t>(), count, nmax, (int64_t)cap2, tbits, v.sctl.as<uint32_t>() + kSortCountWords,
+                              v.hist, count, &sk, &sv, s, true));
     }
     v.sorted_tile = sk;
     v.sorted_inst = sv;

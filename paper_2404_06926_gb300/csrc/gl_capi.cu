@@ -234,7 +234,7 @@ void View::release()
 {
     DevBuf* all[] = {&rec, &radius, &brec, &touched, &dkey, &gidx, &dkey2, &gidx2,
                      &dup_off, &bsum, &count, &itile, &ival, &itile2, &ival2, &iowner, &srec0, &srec1, &srec2, &srec3, &sgid, &g2d, &gpart, &gmask, &work, &items, &heads, &segstate,
-                     &hist, &ranges, &tile_order, &Tfin, &ncon, &rgb, &depth, &opac};
+                     &hist, &sctl, &ranges, &tile_order, &Tfin, &ncon, &rgb, &depth, &opac};
     for (DevBuf* b : all) b->release();
     desc.release();
     if (h_count) cudaFreeHost(h_count);
@@ -1101,7 +1101,7 @@ gl_status enqueue_step(gl_map* m, const StepPlan& sp, cudaStream_t s, bool sync_
     View& v = m->ctx.view;
     const int V = sp.V;
     GL_TRY(v.rgb.reserve(12 * (size_t)sp.P));
-    GL_TRY(bin_views(v, m->params(), sp.cams, sp.extra, V, step_tile(m), s, sync_free));
+    GL_TRY(bin_views(v, m->params(), sp.cams, sp.extra, V, step_tile(m), s, sync_free, true));
     GL_TRY(raster_forward(v, v.rgb.as<float>(), nullptr, nullptr, s, false));
     GL_TRY(m->dLdC.reserve(12 * (size_t)sp.P));
     GL_TRY(m->ctx.loss_part.reserve(sizeof(float) * 14 * (size_t)v.nltiles));
@@ -1171,7 +1171,7 @@ std::vector<int64_t> graph_key(const gl_map* m, const StepPlan& sp)
     const DevBuf* bufs[] = {&v.rec, &v.radius, &v.brec, &v.touched, &v.dkey,
                             &v.gidx, &v.dkey2, &v.gidx2, &v.dup_off, &v.g2d, &v.bsum, &v.count, &v.itile,
                             &v.ival, &v.itile2, &v.ival2, &v.iowner, &v.srec0, &v.srec1, &v.srec2, &v.srec3,
-                            &v.sgid, &v.hist, &v.ranges, &v.tile_order, &v.Tfin, &v.ncon, &v.rgb, &v.work, &v.gpart, &v.gmask,
+                            &v.sgid, &v.hist, &v.sctl, &v.ranges, &v.tile_order, &v.Tfin, &v.ncon, &v.rgb, &v.work, &v.gpart, &v.gmask,
                             &v.items, &v.heads, &v.segstate,
                             &v.desc, &m->dLdC, &m->ctx.loss_part, &m->loss_dev};
     for (const DevBuf* b : bufs) {

@@ -168,7 +168,8 @@ struct View {
     DevBuf iowner;            // u32 owning (view, Gaussian) per instance id
     DevBuf srec0, srec1, srec2, srec3;  // records in sorted-instance order
     DevBuf sgid;              // u32 owning (view, Gaussian) per sorted instance
-    DevBuf hist;              // radix histograms
+    DevBuf hist;              // radix look-back words
+    DevBuf sctl;              // radix digit counts and tile counters: depth sort, tile sort
     DevBuf ranges;            // uint2 per global tile
     DevBuf tile_order;        // u32 tile launch order (heaviest first)
     // per pixel (concatenated over views)
@@ -184,7 +185,10 @@ struct View {
     // lane (1, 2, 4), persistent grid with a unit counter in `work`
     int nb = 1, pd = 1;
     bool persistent = false;
-    DevBuf work;              // int[2] unit counters (forward, backward)
+    DevBuf work;              // int[8] unit counters (0, 1 forward, 2 backward)
+    // what the binning left cleared for the next backward: its unit counter,
+    // and (bin_views with `grad`) the rows of g2d of the visible pairs
+    bool work_clean = false, g2d_clean = false;
     // deterministic backward: per (instance, pixel block) sums, reduced per
     // (view, Gaussian) in a fixed order (floats: instances x blocks x kGradStride)
     bool det = false;
@@ -237,12 +241,13 @@ struct gl_ctx_impl {
 // capacity set the overflow flag (count[1]), every later kernel of the step
 // sees zero instances, and the Adam updates skip themselves; the caller
 // checks the flag after the step.  Used for steps captured in a CUDA graph.
+// grad: a backward follows, the rows of g2d are cleared along the way.
 gl_status bin_views(View& v, const GParams& p, const Cam* cams, const ViewExtra* extra, int V, int Ts,
-                    cudaStream_t s, bool sync_free = false);
+                    cudaStream_t s, bool sync_free = false, bool grad = false);
 // The single-view case.
 gl_status bin_view(View& v, const GParams& p, const Cam& cam, int Ts, cudaStream_t s);
 
-// Forward raster of a binned view into (rgb, depth, opacity) device images
+// Forward raster of a binned view (once per binning) into (rgb, depth, opacity) device images
 // (depth/opacity may be null) plus T_final / n_contrib in `v`.
 // extras: also blend depth and opacity (needed for those outputs and for a
 // later backward with depth or opacity gradients on split tiles).
@@ -301,16 +306,19 @@ gl_status photometric_loss_views(const View& v, const float* rgb, float lambda, 
 gl_status apply_exposure(const float* src, float* dst, const float E[12], int64_t P,
                          cudaStream_t s);
 
+// Words of digit counts and tile counters of one radix sort.
+constexpr int kSortCountWords = 4 * 256 + 64;
+
 // Stable radix sort of (u32 key, u32 value) pairs over bits [0, bits); n on
-// the device, at most n_max; scratch sized for max(n_max, n_reserve) keys;
-// ctl[8] is raised if a look-back wait gave up.  Returns in *out_k/*out_v the
+// the device, at most n_max; `counts` holds kSortCountWords zeros; scratch
+// sized for max(n_max, n_reserve) keys; ctl[8] is raised if a look-back wait gave up.  Returns in *out_k/*out_v the
 // buffers holding the result.  index_values: the input values are 0..n-1 and
 // v0 is not read (it still serves as an output buffer).  n_kept (device, may
 // be null): keys 0xffffffff are dropped from the result, whose length is
-// written to *n_kept.
+// added to *n_kept (zero before).
 gl_status radix_sort_u32(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
-                         const uint64_t* n_dev, int64_t n_max, int64_t n_reserve, int bits, DevBuf& scratch,
-                         uint64_t* ctl, uint32_t** out_k, uint32_t** out_v, cudaStream_t s,
+                         const uint64_t* n_dev, int64_t n_max, int64_t n_reserve, int bits, uint32_t* counts,
+                         DevBuf& scratch, uint64_t* ctl, uint32_t** out_k, uint32_t** out_v, cudaStream_t s,
                          bool index_values = false, uint64_t* n_kept = nullptr);
 // Bytes of the counters copied to View::h_count (count[0..8]).
 constexpr size_t kCountCopy = 9 * sizeof(uint64_t);

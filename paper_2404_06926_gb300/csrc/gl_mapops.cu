@@ -288,10 +288,10 @@ gl_status sky_create(float* means, float* log_scales, float* quats, float* logit
     G.nx = (int)std::min(1024.0, std::floor(2.0 * radius / (double)G.c) + 1.0);
     G.nz = (int)std::min(1024.0, std::floor(radius / (double)G.c) + 1.0);
     struct Tmp {
-        DevBuf keys, vals, keys2, vals2, scratch, ctl;
+        DevBuf keys, vals, keys2, vals2, counts, scratch, ctl;
         ~Tmp()
         {
-            for (DevBuf* b : {&keys, &vals, &keys2, &vals2, &scratch, &ctl}) b->release();
+            for (DevBuf* b : {&keys, &vals, &keys2, &vals2, &counts, &scratch, &ctl}) b->release();
         }
     } T;
     const size_t nn = (size_t)n;
@@ -300,13 +300,15 @@ gl_status sky_create(float* means, float* log_scales, float* quats, float* logit
     GL_TRY(T.keys2.reserve(4 * nn));
     GL_TRY(T.vals2.reserve(4 * nn));
     GL_TRY(T.ctl.reserve(16 * sizeof(uint64_t)));
+    GL_TRY(T.counts.reserve(sizeof(uint32_t) * kSortCountWords));
+    GL_CUDA_TRY(cudaMemsetAsync(T.counts.p, 0, sizeof(uint32_t) * kSortCountWords, s));
     uint64_t* ctl = T.ctl.as<uint64_t>();
     k_sky_cells<<<grid, kThreads, 0, s>>>(means, n, G, T.keys.as<uint32_t>(), T.vals.as<uint32_t>(), ctl);
     count_launches(2);
     GL_CUDA_TRY(cudaGetLastError());
     uint32_t *sk, *sv;
     GL_TRY(radix_sort_u32(T.keys.as<uint32_t>(), T.vals.as<uint32_t>(), T.keys2.as<uint32_t>(),
-                          T.vals2.as<uint32_t>(), ctl, n, n, 30, T.scratch, ctl, &sk, &sv, s));
+                          T.vals2.as<uint32_t>(), ctl, n, n, 30, T.counts.as<uint32_t>(), T.scratch, ctl, &sk, &sv, s));
     const float logit = logf(opacity / (1.0f - opacity));
     k_sky_nn<<<grid, kThreads, 0, s>>>(means, n, G, sk, sv, log_scales, quats, logits, sh, K, logit);
     count_launches(1);

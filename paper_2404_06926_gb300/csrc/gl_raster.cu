@@ -1596,15 +1596,10 @@ gl_status raster_forward(View& v, float* rgb, float* depth, float* opac, cudaStr
     GL_TRY(v.ncon.reserve(4 * P));
     if (v.ntiles == 0) return GL_OK;
     GL_TRY(check_exec(v));
-    GL_TRY(v.work.reserve(32));
     const int64_t split = split_items_bound(v);
     if (split > 0) GL_TRY(v.segstate.reserve(sizeof(float) * kSegFields * (size_t)(v.Ts * v.Ts) * (size_t)split));
     PhaseScope ps(v.prof, PH_RASTER_FWD, s);
-    int* work = nullptr;
-    if (v.persistent) {
-        work = v.work.as<int>();
-        GL_CUDA_TRY(cudaMemsetAsync(work, 0, 8 * sizeof(int), s));
-    }
+    int* work = v.persistent ? v.work.as<int>() : nullptr;   // cleared with the items
     const RasterArgs A = make_args(v, work);
     RasterOut O{rgb, depth, opac, v.Tfin.as<float>(), v.ncon.as<uint32_t>()};
     const int nblk = blocks_per_tile(v);
@@ -1624,19 +1619,20 @@ gl_status raster_backward(View& v, const float* dL_drgb, const float* dL_ddepth,
     const size_t pairs = (size_t)v.n * v.V;
     GL_TRY(v.g2d.reserve(sizeof(float) * kGradStride * std::max<size_t>(pairs, 1)));
     GL_TRY(check_exec(v));
-    GL_TRY(v.work.reserve(32));
     PhaseScope ps(v.prof, PH_RASTER_BWD, s);
     const bool det = v.det && v.ntiles > 0 && v.I != 0;
     // the per-Gaussian backward works on 8x4 pixel blocks whatever the
     // forward's pixels per lane
     const int nblk = v.pg ? v.Ts * v.Ts / 32 : blocks_per_tile(v);
-    if (!det) GL_CUDA_TRY(cudaMemsetAsync(v.g2d.p, 0, sizeof(float) * kGradStride * pairs, s));
+    if (!det && !v.g2d_clean) GL_CUDA_TRY(cudaMemsetAsync(v.g2d.p, 0, sizeof(float) * kGradStride * pairs, s));
+    v.g2d_clean = false;   // a second backward of the same binning starts over
     if (v.ntiles == 0 || v.I == 0) return GL_OK;
     int* work = nullptr;
     if (v.persistent) {
-        work = v.work.as<int>() + 1;
-        GL_CUDA_TRY(cudaMemsetAsync(work, 0, sizeof(int), s));
+        work = v.work.as<int>() + 2;
+        if (!v.work_clean) GL_CUDA_TRY(cudaMemsetAsync(work, 0, sizeof(int), s));
     }
+    v.work_clean = false;
     RasterArgs A = make_args(v, work);
     A.nblk = nblk;
     RasterGrad G{v.Tfin.as<float>(), v.ncon.as<uint32_t>(), dL_drgb, dL_ddepth, dL_dopac, v.g2d.as<float>(),
