@@ -396,6 +396,20 @@ bool is_device_ptr(const void* p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// A float array that a kernel on the current device can read and write.
+bool is_local_array(const void* p)
+{
+    cudaPointerAttributes a;
+    int dev = -1;
+    if (!p || ((uintptr_t)p & 3) || cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev);
+}
+
+bool overlap(const float* a, size_t na, const float* b, size_t nb) { return a && b && a < b + nb && b < a + na; }
+
 gl_status check_tile(int t)
 {
     if (t != 8 && t != 16 && t != 32) { set_error("tile_size must be 8, 16 or 32"); return GL_ERR_INVALID; }
@@ -756,18 +770,33 @@ gl_status map_reserve(gl_map* m, int64_t need)
 gl_status zero_moments(gl_map* m, int64_t from, int64_t count)
 {
     if (count <= 0) return GL_OK;
+    ArrayMove mv[2 * NPARAM];
     for (int w = 0; w < NPARAM; w++) {
-        const size_t rb = 4 * m->row_floats(w);
-        GL_CUDA_TRY(cudaMemsetAsync(static_cast<char*>(m->mom1[w].p) + rb * from, 0, rb * count, m->stream));
-        GL_CUDA_TRY(cudaMemsetAsync(static_cast<char*>(m->mom2[w].p) + rb * from, 0, rb * count, m->stream));
+        const size_t row = m->row_floats(w);
+        mv[2 * w] = {m->mom1[w].as<float>() + row * from, nullptr, row * count};
+        mv[2 * w + 1] = {m->mom2[w].as<float>() + row * from, nullptr, row * count};
     }
-    return GL_OK;
+    return move_arrays(mv, 2 * NPARAM, m->stream);
 }
 
 gl_status from_device(float* dst, const float* src, size_t count, cudaStream_t s)
 {
     GL_CUDA_TRY(cudaMemcpyAsync(dst, src, 4 * count, is_device_ptr(dst) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     return GL_OK;
+}
+
+// The live rows of five map arrays into the caller's arrays (null: skipped).
+gl_status copy_rows_out(gl_map* m, DevBuf* src, float* const dst[NPARAM])
+{
+    ArrayMove mv[NPARAM];
+    int k = 0;
+    for (int w = 0; w < NPARAM; w++) {
+        if (!dst[w] || m->n == 0) continue;
+        const size_t cnt = m->row_floats(w) * (size_t)m->n;
+        if (is_local_array(dst[w])) mv[k++] = {dst[w], src[w].as<float>(), cnt};
+        else GL_TRY(from_device(dst[w], src[w].as<float>(), cnt, m->stream));
+    }
+    return move_arrays(mv, k, m->stream);
 }
 
 Keyframe* get_kf(gl_map* m, int64_t id, bool create, gl_status* st)
@@ -790,16 +819,19 @@ Keyframe* get_kf(gl_map* m, int64_t id, bool create, gl_status* st)
     return raw;
 }
 
-gl_status render_internal(gl_map* m, const Cam& cam, int Ts)
+// Render into the given device images, or the view's own where null.
+gl_status render_internal(gl_map* m, const Cam& cam, int Ts, float* rgb = nullptr, float* depth = nullptr,
+                          float* opac = nullptr)
 {
     View& v = m->ctx.view;
     const size_t P = (size_t)cam.W * cam.H;
-    GL_TRY(v.rgb.reserve(12 * P));
-    GL_TRY(v.depth.reserve(4 * P));
-    GL_TRY(v.opac.reserve(4 * P));
+    if (!rgb) GL_TRY(v.rgb.reserve(12 * P));
+    if (!depth) GL_TRY(v.depth.reserve(4 * P));
+    if (!opac) GL_TRY(v.opac.reserve(4 * P));
     map_exec_knobs(m, v, Ts);
     GL_TRY(bin_view(v, m->params(), cam, Ts, m->stream));
-    return raster_forward(v, v.rgb.as<float>(), v.depth.as<float>(), v.opac.as<float>(), m->stream);
+    return raster_forward(v, rgb ? rgb : v.rgb.as<float>(), depth ? depth : v.depth.as<float>(),
+                          opac ? opac : v.opac.as<float>(), m->stream);
 }
 
 }  // namespace
@@ -964,19 +996,33 @@ extern "C" gl_status gl_render(gl_map* m, const gl_pose* pose, const gl_intrinsi
     Cam cam;
     GL_TRY(make_cam(pose, K, cam));
     if (E34 && !finite_all(E34, 12)) { set_error("exposure contains NaN or Inf"); return GL_ERR_INVALID; }
-    GL_TRY(render_internal(m, cam, m->cfg.tile_size));
+    // images in the caller's device memory are rendered in place (the colour
+    // only without an exposure)
+    float* depth = is_local_array(out_depth) ? out_depth : nullptr;
+    float* opac = is_local_array(out_opacity) ? out_opacity : nullptr;
+    float* rgb = !E34 && is_local_array(out_rgb) ? out_rgb : nullptr;
+    {
+        const size_t px = (size_t)cam.W * cam.H;
+        if (overlap(rgb, 3 * px, depth, px) || overlap(rgb, 3 * px, opac, px) || overlap(depth, px, opac, px))
+            rgb = depth = opac = nullptr;   // copied out one after the other
+    }
+    GL_TRY(render_internal(m, cam, m->cfg.tile_size, rgb, depth, opac));
     View& v = m->ctx.view;
     const size_t P = (size_t)cam.W * cam.H;
     const float ident[12] = {1, 0, 0, 0, 0, 1, 0, 0, 0, 0, 1, 0};
-    if (is_device_ptr(out_rgb)) {
+    if (!rgb && is_device_ptr(out_rgb)) {
         GL_TRY(apply_exposure(v.rgb.as<float>(), out_rgb, E34 ? E34 : ident, (int64_t)P, m->stream));
-    } else {
-        GL_TRY(m->stage_img.reserve(12 * P));
-        GL_TRY(apply_exposure(v.rgb.as<float>(), m->stage_img.as<float>(), E34 ? E34 : ident, (int64_t)P, m->stream));
-        GL_CUDA_TRY(cudaMemcpyAsync(out_rgb, m->stage_img.p, 12 * P, cudaMemcpyDeviceToHost, m->stream));
+    } else if (!rgb) {
+        const float* src = v.rgb.as<float>();
+        if (E34) {
+            GL_TRY(m->stage_img.reserve(12 * P));
+            GL_TRY(apply_exposure(src, m->stage_img.as<float>(), E34, (int64_t)P, m->stream));
+            src = m->stage_img.as<float>();
+        }
+        GL_CUDA_TRY(cudaMemcpyAsync(out_rgb, src, 12 * P, cudaMemcpyDeviceToHost, m->stream));
     }
-    if (out_depth) GL_TRY(from_device(out_depth, v.depth.as<float>(), P, m->stream));
-    if (out_opacity) GL_TRY(from_device(out_opacity, v.opac.as<float>(), P, m->stream));
+    if (out_depth && !depth) GL_TRY(from_device(out_depth, v.depth.as<float>(), P, m->stream));
+    if (out_opacity && !opac) GL_TRY(from_device(out_opacity, v.opac.as<float>(), P, m->stream));
     GL_CUDA_TRY(cudaStreamSynchronize(m->stream));
     return sort_wait_status(v, m->stream);
 }
@@ -1311,8 +1357,7 @@ extern "C" gl_status gl_map_get_params(gl_map* m, gl_gaussians* out, int64_t* n_
     if (n_out) *n_out = m->n;
     if (out->n < m->n) { set_error("output arrays too small"); return GL_ERR_INVALID; }
     float* dst[NPARAM] = {out->means, out->log_scales, out->quats, out->logits, out->sh};
-    for (int w = 0; w < NPARAM; w++)
-        if (dst[w]) GL_TRY(from_device(dst[w], m->prm[w].as<float>(), m->row_floats(w) * (size_t)m->n, m->stream));
+    GL_TRY(copy_rows_out(m, m->prm, dst));
     GL_CUDA_TRY(cudaStreamSynchronize(m->stream));
     return GL_OK;
 }
@@ -1323,8 +1368,7 @@ extern "C" gl_status gl_map_get_moments(gl_map* m, int32_t which, gl_gaussians* 
     if (out->sh_degree != m->deg || out->n < m->n) { set_error("output shape differs"); return GL_ERR_INVALID; }
     DevBuf* src = which == 1 ? m->mom1 : m->mom2;
     float* dst[NPARAM] = {out->means, out->log_scales, out->quats, out->logits, out->sh};
-    for (int w = 0; w < NPARAM; w++)
-        if (dst[w]) GL_TRY(from_device(dst[w], src[w].as<float>(), m->row_floats(w) * (size_t)m->n, m->stream));
+    GL_TRY(copy_rows_out(m, src, dst));
     GL_CUDA_TRY(cudaStreamSynchronize(m->stream));
     return GL_OK;
 }
@@ -1336,15 +1380,20 @@ extern "C" gl_status gl_map_set_params(gl_map* m, const gl_gaussians* in)
     if (in->sh_degree != m->deg) { set_error("sh_degree differs from the map"); return GL_ERR_INVALID; }
     GL_TRY(map_reserve(m, in->n));
     const float* src[NPARAM] = {in->means, in->log_scales, in->quats, in->logits, in->sh};
+    ArrayMove mv[3 * NPARAM];
+    int k = 0;
     for (int w = 0; w < NPARAM; w++) {
         const size_t cnt = m->row_floats(w) * (size_t)in->n;
-        GL_CUDA_TRY(cudaMemcpyAsync(m->prm[w].p, src[w], 4 * cnt,
-                                    is_device_ptr(src[w]) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                                    m->stream));
+        if (is_local_array(src[w])) mv[k++] = {m->prm[w].as<float>(), src[w], cnt};
+        else GL_CUDA_TRY(cudaMemcpyAsync(m->prm[w].p, src[w], 4 * cnt,
+                                         is_device_ptr(src[w]) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                                         m->stream));
+        mv[k++] = {m->mom1[w].as<float>(), nullptr, cnt};
+        mv[k++] = {m->mom2[w].as<float>(), nullptr, cnt};
     }
+    GL_TRY(move_arrays(mv, k, m->stream));
     GL_CUDA_TRY(cudaMemsetAsync(m->kind.p, 0, (size_t)in->n, m->stream));
     m->n = in->n;
-    GL_TRY(zero_moments(m, 0, m->n));
     m->step = 0;
     GL_CUDA_TRY(cudaStreamSynchronize(m->stream));
     return GL_OK;
@@ -1849,12 +1898,13 @@ int64_t map_capacity(const gl_map* m) { return m->cap; }
 
 gl_status map_snapshot(gl_map* m, DevBuf* dst, int64_t* n_out, cudaEvent_t done)
 {
+    ArrayMove mv[NPARAM];
     for (int w = 0; w < NPARAM; w++) {
-        const size_t b = 4 * m->row_floats(w) * (size_t)std::max<int64_t>(m->n, 1);
-        GL_TRY(dst[w].reserve(b));
-        if (m->n) GL_CUDA_TRY(cudaMemcpyAsync(dst[w].p, m->prm[w].p, 4 * m->row_floats(w) * (size_t)m->n,
-                                              cudaMemcpyDeviceToDevice, m->stream));
+        const size_t cnt = m->row_floats(w) * (size_t)m->n;
+        GL_TRY(dst[w].reserve(4 * m->row_floats(w) * (size_t)std::max<int64_t>(m->n, 1)));
+        mv[w] = {dst[w].as<float>(), m->prm[w].as<float>(), cnt};
     }
+    GL_TRY(move_arrays(mv, NPARAM, m->stream));
     GL_CUDA_TRY(cudaEventRecord(done, m->stream));
     *n_out = m->n;
     return GL_OK;

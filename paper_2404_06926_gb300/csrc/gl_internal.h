@@ -367,6 +367,17 @@ GParams snapshot_params(const gl_map* m, const DevBuf* src, int64_t n);
 // Registered keyframes that hold an image, by ascending id (image = null).
 void map_keyframes(const gl_map* m, std::vector<gl_keyframe>& out);
 
+// Copies (src null: zeros) of float arrays in device memory of the current
+// device, up to kMaxMoves of them in one launch; arrays need not be aligned
+// beyond a float's size, empty ones are skipped.
+struct ArrayMove {
+    float* dst;
+    const float* src;
+    size_t count;
+};
+constexpr int kMaxMoves = 16;
+gl_status move_arrays(const ArrayMove* moves, int n, cudaStream_t s);
+
 // Map-side kernels.
 gl_status sky_create(float* means, float* log_scales, float* quats, float* logits, float* sh,
                      int K, int64_t n, double radius, uint64_t seed, float opacity,

@@ -99,3 +99,51 @@ def test_split_list_lengths(n, opacity, ppl, persistent):
 @pytest.mark.parametrize("bd", [32, 64, 256])
 def test_split_segments_of_several_runs(seg, bd):
     _check_stack(2100, 0.02, False, segment=seg, batch_depth=bd)
+
+
+@pytest.mark.parametrize("n", [1, 3, 683, 2731, 5000])   # around the copy's chunk of 8192 floats
+def test_parameter_copies(n):
+    """Parameters set and read back (aligned, and rows into the middle of larger
+    arrays), and a new map's moments, are exact."""
+    from paper_2404_06926_gb300 import binding
+    rng = np.random.default_rng(n)
+    p = _dev(dict(means=rng.normal(size=(n, 3)), log_scales=rng.normal(size=(n, 3)), quats=rng.normal(size=(n, 4)),
+                  logits=rng.normal(size=n), sh=rng.normal(size=(n, 4, 3))))
+    m = binding.Map(binding.default_config(n_sky=0, sh_degree=1, capacity_hint=n))
+    m.set_params(p)
+    out = m.get_params()
+    host = {k: np.zeros(v.shape, np.float32) for k, v in p.items()}
+    gs = binding.gaussians(host)
+    binding.check(binding.lib().gl_map_get_params(m._h, binding.C.byref(gs), None))
+    odd = {k: torch.zeros(v.numel() + 1, device="cuda") for k, v in p.items()}
+    go = binding.gaussians({k: v[1:].view(p[k].shape) for k, v in odd.items()})   # 4-byte aligned only
+    binding.check(binding.lib().gl_map_get_params(m._h, binding.C.byref(go), None))
+    torch.cuda.synchronize()
+    for k in NAMES:
+        assert torch.equal(torch.as_tensor(out[k]).cpu().reshape(-1), p[k].cpu().reshape(-1)), k
+        assert np.array_equal(host[k], p[k].cpu().numpy()), k
+        assert torch.equal(odd[k][1:], p[k].reshape(-1)) and odd[k][0] == 0, k
+    for which in (1, 2):
+        assert all(float(torch.as_tensor(v).abs().max()) == 0 for v in m.get_moments(which).values())
+
+
+def test_render_into_device_images():
+    """Images rendered in place equal those copied to the host, also where two
+    of them share memory (the later copy wins)."""
+    from paper_2404_06926_gb300 import binding
+    sc = scenes.small_frustum(n=300)
+    cam = sc["cam"]
+    H, W = cam["height"], cam["width"]
+    m = binding.Map(binding.default_config(n_sky=0, sh_degree=0, capacity_hint=300))
+    m.set_params(_dev(sc["params"]))
+    hd, ho = np.empty((H, W), np.float32), np.empty((H, W), np.float32)
+    hc = m.render(cam, out_depth=hd, out_opacity=ho)
+    c, d, o = (torch.empty(s, device="cuda") for s in ((H, W, 3), (H, W), (H, W)))
+    m.render(cam, out_rgb=c, out_depth=d, out_opacity=o)
+    assert np.array_equal(c.cpu().numpy(), hc) and np.array_equal(d.cpu().numpy(), hd)
+    assert np.array_equal(o.cpu().numpy(), ho)
+    m.render(cam, out_rgb=c, out_depth=d, out_opacity=d)
+    assert np.array_equal(d.cpu().numpy(), ho)
+    E = np.concatenate([np.eye(3, dtype=np.float32), np.full((3, 1), 0.25, np.float32)], 1)
+    m.render(cam, E=E, out_rgb=c)
+    assert np.allclose(c.cpu().numpy(), hc + 0.25, atol=1e-6)
