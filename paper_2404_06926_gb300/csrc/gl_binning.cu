@@ -858,6 +858,11 @@ int64_t work_items_bound(const View& v)
 
 gl_status build_items(View& v, cudaStream_t s)
 {
+    if (v.seg_auto && v.seg > 0 && reserve_segstate(v) != GL_OK) {
+        if (alloc_frozen()) return GL_ERR_CAPACITY;
+        cudaGetLastError();
+        v.seg = 0;
+    }
     GL_TRY(v.items.reserve(sizeof(uint2) * (size_t)std::max<int64_t>(work_items_bound(v), 1)));
     GL_TRY(v.tile_order.reserve(4 * (size_t)std::max(v.ntiles, 1)));
     GL_TRY(v.heads.reserve(4 * (size_t)std::max(v.ntiles, 1)));

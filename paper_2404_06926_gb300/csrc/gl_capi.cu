@@ -562,7 +562,7 @@ extern "C" gl_status gl_rasterize_forward(gl_ctx* ctx, const gl_gaussians* g, co
     c.view.nb = batch_subs(c.exec.batch_depth, c.view.det);
     c.view.pd = std::min(c.exec.pixels_per_lane, tile_size / 4);
     c.view.persistent = c.exec.persistent != 0;
-    c.view.seg = c.exec.segment;
+    c.view.set_segment(c.exec.segment);
     c.view.cull = c.exec.exact_cull != 0;
     c.view.pg = c.exec.per_gaussian != 0;
     GL_TRY(bin_view(c.view, params_of(g), cam, tile_size, c.stream));
@@ -1134,7 +1134,7 @@ void apply_exec(gl_map* m)
     v.nb = batch_subs(m->exec.batch_depth, v.det);
     v.pd = m->exec.pixels_per_lane;
     v.persistent = m->exec.persistent != 0;
-    v.seg = m->exec.segment;
+    v.set_segment(m->exec.segment);
     v.cull = m->exec.exact_cull != 0;
     v.pg = m->exec.per_gaussian != 0;
 }
@@ -1887,7 +1887,7 @@ void map_exec_knobs(const gl_map* m, View& v, int Ts)
     v.nb = batch_subs(m->exec.batch_depth, m->exec.deterministic != 0);
     v.pd = std::min(m->exec.pixels_per_lane, Ts / 4);
     v.persistent = m->exec.persistent != 0;
-    v.seg = m->exec.segment;
+    v.set_segment(m->exec.segment);
     v.cull = m->exec.exact_cull != 0;
     v.pg = m->exec.per_gaussian != 0;
 }

@@ -196,6 +196,18 @@ struct View {
     // segmented raster: tiles whose list holds >= 2 seg records are split
     // into segments of seg records (seg a power of two; 0: never split)
     int seg = 0;
+    bool seg_auto = false;    // seg was not asked for: dropped where its state finds no memory
+    // The execution knob: 0 takes kAutoSegment.  Without segments a list is
+    // one warp's serial chain per pixel block, and the deepest tile's chain
+    // is the kernel's time; lists shorter than 2 kAutoSegment stay whole, so
+    // small scenes run as they did.  250k Gaussians at 640x480: forward 423 ->
+    // 140 us, backward 650 -> 91 us.
+    static constexpr int kAutoSegment = 512;
+    void set_segment(int knob)
+    {
+        seg_auto = knob == 0;
+        seg = seg_auto ? kAutoSegment : knob;
+    }
     // exact tile culling: only tiles where the Gaussian can reach alpha >=
     // 1/255 at a pixel centre get an instance
     bool cull = true;
@@ -256,6 +268,8 @@ gl_status raster_forward(View& v, float* rgb, float* depth, float* opac, cudaStr
 // Upper bound of the work items of a binned step (every tile once, plus one
 // per seg records of the instance capacity).
 int64_t work_items_bound(const View& v);
+// The split tiles' state for the current capacity.
+gl_status reserve_segstate(View& v);
 // Build the work items of a binned step (after the tile order).
 gl_status build_items(View& v, cudaStream_t s);
 

@@ -1585,6 +1585,11 @@ void fwd_dispatch(const View& v, const RasterArgs& A, const RasterOut& O, int64_
     }
 }
 
+gl_status reserve_segstate(View& v)
+{
+    return v.segstate.reserve(sizeof(float) * kSegFields * (size_t)(v.Ts * v.Ts) * (size_t)split_items_bound(v));
+}
+
 gl_status raster_forward(View& v, float* rgb, float* depth, float* opac, cudaStream_t s, bool extras)
 {
     if (!extras && (depth || opac)) {
@@ -1596,8 +1601,7 @@ gl_status raster_forward(View& v, float* rgb, float* depth, float* opac, cudaStr
     GL_TRY(v.ncon.reserve(4 * P));
     if (v.ntiles == 0) return GL_OK;
     GL_TRY(check_exec(v));
-    const int64_t split = split_items_bound(v);
-    if (split > 0) GL_TRY(v.segstate.reserve(sizeof(float) * kSegFields * (size_t)(v.Ts * v.Ts) * (size_t)split));
+    if (v.seg > 0) GL_TRY(reserve_segstate(v));
     PhaseScope ps(v.prof, PH_RASTER_FWD, s);
     int* work = v.persistent ? v.work.as<int>() : nullptr;   // cleared with the items
     const RasterArgs A = make_args(v, work);

@@ -139,10 +139,12 @@ double bytes_per_gaussian(int deg)
 }
 
 // Scratch of one step over views of P pixels in total (per-(view, Gaussian)
-// records and binning, per-instance and per-pixel buffers).
+// records and binning, per-instance and per-pixel buffers; an instance's share
+// of the split tiles' states is 24 bytes with 16x16 tiles and 512-record
+// segments).
 double step_scratch(double views, double n, double P, double inst_per_px)
 {
-    return views * n * 170.0 + P * 110.0 + inst_per_px * P * 1.25 * 90.0;
+    return views * n * 170.0 + P * 110.0 + inst_per_px * P * 1.25 * 114.0;
 }
 
 void finish(gl_server* s, Req* q, const gl_result& res)

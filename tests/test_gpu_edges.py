@@ -147,3 +147,8 @@ def test_render_into_device_images():
     E = np.concatenate([np.eye(3, dtype=np.float32), np.full((3, 1), 0.25, np.float32)], 1)
     m.render(cam, E=E, out_rgb=c)
     assert np.allclose(c.cpu().numpy(), hc + 0.25, atol=1e-6)
+
+
+@pytest.mark.parametrize("n", [1023, 1024, 1500])
+def test_default_execution_splits_deep_lists(n):
+    _check_stack(n, 0.02, True)
