@@ -223,8 +223,7 @@ GL_API gl_status gl_optimize_step(gl_map* map, const gl_keyframe* views, int32_t
  *                    tile, with a 2^-7 slack); renders are bit-identical
  *                    either way, the instance lists (and contributor
  *                    positions) shorter.
- *   segment          0 (the library's choice, 512 at present), or a power of
- *                    two in 64..65536: a tile whose list
+ *   segment          0, or a power of two in 64..65536: a tile whose list
  *                    holds at least 2 x segment Gaussians is rendered and
  *                    back-propagated as segments of `segment` consecutive
  *                    Gaussians by separate warps; the transmittance is then

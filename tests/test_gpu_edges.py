@@ -152,3 +152,32 @@ def test_render_into_device_images():
 @pytest.mark.parametrize("n", [1023, 1024, 1500])
 def test_default_execution_splits_deep_lists(n):
     _check_stack(n, 0.02, True)
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 257])
+@pytest.mark.parametrize("tile", [8, 16])
+def test_exact_culling_of_mixed_rectangles(n, tile):
+    """Rectangles from one tile to more than 64 within a warp: the instances
+    are the oracle's, bit for bit."""
+    from paper_2404_06926_gb300 import binding
+    rng = np.random.default_rng(n)
+    cam = scenes.camera(203, 151, 150.0, 150.0, 101.0, 75.0)
+    z = rng.uniform(0.1, 6.0, n)   # some behind the near plane
+    q = rng.normal(size=(n, 4))
+    params = dict(means=np.stack([rng.uniform(-0.8, 0.8, n) * z, rng.uniform(-0.6, 0.6, n) * z, z], 1).astype(np.float32),
+                  log_scales=rng.uniform(-5.0, -0.5, (n, 3)).astype(np.float32),
+                  quats=(q / np.linalg.norm(q, axis=1, keepdims=True)).astype(np.float32),
+                  logits=rng.normal(0, 2, n).astype(np.float32), sh=rng.normal(0, 0.5, (n, 1, 3)).astype(np.float32))
+    pre, bins, _ = oracle.forward(params, cam, tile)
+    ctx = binding.Ctx()
+    ctx.forward(_dev(params), cam, tile)
+    TX, TY = -(-cam["width"] // tile), -(-cam["height"] // tile)
+    out = ctx.preprocess(n, "cuda")
+    vis = pre["radius"] > 0
+    assert np.array_equal(out["radius"].cpu().numpy(), pre["radius"])
+    assert np.array_equal(out["rect"].cpu().numpy()[vis], pre["rect"][vis])
+    assert not out["rect"].cpu().numpy()[~vis].any()
+    assert ctx.num_instances() == bins["I"]
+    keys, vals, _ = ctx.instances(TX * TY, "cuda")
+    assert np.array_equal(keys.cpu().numpy().view(np.uint64), bins["keys"])
+    assert np.array_equal(vals.cpu().numpy().view(np.uint32), bins["vals"])
