@@ -302,24 +302,28 @@ __device__ __forceinline__ void blend_range(const RasterArgs& A, uint32_t a, uin
     }
 }
 
-// Per-lane pixel geometry of a unit.
-template <int D>
+// Per-lane pixel geometry of a unit: lane l owns pixels (l % 8, l / 8 + 4 j),
+// or (HALF) one pixel of its half-warp's 4 x 4 block: the lower half-warp has
+// the left block, the upper one the right.
+template <int D, bool HALF = false>
 struct LanePix {
-    int x;
+    int x, y;
     float px, py[D];   // relative to the tile's origin, as the records' means
     bool inside[D];
     int p[D];          // pixel index within the tile
     float bx0, bx1, by0, by1;
     __device__ __forceinline__ LanePix(const Unit& U, int TS, int lane)
     {
-        x = U.x0 + (lane & 7);
-        px = (float)(U.lx0 + (lane & 7));
+        static_assert(!HALF || D == 1, "a half-warp block has a pixel per lane");
+        const int lx = HALF ? (lane >> 4) * 4 + (lane & 3) : lane & 7, ly = HALF ? (lane >> 2) & 3 : lane >> 3;
+        x = U.x0 + lx;
+        y = U.y0 + ly;
+        px = (float)(U.lx0 + lx);
 #pragma unroll
         for (int j = 0; j < D; j++) {
-            const int y = U.y0 + (lane >> 3) + 4 * j;
-            py[j] = (float)(U.ly0 + (lane >> 3) + 4 * j);
-            inside[j] = x < U.W && y < U.H;
-            p[j] = (U.ly0 + (lane >> 3) + 4 * j) * TS + U.lx0 + (lane & 7);
+            py[j] = (float)(U.ly0 + ly + 4 * j);
+            inside[j] = x < U.W && y + 4 * j < U.H;
+            p[j] = (U.ly0 + ly + 4 * j) * TS + U.lx0 + lx;
         }
         bx0 = (float)U.x0;
         bx1 = (float)(U.x0 + 7);
@@ -328,7 +332,7 @@ struct LanePix {
     }
     __device__ __forceinline__ size_t pix(const Unit& U, int j) const
     {
-        return (size_t)U.pix_base + (size_t)(U.y0 + (threadIdx.x & 31) / 8 + 4 * j) * U.W + x;
+        return (size_t)U.pix_base + (size_t)(y + 4 * j) * U.W + x;
     }
 };
 
@@ -973,6 +977,265 @@ __device__ __forceinline__ void bwd_item(int u, const RasterArgs& A, const Raste
     __syncwarp();
 }
 
+// Half-warp blocks (one pixel per lane).  A Gaussian of the usual few pixels
+// reaches a quarter to a third of an 8 x 4 block, so a warp whose lanes all
+// evaluate the same hit idles most of them.  Here each half-warp has its own
+// 4 x 4 block and its own list of hits, and the two lists are walked side by
+// side: a step evaluates two different Gaussians.  Hits wait in a ring per
+// half-warp until sixteen are there, so that the halves' shares of a batch
+// even out.
+// Against the whole-warp backward: 79 -> 72 us (250k Gaussians, 640x512), 235 ->
+// 220 us (1M, 1280x1024), 92 -> 81 us (300k, 957x717), 3,959 -> 3,772 us (12
+// views of 2M).  The forward has no sums to add up and loses what its two
+// lists cost (185 -> 193 us, 1M; 3,347 -> 3,566 us): it keeps whole warps.
+constexpr int kRing = 48;    // three groups of 16: up to 16 waiting, a batch of 32 staged on top
+struct HalfRing {
+    float4 r0[kRing], r1[kRing], r2[kRing];
+    __device__ __forceinline__ void put(int k, const float4 a, const float4 b, const float4 c)
+    {
+        r0[k] = a; r1[k] = b; r2[k] = c;
+    }
+};
+
+// The waiting hits of the two half-warps (the same values in every lane):
+// entries tail .. tail + n of the ring, tail a multiple of 16.
+struct HalfQueue {
+    int head[2], tail[2], n[2];
+    __device__ __forceinline__ HalfQueue() { head[0] = head[1] = tail[0] = tail[1] = n[0] = n[1] = 0; }
+    // stage a batch's hits of half h (lane mask m), REV: in reverse lane order
+    template <bool REV>
+    __device__ __forceinline__ void stage(HalfRing& R, int h, unsigned m, unsigned lt, bool hit, const float4 a,
+                                          const float4 b, const float4 c)
+    {
+        const int cnt = __popc(m);
+        if (hit) {
+            const int r = __popc(m & lt);
+            int k = head[h] + (REV ? cnt - 1 - r : r);
+            if (k >= kRing) k -= kRing;
+            R.put(k, a, b, c);
+        }
+        head[h] += cnt;
+        if (head[h] >= kRing) head[h] -= kRing;
+        n[h] += cnt;
+    }
+    // the group of half h (up to 16 hits) has been walked
+    __device__ __forceinline__ void pop(int h)
+    {
+        tail[h] = tail[h] == kRing - 16 ? 0 : tail[h] + 16;
+        if (n[h] < 16) {   // all of them: the next hits start a group
+            n[h] = 0;
+            head[h] = tail[h];
+        } else {
+            n[h] -= 16;
+            if (n[h] == 0) head[h] = tail[h];
+        }
+    }
+};
+
+// The per-pixel backward over half-warp blocks (one pixel per lane, not
+// deterministic; the sums of a hit's two halves would need a row each).  A
+// group of up to sixteen hits per half-warp is walked, then the warp turns
+// over: lane (half, hit) adds up its hit over the half's sixteen pixels, so no
+// sum crosses lanes.  Bound by
+// instruction issue (67% of the cycles issue on the 1M view).
+struct BwdHalf {
+    static constexpr int S = 17;      // row stride (float2): the rows of a half on different banks
+    HalfRing ring[2];                 // hits; r1.w owner, r2.w list position (bits)
+    float4 pix[32];                   // per lane's pixel: dL/dC, dL/dD
+    float2 sv[32 * S];                // per (half, hit): (blend weight, dL/d(exponent)) of its pixels
+};
+
+template <bool EXTRA>
+__device__ __forceinline__ void half_turn_over(const RasterGrad& G, const BwdHalf& W, int at, bool on, float bx,
+                                               float by, int lane)
+{
+    const int half = lane >> 4;
+    const HalfRing& R = W.ring[half];
+    const float4 a = R.r0[at + (lane & 15)];
+    const float2* row = W.sv + lane * BwdHalf::S;
+    const float4* pc = W.pix + half * 16;
+    float c0 = 0.f, c1 = 0.f, c2 = 0.f, cD = 0.f, mxx = 0.f;
+    float m0[4] = {0.f, 0.f, 0.f, 0.f}, mx[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int x = 0; x < 4; x++) {
+        const float dx = a.x - (bx + (float)x), dx2 = dx * dx;
+#pragma unroll
+        for (int y = 0; y < 4; y++) {
+            const float2 v = row[y * 4 + x];
+            const float4 g = pc[y * 4 + x];
+            c0 = fmaf(v.x, g.x, c0); c1 = fmaf(v.x, g.y, c1); c2 = fmaf(v.x, g.z, c2);
+            if (EXTRA) cD = fmaf(v.x, g.w, cD);
+            m0[y] += v.y;
+            mx[y] = fmaf(v.y, dx, mx[y]);
+            mxx = fmaf(v.y, dx2, mxx);
+        }
+    }
+    float gy = 0.f, gxy = 0.f, gyy = 0.f;
+#pragma unroll
+    for (int y = 0; y < 4; y++) {
+        const float dy = a.y - (by + (float)y), t = dy * m0[y];
+        gy += t;
+        gxy = fmaf(dy, mx[y], gxy);
+        gyy = fmaf(dy, t, gyy);
+    }
+    if (on) {
+        const uint32_t id = __float_as_uint(R.r1[at + (lane & 15)].w);
+        float* dst = G.g2d + (size_t)id * kGradStride;
+        atomicAdd(reinterpret_cast<float4*>(dst), make_float4(c0, c1, c2, (m0[0] + m0[1]) + (m0[2] + m0[3])));
+        atomicAdd(reinterpret_cast<float4*>(dst + 4), make_float4((mx[0] + mx[1]) + (mx[2] + mx[3]), gy, mxx, gxy));
+        if (EXTRA) atomicAdd(reinterpret_cast<float2*>(dst + 8), make_float2(gyy, cD));
+        else atomicAdd(dst + 8, gyy);
+    }
+}
+
+template <bool EXTRA>
+__device__ __forceinline__ void bwd_half_item(int u, const RasterArgs& A, const RasterGrad& G, BwdHalf& W, int lane)
+{
+    Unit U;
+    unit_of<1>(u, A, U);
+    const LanePix<1, true> L(U, A.TS, lane);
+    const unsigned lt = (1u << lane) - 1u;
+    const int half = lane >> 4, l16 = lane & 15;
+    HalfRing& R = W.ring[half];
+    float T = 1.0f, R0 = 0.f, R1 = 0.f, R2 = 0.f, RD = 0.f, RO = 0.f;   // as bwd_item
+    float g0 = 0.f, g1 = 0.f, g2 = 0.f, gD = 0.f, gO = 0.f;
+    uint32_t last = 0;
+    if (L.inside[0]) {
+        const size_t p = L.pix(U, 0);
+        last = G.ncon[p];
+        g0 = G.dL_drgb[3 * p]; g1 = G.dL_drgb[3 * p + 1]; g2 = G.dL_drgb[3 * p + 2];
+        if (EXTRA) {
+            gD = G.dL_ddepth ? G.dL_ddepth[p] : 0.0f;
+            gO = G.dL_dopac ? G.dL_dopac[p] : 0.0f;
+        }
+        if (U.nseg == 1) {
+            T = G.Tfin[p];
+        } else if (last > U.rs - U.trs) {   // (no state behind the stop segment)
+            const float* S = A.segstate;
+            const int i = L.p[0];
+            T = S[seg_at(U.w, 0, i, A.TS)];
+            R0 = S[seg_at(U.w, 1, i, A.TS)];
+            R1 = S[seg_at(U.w, 2, i, A.TS)];
+            R2 = S[seg_at(U.w, 3, i, A.TS)];
+            if (EXTRA) {
+                RD = S[seg_at(U.w, 4, i, A.TS)];
+                RO = S[seg_at(U.w, 5, i, A.TS)];
+            }
+        }
+    }
+    W.pix[lane] = make_float4(g0, g1, g2, gD);
+    // positions at or beyond a half's last contributor reach none of its pixels
+    uint32_t hmax = last;
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) hmax = max(hmax, __shfl_xor_sync(kFull, hmax, off));
+    const uint32_t last0 = __shfl_sync(kFull, hmax, 0), last1 = __shfl_sync(kFull, hmax, 16);
+    const uint32_t end = min(U.re, U.trs + max(last0, last1));
+    if (end <= U.rs) return;
+    const float bx = (float)(U.lx0 + 4 * half), by = (float)U.ly0;
+    HalfQueue Q;
+    // batches of 32 from the back, the last one clipped at rs: i = hi - 32 + lane
+    uint32_t hi = end;
+    float4 n0, n1, n2, n3;
+    uint32_t ng = 0;
+    if (hi - U.rs + lane >= 32u) {
+        const uint32_t i = hi - 32u + lane;
+        n0 = A.s0[i]; n1 = A.s1[i]; n2 = A.s2[i]; n3 = A.s3[i];
+        ng = A.sgid[i];
+    }
+    while (true) {
+        const uint32_t left = hi - U.rs;   // records of this and the batches before it
+        const bool valid = left + lane >= 32u, more = left > 32u;
+        const uint32_t pos = hi - 32u + lane - U.trs;
+        const float4 c0 = n0, c3 = n3;
+        float4 c1 = n1, c2 = n2;
+        c1.w = __uint_as_float(ng);
+        c2.w = __uint_as_float(pos);
+        if (more && left - 32u + lane >= 32u) {
+            const uint32_t i = hi - 64u + lane;
+            n0 = A.s0[i]; n1 = A.s1[i]; n2 = A.s2[i]; n3 = A.s3[i];
+            ng = A.sgid[i];
+        }
+        const bool rows = valid && !(c3.w < L.by0 || c3.z > L.by1);
+        const bool h0 = rows && pos < last0 && !(c3.y < L.bx0 || c3.x > L.bx0 + 3.0f);
+        const bool h1 = rows && pos < last1 && !(c3.y < L.bx0 + 4.0f || c3.x > L.bx0 + 7.0f);
+        const unsigned m0 = __ballot_sync(kFull, h0), m1 = __ballot_sync(kFull, h1);
+        Q.stage<true>(W.ring[0], 0, m0, lt, h0, c0, c1, c2);
+        Q.stage<true>(W.ring[1], 1, m1, lt, h1, c0, c1, c2);
+        const int keep = more ? 16 : 0;   // the last batch leaves none waiting
+        while (max(Q.n[0], Q.n[1]) > keep) {
+            const int k0 = min(Q.n[0], 16), k1 = min(Q.n[1], 16), steps = max(k0, k1);
+            const int mine = half ? k1 : k0, at = half ? Q.tail[1] : Q.tail[0];
+            if (l16 >= mine && l16 < ((steps + 1) & ~1)) {
+                R.r0[at + l16] = R.r2[at + l16] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                R.r1[at + l16] = make_float4(0.0f, -3.0e38f, 0.0f, 0.0f);
+            }
+            __syncwarp();
+            float2* sv = W.sv + half * 16 * BwdHalf::S + l16;
+            for (int k = 0; k < steps; k += 2, sv += 2 * BwdHalf::S) {
+                float4 a[2], b[2], c[2];
+                float al[2];
+#pragma unroll
+                for (int e = 0; e < 2; e++) {
+                    a[e] = R.r0[at + k + e];
+                    b[e] = R.r1[at + k + e];
+                    c[e] = R.r2[at + k + e];
+                }
+#pragma unroll
+                for (int e = 0; e < 2; e++) {
+                    float dx, dy, alpha;
+                    bool capped;
+                    const bool live = pair_eval_nb(a[e], b[e], L.px, L.py[0], dx, dy, alpha, capped) &&
+                                      __float_as_uint(c[e].w) < last;
+                    al[e] = live ? alpha : 0.0f;
+                }
+#pragma unroll
+                for (int e = 0; e < 2; e++) {
+                    // as bwd_item
+                    T = __fdividef(T, 1.0f - al[e]);
+                    const float wgt = al[e] * T;
+                    const float d0 = c[e].x - R0, d1 = c[e].y - R1, d2 = c[e].z - R2;
+                    float dot = g0 * d0 + g1 * d1 + g2 * d2;
+                    R0 = fmaf(al[e], d0, R0);
+                    R1 = fmaf(al[e], d1, R1);
+                    R2 = fmaf(al[e], d2, R2);
+                    if (EXTRA) {
+                        const float dD = b[e].z - RD, dO = 1.0f - RO;
+                        dot += gD * dD + gO * dO;
+                        RD = fmaf(al[e], dD, RD);
+                        RO = fmaf(al[e], dO, RO);
+                    }
+                    sv[e * BwdHalf::S] = make_float2(wgt, al[e] < kAlphaMax ? wgt * dot : 0.0f);
+                }
+            }
+            __syncwarp();
+            half_turn_over<EXTRA>(G, W, at, l16 < mine, bx, by, lane);
+            __syncwarp();
+            Q.pop(0);
+            Q.pop(1);
+        }
+        if (!more) break;
+        hi -= 32u;
+    }
+}
+
+constexpr int kWpbHalf = 4;       // 43.5 KB of shared memory a CTA
+constexpr int kMinBlocksHalf = 5; // 96 registers, 20 warps per SM
+
+template <bool EXTRA>
+__global__ void __launch_bounds__(32 * kWpbHalf, kMinBlocksHalf) k_raster_bwd_half(RasterArgs A, RasterGrad G)
+{
+    __shared__ BwdHalf sw[kWpbHalf];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nunits = (int)A.ctl[6] * A.nblk;
+    int u = A.work ? next_unit(A.work, lane) : blockIdx.x * kWpbHalf + w;
+    while (u < nunits) {
+        bwd_half_item<EXTRA>(u, A, G, sw[w], lane);
+        __syncwarp();
+        if (!A.work) break;
+        u = next_unit(A.work, lane);
+    }
+}
+
 template <bool EXTRA, int NB, int D, bool DET>
 __global__ void __launch_bounds__(32 * wpb_bwd<NB>(), minb_bwd<NB, D>()) k_raster_bwd(RasterArgs A, RasterGrad G)
 {
@@ -1530,6 +1793,13 @@ void bwd_dispatch(int nb, int pd, bool det, bool pg, const RasterArgs& A, const 
         if (pd == 1) bwd_launch<EXTRA, 1, 1, true>(A, G, units, persistent, s);
         else if (pd == 2) bwd_launch<EXTRA, 1, 2, true>(A, G, units, persistent, s);
         else bwd_launch<EXTRA, 1, 4, true>(A, G, units, persistent, s);
+    } else if (pd == 1 && units >= (int64_t)kMinBlocksHalf * kWpbHalf * sm_count()) {
+        // more pixel blocks than resident warps.  Below, a warp has one block
+        // and its chain is the time, which the two lists lengthen: 17.8 -> 22.4
+        // us on 5k Gaussians at 256x192 (1.5k blocks; the line lies at 3.0k).
+        // (Hits wait in a ring, whatever the batch depth.)
+        const int grid = grid_for(k_raster_bwd_half<EXTRA>, units, persistent, kWpbHalf);
+        k_raster_bwd_half<EXTRA><<<grid, 32 * kWpbHalf, 0, s>>>(A, G);
     } else if (nb == 4) {   // deeper batches: one pixel per lane
         bwd_launch<EXTRA, 4, 1, false>(A, G, units, persistent, s);
     } else if (nb == 8) {

@@ -181,3 +181,37 @@ def test_exact_culling_of_mixed_rectangles(n, tile):
     keys, vals, _ = ctx.instances(TX * TY, "cuda")
     assert np.array_equal(keys.cpu().numpy().view(np.uint64), bins["keys"])
     assert np.array_equal(vals.cpu().numpy().view(np.uint32), bins["vals"])
+
+
+@pytest.mark.parametrize("n,seg", [(60, 0), (700, 0), (700, 64)])
+@pytest.mark.parametrize("extra", [False, True])
+def test_backward_with_more_blocks_than_warps(n, seg, extra):
+    """A frame large enough for the half-warp backward (3,192 pixel blocks), of
+    ragged size, with Gaussians from under a pixel to half the frame."""
+    from paper_2404_06926_gb300 import binding
+    rng = np.random.default_rng(n)
+    W, H = 331, 300
+    cam = scenes.camera(W, H, 250.0, 250.0, W / 2, H / 2)
+    z = rng.uniform(1.0, 6.0, n)
+    q = rng.normal(size=(n, 4))
+    params = dict(means=np.stack([rng.uniform(-0.7, 0.7, n) * z, rng.uniform(-0.6, 0.6, n) * z, z], 1).astype(np.float32),
+                  log_scales=rng.uniform(-6.0, -0.5, (n, 3)).astype(np.float32),
+                  quats=(q / np.linalg.norm(q, axis=1, keepdims=True)).astype(np.float32),
+                  logits=rng.normal(0, 1.5, n).astype(np.float32), sh=rng.normal(0, 0.5, (n, 1, 3)).astype(np.float32))
+    pre, bins, img = oracle.forward(params, cam, 16)
+    dC = (rng.normal(size=(H, W, 3)) * 1e-3).astype(np.float32)
+    dD = (rng.normal(size=(H, W)) * 1e-4).astype(np.float32) if extra else None
+    dO = (rng.normal(size=(H, W)) * 1e-3).astype(np.float32) if extra else None
+    g = oracle.backward(params, cam, pre, bins, dC.astype(np.float64), None if dD is None else dD.astype(np.float64),
+                        None if dO is None else dO.astype(np.float64))
+    ctx = binding.Ctx()
+    ctx.set_exec(segment=seg, persistent=1 if seg else 0)
+    p = _dev(params)
+    ctx.forward(p, cam, 16)
+    tt = lambda a: None if a is None else torch.from_numpy(a).cuda()
+    gg, _ = ctx.backward(p, tt(dC), tt(dD), tt(dO))
+    vis = pre["radius"] > 0
+    for name in NAMES:
+        a, ref = gg[name].cpu().numpy().astype(np.float64)[vis].ravel(), np.asarray(g[name], np.float64)[vis].ravel()
+        rel = np.abs(a - ref) / np.maximum(np.abs(ref), 1e-4 * np.abs(ref).max())
+        assert np.median(rel) < 1e-3 and np.percentile(rel, 99) < 1e-2, (name, np.median(rel), np.percentile(rel, 99))
