@@ -167,7 +167,7 @@ struct View {
     DevBuf itile, ival, itile2, ival2;  // u32 global tile id, u32 instance id (sort; input ids implied)
     DevBuf iowner;            // u32 owning (view, Gaussian) per instance id
     DevBuf srec0, srec1, srec2, srec3;  // records in sorted-instance order
-    DevBuf sgid;              // u32 owning (view, Gaussian) per sorted instance
+    DevBuf sgid;              // u32 owning (view, Gaussian) per sorted instance (deterministic binning)
     DevBuf hist;              // radix look-back words
     DevBuf sctl;              // radix digit counts and tile counters: depth sort, tile sort
     DevBuf ranges;            // uint2 per global tile
@@ -178,7 +178,8 @@ struct View {
     // sorted-order results of the last forward (pointers into the buffers above)
     const uint32_t* sorted_g = nullptr;
     const uint32_t* sorted_tile = nullptr;
-    const uint32_t* sorted_inst = nullptr;
+    const uint32_t* sorted_inst = nullptr;    // emission index (deterministic binning; else null)
+    const uint32_t* sorted_owner = nullptr;   // owning (view, Gaussian) (null: through sorted_inst and iowner)
     uint64_t* h_count = nullptr;          // pinned copy of count[0..8]
     Prof* prof = nullptr;                 // optional phase timers
     // raster execution: records per lane per batch (1: 32, 2: 64), pixels per

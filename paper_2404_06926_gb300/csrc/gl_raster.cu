@@ -1632,7 +1632,8 @@ k_part_reduce(const float* __restrict__ part, const uint32_t* __restrict__ pmask
     }
 }
 
-// Records in sorted-instance order (and the owning Gaussian of each), the
+// Records in sorted-instance order (and, where instance ids were sorted, the
+// owning Gaussian of each), the
 // mean made relative to the origin of the instance's tile: (u_hi - x0) is
 // exact near the tile (Sterbenz), and adding u_lo leaves an offset accurate
 // to float precision of a number of pixels, not of the image coordinate.
@@ -1648,7 +1649,7 @@ __global__ void k_permute(const uint64_t* __restrict__ n_dev, uint32_t* __restri
 {
     const uint64_t I = *n_dev;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < I; i += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t g = owner[sinst[i]];
+        const uint32_t g = sinst ? owner[sinst[i]] : owner[i];
         const int tile = (int)stile[i];
         if (i == 0 || stile[i - 1] != (uint32_t)tile) ranges[2 * tile] = (uint32_t)i;
         if (i == I - 1 || stile[i + 1] != (uint32_t)tile) ranges[2 * tile + 1] = (uint32_t)(i + 1);
@@ -1661,7 +1662,7 @@ __global__ void k_permute(const uint64_t* __restrict__ n_dev, uint32_t* __restri
         a.x = __fadd_rn(__fsub_rn(a.x, x0), c.w);
         a.y = __fadd_rn(__fsub_rn(a.y, y0), b.w);
         s0[i] = a; s1[i] = b; s2[i] = c; s3[i] = box;
-        sg[i] = g;
+        if (sinst) sg[i] = g;
     }
 }
 
@@ -1719,7 +1720,7 @@ RasterArgs make_args(View& v, int* work)
     A.s1 = v.srec1.as<float4>();
     A.s2 = v.srec2.as<float4>();
     A.s3 = v.srec3.as<float4>();
-    A.sgid = v.sgid.as<uint32_t>();
+    A.sgid = v.sorted_owner ? v.sorted_owner : v.sgid.as<uint32_t>();
     A.views = v.d_desc();
     A.segstate = v.segstate.as<float>();
     A.work = work;
@@ -1825,10 +1826,10 @@ gl_status permute_records(View& v, int64_t nmax, cudaStream_t s)
     GL_TRY(v.srec1.reserve(16 * I));
     GL_TRY(v.srec2.reserve(16 * I));
     GL_TRY(v.srec3.reserve(16 * I));
-    GL_TRY(v.sgid.reserve(4 * I));
+    if (v.sorted_inst) GL_TRY(v.sgid.reserve(4 * I));
     const int blocks = (int)std::min<size_t>(8 * (size_t)sm_count(), (I + 255) / 256);
     k_permute<<<blocks, 256, 0, s>>>(v.count.as<uint64_t>(), v.ranges.as<uint32_t>(), v.sorted_inst, v.sorted_tile, v.d_desc(), v.V, v.Ts,
-                                     v.iowner.as<uint32_t>(),
+                                     v.sorted_owner ? v.sorted_owner : v.iowner.as<uint32_t>(),
                                      v.rec.as<float4>(), v.srec0.as<float4>(), v.srec1.as<float4>(),
                                      v.srec2.as<float4>(), v.srec3.as<float4>(), v.sgid.as<uint32_t>());
     count_launches(1);
