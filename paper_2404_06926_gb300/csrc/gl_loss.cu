@@ -6,12 +6,13 @@
 // C2 = 0.03^2 -- the D-SSIM of 3DGS the paper cites.
 //
 // One CTA per 32x32 output tile and channel, the three channels of a tile in
-// one cluster.  A CTA loads the channel's exposed colour x and target y over
+// one cluster (k_loss_split), or for large launches one CTA per tile that
+// takes the channels in turn (k_loss; the rule is at launch_loss).  A CTA loads the channel's exposed colour x and target y over
 // the tile plus a 10-pixel halo as (x, y) pairs, blurs the five moment maps
 // separably over a 5-pixel halo, forms the SSIM map and its partials w.r.t. (mu_x, E[x^2], E[xy]) and
 // blurs those back (the adjoint of a zero-padded symmetric correlation is the
-// same correlation).  dL/dC = A^T dL/dE[C] needs all three channels: each CTA
-// leaves its dL/dE[C] in shared memory and, after a cluster barrier, CTA j
+// same correlation).  dL/dC = A^T dL/dE[C] needs all three channels: k_loss adds
+// them up in registers; in a cluster each CTA leaves its dL/dE[C] in shared memory and, after a cluster barrier, CTA j
 // reads the other two and writes component j.
 //
 // Bound: FP32 issue.  Four of the maps are kept as pairs, (mu_x, mu_y) and
@@ -94,12 +95,13 @@ struct LossOne {
     int W, H;
 };
 
-// Grid: a cluster of three CTAs (the channels) per 32x32 loss tile over all
-// views.  With `views` null the single view `one` is used; otherwise view,
+// Grid: a cluster of three CTAs (the channels; SPLIT) or one CTA per 32x32
+// loss tile over all views.  With `views` null the single view `one` is used; otherwise view,
 // images, exposure and weight come from the descriptors and images are the
 // concatenated ones.
-__global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(kThreads, 3)
-k_loss(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __restrict__ rgb_all,
+template <bool SPLIT>
+__device__ __forceinline__ void
+loss_tile(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __restrict__ rgb_all,
        float* __restrict__ dL_all, float lambda, float* __restrict__ part)
 {
     namespace cg = cooperative_groups;
@@ -109,8 +111,8 @@ k_loss(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __re
     float* dL_drgb = one.dL;
     int W = one.W, H = one.H;
     float weight = 1.0f;
-    const int ch = blockIdx.x % 3;   // the rank in the cluster
-    int lt = blockIdx.x / 3;
+    int lt = SPLIT ? blockIdx.x / 3 : blockIdx.x;
+    const int tile = lt;
     if (views) {
         const int v = view_of_ltile(views, V, lt);
         const ViewDesc& d = views[v];
@@ -132,17 +134,24 @@ k_loss(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __re
     float* hp = reinterpret_cast<float*>(hm + 2 * RA * RB);        // E[xy]
     float2* hab = hm;                                              // RB rows x HS (reuses hm)
     float* hc = reinterpret_cast<float*>(hab + RB * HS);           // RB rows x HS
-    __shared__ float red[6][kThreads / 32];
+    __shared__ float red[kNP][kThreads / 32];
     __shared__ float chsum[3][2];    // in CTA 0 of the cluster: the channels' sums of |.| and SSIM
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const float e0 = E ? E[4 * ch] : (ch == 0 ? 1.0f : 0.0f), e1 = E ? E[4 * ch + 1] : (ch == 1 ? 1.0f : 0.0f);
-    const float e2 = E ? E[4 * ch + 2] : (ch == 2 ? 1.0f : 0.0f), e3 = E ? E[4 * ch + 3] : 0.0f;
     const int LTX = (W + LT - 1) / LT;
     const int ox = (lt % LTX) * LT, oy = (lt / LTX) * LT;
     const float invN = 1.0f / (3.0f * (float)W * (float)H);
     const float gS = -lambda * invN * weight;
     const float gL1 = (1.0f - lambda) * invN * weight;
 
+    float l1acc = 0.0f, sacc = 0.0f;
+    static_assert(LT * (LT / AVR) == kThreads, "one adjoint run per thread");
+    const int c = tid % LT, r0 = (tid / LT) * AVR;
+    float dC[AVR][3];   // !SPLIT: dL/dC of the thread's pixels
+    const int first = SPLIT ? blockIdx.x % 3 : 0;   // SPLIT: the rank in the cluster
+#pragma unroll 1
+    for (int ch = first; ch < (SPLIT ? first + 1 : 3); ch++) {
+    const float e0 = E ? E[4 * ch] : (ch == 0 ? 1.0f : 0.0f), e1 = E ? E[4 * ch + 1] : (ch == 1 ? 1.0f : 0.0f);
+    const float e2 = E ? E[4 * ch + 2] : (ch == 2 ? 1.0f : 0.0f), e3 = E ? E[4 * ch + 3] : 0.0f;
     // a warp per row, two columns per lane; a tile whose halo lies inside the
     // image takes the loads without bounds
     const bool inner = ox >= 2 * HW && oy >= 2 * HW && ox + LT + 2 * HW <= W && oy + LT + 2 * HW <= H;
@@ -208,7 +217,6 @@ k_loss(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __re
     }
     __syncthreads();
     // vertical pass, SSIM and its partials: runs of VR rows of one column
-    float l1acc = 0.0f, sacc = 0.0f;
     if (tid < RB * (RB / VR)) {
         const int c = tid % RB, r0 = (tid / RB) * VR;
         float2 m[VR], q[VR];
@@ -286,8 +294,6 @@ k_loss(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __re
     __syncthreads();
     // adjoint, vertical, and dL/dE[C] of the tile's pixels: runs of AVR rows
     // of a column (x, y read again: their shared copy is overwritten)
-    static_assert(LT * (LT / AVR) == kThreads, "one adjoint run per thread");
-    const int c = tid % LT, r0 = (tid / LT) * AVR;
     float pe[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // exposure gradient: sum g C_j (j < 3), sum g
     float g[AVR];
     {
@@ -319,30 +325,45 @@ k_loss(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __re
                 g[o] = a[o].x + 2.f * x * a[o].y + y * b[o] + gL1 * (d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f));
                 pe[0] += g[o] * c0; pe[1] += g[o] * c1; pe[2] += g[o] * c2; pe[3] += g[o];
             }
-            gout[(r0 + o) * LT + c] = g[o];
+            if (SPLIT) {
+                gout[(r0 + o) * LT + c] = g[o];
+            } else {
+                dC[o][0] = ch == 0 ? e0 * g[o] : fmaf(e0, g[o], dC[o][0]);
+                dC[o][1] = ch == 0 ? e1 * g[o] : fmaf(e1, g[o], dC[o][1]);
+                dC[o][2] = ch == 0 ? e2 * g[o] : fmaf(e2, g[o], dC[o][2]);
+            }
         }
     }
-    {
-        const float vals[6] = {pe[0], pe[1], pe[2], pe[3], l1acc, sacc};
 #pragma unroll
-        for (int i = 0; i < 6; i++) {
+    for (int i = 0; i < 4; i++) {
+        float v = pe[i];
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
+        if (lane == 0) red[4 * ch + i][wid] = v;
+    }
+    }
+    {
+        const float vals[2] = {l1acc, sacc};
+#pragma unroll
+        for (int i = 0; i < 2; i++) {
             float v = vals[i];
             for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
-            if (lane == 0) red[i][wid] = v;
+            if (lane == 0) red[12 + i][wid] = v;
         }
     }
     __syncthreads();
-    cg::cluster_group cluster = cg::this_cluster();
-    float* prow = part + (size_t)(blockIdx.x / 3) * kNP;
-    if (tid < 6) {
-        float v = 0.0f;
-        for (int ww = 0; ww < kThreads / 32; ww++) v += red[tid][ww];
-        if (tid < 4) prow[4 * ch + tid] = v;
-        else cluster.map_shared_rank(&chsum[0][0], 0)[2 * ch + tid - 4] = v;
-    }
-    cluster.sync();
-    // component ch of dL/dC = sum over channels k of A[k][ch] dL/dE[C]_k
-    {
+    float* prow = part + (size_t)tile * kNP;
+    if constexpr (SPLIT) {
+        const int ch = first;
+        cg::cluster_group cluster = cg::this_cluster();
+        if (tid < 6) {
+            const int k = tid < 4 ? 4 * ch + tid : 8 + tid;
+            float v = 0.0f;
+            for (int ww = 0; ww < kThreads / 32; ww++) v += red[k][ww];
+            if (tid < 4) prow[k] = v;
+            else cluster.map_shared_rank(&chsum[0][0], 0)[2 * ch + tid - 4] = v;
+        }
+        cluster.sync();
+        // component ch of dL/dC = sum over channels k of A[k][ch] dL/dE[C]_k
         const float f0 = E ? E[ch] : (ch == 0 ? 1.0f : 0.0f), f1 = E ? E[4 + ch] : (ch == 1 ? 1.0f : 0.0f);
         const float f2 = E ? E[8 + ch] : (ch == 2 ? 1.0f : 0.0f);
         const float* g0 = cluster.map_shared_rank(gout, 0);
@@ -354,9 +375,39 @@ k_loss(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __re
             const float v = fmaf(f2, g2[i], fmaf(f1, g1[i], f0 * g0[i]));
             if (gx < W && gy < H) dL_drgb[3 * ((size_t)gy * W + gx) + ch] = v;
         }
+        if (ch == 0 && tid < 2) prow[12 + tid] = chsum[0][tid] + chsum[1][tid] + chsum[2][tid];
+        cluster.sync();   // the shared memory read by the other CTAs stays until they are done
+    } else {
+        if (tid < kNP) {
+            float v = 0.0f;
+            for (int ww = 0; ww < kThreads / 32; ww++) v += red[tid][ww];
+            prow[tid] = v;
+        }
+#pragma unroll
+        for (int o = 0; o < AVR; o++) {
+            const int gx = ox + c, gy = oy + r0 + o;
+            if (gx < W && gy < H) {
+                const size_t p = 3 * ((size_t)gy * W + gx);
+                dL_drgb[p] = dC[o][0];
+                dL_drgb[p + 1] = dC[o][1];
+                dL_drgb[p + 2] = dC[o][2];
+            }
+        }
     }
-    if (ch == 0 && tid < 2) prow[12 + tid] = chsum[0][tid] + chsum[1][tid] + chsum[2][tid];
-    cluster.sync();   // the shared memory read by the other CTAs stays until they are done
+}
+
+__global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(kThreads, 3)
+k_loss_split(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __restrict__ rgb_all,
+             float* __restrict__ dL_all, float lambda, float* __restrict__ part)
+{
+    loss_tile<true>(one, views, V, rgb_all, dL_all, lambda, part);
+}
+
+__global__ void __launch_bounds__(kThreads, 3)
+k_loss(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __restrict__ rgb_all,
+       float* __restrict__ dL_all, float lambda, float* __restrict__ part)
+{
+    loss_tile<false>(one, views, V, rgb_all, dL_all, lambda, part);
 }
 
 // Sums the per-tile partials in a fixed order (float pairs, df_acc).  Single
@@ -476,9 +527,26 @@ int loss_partials_needed(int W, int H)
 }
 
 namespace {
-gl_status loss_attr()
+// Tiles per SM from which a CTA takes all three channels of a tile: two waves
+// of CTAs.  Then no cluster waits for its slowest channel and the channels
+// share the rows in L1; below, a third of the chain per CTA counts more.  A
+// cluster and one CTA per tile: 105 and 97 us (1280x1024, 1,280 tiles), 850 and
+// 656 (12 views, 9.5k); with four CTAs per SM (an earlier form of the moments)
+// 13 and 26 us (256x192, 48), 29 and 36 (647x481, 336), 57 and 62 (957x717, 690);
+// the line lies at 1.2k.
+constexpr int kWholeTilesPerSm = 8;
+
+gl_status launch_loss(const LossOne& one, const ViewDesc* views, int V, const float* rgb, float* dL, float lambda,
+                      float* part, int tiles, cudaStream_t s)
 {
-    return ensure_smem_limit(reinterpret_cast<const void*>(&k_loss), (int)kSmemBytes);
+    GL_TRY(ensure_smem_limit(reinterpret_cast<const void*>(&k_loss_split), (int)kSmemBytes));
+    GL_TRY(ensure_smem_limit(reinterpret_cast<const void*>(&k_loss), (int)kSmemBytes));
+    if (tiles < kWholeTilesPerSm * sm_count()) {
+        k_loss_split<<<3 * tiles, kThreads, kSmemBytes, s>>>(one, views, V, rgb, dL, lambda, part);
+    } else {
+        k_loss<<<tiles, kThreads, kSmemBytes, s>>>(one, views, V, rgb, dL, lambda, part);
+    }
+    return GL_OK;
 }
 }  // namespace
 
@@ -486,10 +554,9 @@ gl_status photometric_loss(const float* rgb, const float* target, const float* E
                            float lambda, float* dL_drgb, float* part, float* loss_out, float* dE_out,
                            cudaStream_t s)
 {
-    GL_TRY(loss_attr());
     const int nblk = ((W + LT - 1) / LT) * ((H + LT - 1) / LT);
     LossOne one{rgb, target, E, dL_drgb, W, H};
-    k_loss<<<3 * nblk, kThreads, kSmemBytes, s>>>(one, nullptr, 0, nullptr, nullptr, lambda, part);
+    GL_TRY(launch_loss(one, nullptr, 0, nullptr, nullptr, lambda, part, nblk, s));
     k_loss_final<<<1, kRedThreads, 0, s>>>(part, nblk, W, H, lambda, loss_out, dE_out, nullptr, nullptr, 0.f, 0.f,
                                         0.f, 0.f, nullptr);
     count_launches(2);
@@ -501,10 +568,8 @@ gl_status photometric_loss_views(const View& v, const float* rgb, float lambda, 
                                  float* loss_v, float b1, float b2, float eps, float lr, cudaStream_t s,
                                  const uint64_t* abort)
 {
-    GL_TRY(loss_attr());
     LossOne one{};
-    k_loss<<<3 * v.nltiles, kThreads, kSmemBytes, s>>>(one, v.d_desc(), v.V, rgb, dL_drgb, lambda,
-                                                                     part);
+    GL_TRY(launch_loss(one, v.d_desc(), v.V, rgb, dL_drgb, lambda, part, v.nltiles, s));
     k_loss_final<<<v.V, kRedThreads, 0, s>>>(part, 0, 0, 0, lambda, nullptr, nullptr, v.d_desc(), loss_v, b1, b2, eps,
                                           lr, abort);
     count_launches(2);
