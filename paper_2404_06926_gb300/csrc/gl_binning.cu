@@ -862,6 +862,16 @@ __global__ void k_accumulate_counts(const int* __restrict__ radius, int64_t n, c
     }
 }
 
+// Pinned host memory is written in place: a copy node costs a gap of several
+// microseconds after the last kernel, and there were two.
+__global__ void k_report(const float* __restrict__ loss, int V, const uint64_t* __restrict__ count, int nc,
+                         float* __restrict__ h_loss, uint64_t* __restrict__ h_count)
+{
+    const int i = threadIdx.x;
+    if (i < V) h_loss[i] = loss[i];
+    if (i < nc) h_count[i] = count[i];
+}
+
 int ceil_log2(int64_t x)
 {
     int b = 0;
@@ -985,6 +995,16 @@ gl_status sort_wait_selftest(int32_t* expired)
     uint64_t flag = 0;
     GL_CUDA_TRY(cudaMemcpy(&flag, c + 8, sizeof(flag), cudaMemcpyDeviceToHost));
     *expired = flag ? 1 : 0;
+    return GL_OK;
+}
+
+gl_status report_step(const View& v, const float* loss_dev, float* h_loss, cudaStream_t s)
+{
+    static_assert(kMaxViews <= 64, "a thread per view");
+    k_report<<<1, 64, 0, s>>>(loss_dev, v.V, v.count.as<uint64_t>(), (int)(kCountCopy / sizeof(uint64_t)), h_loss,
+                              v.h_count);
+    count_launches(1);
+    GL_CUDA_TRY(cudaGetLastError());
     return GL_OK;
 }
 
@@ -1243,8 +1263,8 @@ gl_status bin_views(View& v, const GParams& p, const Cam* cams, const ViewExtra*
         GL_TRY(build_items(v, s));
     }
     // the counters reach the host at the caller's next synchronisation
-    // (sort_wait_status); graph steps copy them at the end of the step
-    if (!sync_free) GL_CUDA_TRY(cudaMemcpyAsync(v.h_count, count, kCountCopy, cudaMemcpyDeviceToHost, s));
+    // (sort_wait_status); steps report them at their end
+    if (!sync_free && !grad) GL_CUDA_TRY(cudaMemcpyAsync(v.h_count, count, kCountCopy, cudaMemcpyDeviceToHost, s));
     return GL_OK;
 }
 

@@ -683,7 +683,8 @@ struct gl_map {
     gl_ctx_impl ctx;
     DevBuf stage_img, stage_pts, dLdC, loss_dev;
     DevBuf flags, scan;
-    float* h_loss = nullptr;
+    float* h_loss = nullptr;             // pinned: losses of a step's views
+    float* h_expo = nullptr;             // pinned: an exposure on its way to the caller
     std::unordered_map<int64_t, std::unique_ptr<Keyframe>> kfs;
     Prof prof;
     // step execution and the captured step graph
@@ -873,6 +874,7 @@ extern "C" gl_status gl_map_create(const gl_config* cfg, void* stream, gl_map** 
     m->ctx.view.prof = &m->prof;
     GL_TRY(m->ctx.view.init());
     GL_CUDA_TRY(cudaMallocHost(&m->h_loss, sizeof(float) * kMaxViews));
+    GL_CUDA_TRY(cudaMallocHost(&m->h_expo, sizeof(float) * 12));
     GL_TRY(m->loss_dev.reserve(16));
     GL_TRY(map_reserve(m.get(), std::max<int64_t>(cfg->n_sky, 1)));
     if (cfg->n_sky > 0) {
@@ -900,6 +902,7 @@ extern "C" gl_status gl_map_destroy(gl_map* m)
     m->flags.release(); m->scan.release(); m->timed_counts.release();
     for (auto& kv : m->kfs) { kv.second->image.release(); kv.second->expo.release(); }
     if (m->h_loss) cudaFreeHost(m->h_loss);
+    if (m->h_expo) cudaFreeHost(m->h_expo);
     for (auto& g : m->graphs) cudaGraphExecDestroy(g.exec);
     if (m->gstream) cudaStreamDestroy(m->gstream);
     if (m->cstream) {
@@ -1181,22 +1184,16 @@ gl_status enqueue_step(gl_map* m, const StepPlan& sp, cudaStream_t s, bool sync_
     a.abort = ctl;
     if (sync_free) a.bc = v.d_scal();
     GL_TRY(params_adam(v, m->params(), gl_map::mut(m->prm), a, s));
-    if (sync_free) {
-        GL_CUDA_TRY(cudaMemcpyAsync(m->h_loss, m->loss_dev.p, 4 * (size_t)V, cudaMemcpyDeviceToHost, s));
-        GL_CUDA_TRY(cudaMemcpyAsync(v.h_count, v.count.p, kCountCopy, cudaMemcpyDeviceToHost, s));
-    }
-    return GL_OK;
+    return report_step(v, m->loss_dev.as<float>(), m->h_loss, s);
 }
 
-gl_status read_loss(gl_map* m, int V, bool copy, float* out_loss)
+// The mean loss of the step just synchronised with (report_step).
+void read_loss(const gl_map* m, int V, float* out_loss)
 {
-    if (!out_loss) return GL_OK;
-    if (copy) GL_CUDA_TRY(cudaMemcpyAsync(m->h_loss, m->loss_dev.p, 4 * (size_t)V, cudaMemcpyDeviceToHost, m->stream));
-    GL_CUDA_TRY(cudaStreamSynchronize(m->stream));
+    if (!out_loss) return;
     double sum = 0.0;
     for (int i = 0; i < V; i++) sum += m->h_loss[i];
     *out_loss = (float)(sum / V);
-    return GL_OK;
 }
 
 // Everything a captured step bakes in: its shape, the execution knobs and
@@ -1321,7 +1318,7 @@ gl_status run_step(gl_map* m, StepPlan& sp, float* out_loss)
         GL_CUDA_TRY(cudaStreamSynchronize(m->stream));
         GL_TRY(sort_wait_status(v, m->stream));
         if (v.h_count[1] == 0) {
-            if (out_loss) GL_TRY(read_loss(m, sp.V, false, out_loss));
+            read_loss(m, sp.V, out_loss);
             return GL_OK;
         }
         // the instances outgrew the buffers: the replay updated nothing; run
@@ -1334,8 +1331,8 @@ gl_status run_step(gl_map* m, StepPlan& sp, float* out_loss)
         m->timed_steps++;
         m->timed_views += sp.V;
     }
-    GL_TRY(read_loss(m, sp.V, true, out_loss));
     GL_CUDA_TRY(cudaStreamSynchronize(m->stream));
+    read_loss(m, sp.V, out_loss);
     GL_TRY(sort_wait_status(v, m->stream));
     if (graphs) capture_step(m, sp);
     return GL_OK;
@@ -1405,8 +1402,10 @@ extern "C" gl_status gl_map_get_exposure(gl_map* m, int64_t id, float* E34_out)
     gl_status st;
     Keyframe* kf = get_kf(m, id, false, &st);
     if (!kf) return st;
-    GL_CUDA_TRY(cudaMemcpyAsync(E34_out, kf->expo.p, 48, cudaMemcpyDeviceToHost, m->stream));
+    // through pinned memory: a copy to pageable memory is staged by the driver
+    GL_CUDA_TRY(cudaMemcpyAsync(m->h_expo, kf->expo.p, 48, cudaMemcpyDeviceToHost, m->stream));
     GL_CUDA_TRY(cudaStreamSynchronize(m->stream));
+    std::memcpy(E34_out, m->h_expo, 48);
     return GL_OK;
 }
 

@@ -254,7 +254,8 @@ struct gl_ctx_impl {
 // capacity set the overflow flag (count[1]), every later kernel of the step
 // sees zero instances, and the Adam updates skip themselves; the caller
 // checks the flag after the step.  Used for steps captured in a CUDA graph.
-// grad: a backward follows, the rows of g2d are cleared along the way.
+// grad: a step's backward follows: the rows of g2d are cleared along the way,
+// and the counters reach the host with report_step.
 gl_status bin_views(View& v, const GParams& p, const Cam* cams, const ViewExtra* extra, int V, int Ts,
                     cudaStream_t s, bool sync_free = false, bool grad = false);
 // The single-view case.
@@ -335,6 +336,9 @@ gl_status radix_sort_u32(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
                          const uint64_t* n_dev, int64_t n_max, int64_t n_reserve, int bits, uint32_t* counts,
                          DevBuf& scratch, uint64_t* ctl, uint32_t** out_k, uint32_t** out_v, cudaStream_t s,
                          bool index_values = false, uint64_t* n_kept = nullptr);
+// What the host reads of a step, written to pinned host memory by one kernel:
+// the views' losses and the counters of kCountCopy.
+gl_status report_step(const View& v, const float* loss_dev, float* h_loss, cudaStream_t s);
 // Bytes of the counters copied to View::h_count (count[0..8]).
 constexpr size_t kCountCopy = 9 * sizeof(uint64_t);
 // GL_ERR_TIMEOUT (once) if a radix-sort pass gave up a look-back wait, as
