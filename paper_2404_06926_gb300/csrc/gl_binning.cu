@@ -22,7 +22,8 @@ namespace {
 constexpr int kPreThreads = 256;
 constexpr int kScanItems = 4;
 constexpr int kScanBlock = kPreThreads * kScanItems;   // 1024 Gaussians per scan block
-constexpr int kDupChunk = 4096;   // instances one duplication CTA writes at most
+constexpr int kDupChunk = 2048;   // instances one duplication CTA writes at most (4096: 14.0 -> 10.8 us, 250k Gaussians;
+                                  // 26.8 -> 23.7, 1M; 453 -> 458, 12 views of 2M)
 
 // Block-wide exclusive scan (NT threads); returns the exclusive prefix and
 // writes the block total to *total.  `sm` needs NT/32 + 1 entries.
@@ -78,7 +79,9 @@ struct PreClear {
 };
 
 template <int DEG>
-__global__ void __launch_bounds__(kPreThreads)
+// (four CTAs per SM: 66.8 -> 63.9 us on 1M Gaussians, 1,367 -> 1,278 us on 12
+// views of 2M)
+__global__ void __launch_bounds__(kPreThreads, 4)
 k_preprocess(GParams p, const ViewDesc* __restrict__ views, int V, int Ts, bool cull,
              float4* __restrict__ rec, int* __restrict__ radius, uint4* __restrict__ brec,
              uint32_t* __restrict__ touched, uint32_t* __restrict__ dkey, uint64_t* __restrict__ ctl, PreClear clr)
@@ -231,6 +234,12 @@ __global__ void k_set_u64(uint64_t* p, uint64_t v0, uint64_t v1)
 constexpr int kOsThreads = 256;
 constexpr int kOsItems = 15;
 constexpr int kOsTile = kOsThreads * kOsItems;   // 3840 keys per tile
+// Up to kOsSmall keys a tile holds 2048 and a histogram thread 8: with a tile
+// per SM or less, a pass takes as long as one CTA does.  Six passes, tiles of
+// 2048 and 3840 keys: 42.6 and 50.7 us (250k Gaussians), 56 and 60 (500k), 79
+// and 78 (1M), 1,079 and 841 (12 views of 2M).
+constexpr int kOsItemsSmall = 8;
+constexpr int64_t kOsSmall = 800000;
 constexpr int kOsMaxPasses = 4;
 constexpr int kOsTicketOff = kOsMaxPasses * 256;
 static_assert(kOsTicketOff + 64 == kSortCountWords, "layout of the counts");
@@ -252,12 +261,13 @@ __device__ __forceinline__ void st_relaxed_gpu(uint32_t* p, uint32_t v)
 
 // Digit counts of all passes (counts and counters zeroed before) and
 // clearing of the look-back words of the tiles (tile_keys keys each) this
-// sort visits.  A thread loads kOsHistKeys keys before counting any of them.
+// sort visits.  A thread loads HK keys before counting any of them.
 // With n_kept (zeroed before), keys 0xffffffff are left out of the counts and
 // the number of the other keys is added to *n_kept.  For 32-bit keys the top
 // digit takes few values (float keys of one range), so equal top digits of a
 // warp are counted with one shared atomic.
-constexpr int kOsHistKeys = 16;
+constexpr int kOsHistKeys = 16, kOsHistKeysSmall = 8;
+template <int HK>
 __global__ void __launch_bounds__(kOsThreads)
 k_os_hist(const uint32_t* __restrict__ kin, const uint64_t* n_dev, int passes, int tile_keys,
           int64_t tiles_max, uint32_t* __restrict__ counts, uint32_t* __restrict__ status,
@@ -278,10 +288,10 @@ k_os_hist(const uint32_t* __restrict__ kin, const uint64_t* n_dev, int passes, i
         for (uint64_t i = gid; i < nt * 256; i += gsz) status[(uint64_t)p * tiles_max * 256 + i] = 0u;
     __syncthreads();
     // key j of a thread: b + (j / 4 * kOsThreads + threadIdx.x) * 4 + j % 4 (16-byte loads)
-    for (uint64_t b = (uint64_t)blockIdx.x * kOsThreads * kOsHistKeys; b < n; b += gsz * kOsHistKeys) {
-        uint32_t k[kOsHistKeys];
+    for (uint64_t b = (uint64_t)blockIdx.x * kOsThreads * HK; b < n; b += gsz * HK) {
+        uint32_t k[HK];
 #pragma unroll
-        for (int q = 0; q < kOsHistKeys / 4; q++) {
+        for (int q = 0; q < HK / 4; q++) {
             const uint64_t i0 = b + ((uint64_t)q * kOsThreads + threadIdx.x) * 4;
             if (i0 + 3 < n) {
                 const uint4 v = *reinterpret_cast<const uint4*>(kin + i0);
@@ -292,7 +302,7 @@ k_os_hist(const uint32_t* __restrict__ kin, const uint64_t* n_dev, int passes, i
             }
         }
 #pragma unroll
-        for (int j = 0; j < kOsHistKeys; j++) {
+        for (int j = 0; j < HK; j++) {
             const bool ok = b + ((uint64_t)(j / 4) * kOsThreads + threadIdx.x) * 4 + (j % 4) < n;
             const bool use = ok && !(drop && k[j] == 0xffffffffu);
             kept += use;
@@ -928,24 +938,27 @@ gl_status radix_sort_u32(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
         set_error("radix sort: 2^30 keys or more");
         return GL_ERR_CAPACITY;
     }
-    const int64_t tiles_max = (nbig + kOsTile - 1) / kOsTile;
+    const bool small = nbig <= kOsSmall;
+    const int tile_keys = kOsThreads * (small ? kOsItemsSmall : kOsItems);
+    const int hist_keys = kOsThreads * (small ? kOsHistKeysSmall : kOsHistKeys);
+    const int64_t tiles_max = (nbig + tile_keys - 1) / tile_keys;
     GL_TRY(scratch.reserve(sizeof(uint32_t) * (size_t)kOsMaxPasses * tiles_max * 256));
     uint32_t* sc = scratch.as<uint32_t>();
-    const int tile_keys = kOsTile;
     const int64_t tiles = std::max<int64_t>(1, (n_max + tile_keys - 1) / tile_keys);
     const int hblocks = (int)std::min<int64_t>(
-        4 * (int64_t)sm_count(), std::max<int64_t>(1, (n_max + kOsThreads * kOsHistKeys - 1) / (kOsThreads * kOsHistKeys)));
+        4 * (int64_t)sm_count(), std::max<int64_t>(1, (n_max + hist_keys - 1) / hist_keys));
     unsigned long long* kept = reinterpret_cast<unsigned long long*>(n_kept);
-    k_os_hist<<<hblocks, kOsThreads, 0, s>>>(k0, n_dev, passes, tile_keys, tiles_max, counts, sc, kept);
+    const auto hist = small ? k_os_hist<kOsHistKeysSmall> : k_os_hist<kOsHistKeys>;
+    hist<<<hblocks, kOsThreads, 0, s>>>(k0, n_dev, passes, tile_keys, tiles_max, counts, sc, kept);
     uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
     unsigned long long* err = reinterpret_cast<unsigned long long*>(ctl + 8);
     for (int p = 0; p < passes; p++) {
         const uint32_t* vsrc = (p == 0 && index_values) ? nullptr : vi;
         // the first pass drops the 0xffffffff keys; the later ones sort the rest
         const uint64_t* np = (p > 0 && n_kept) ? n_kept : n_dev;
-        k_os_pass<kOsThreads, kOsItems, 3><<<(unsigned)tiles, kOsThreads, 0, s>>>(ki, vsrc, ko, vo, np, p,
-                                                                                  tiles_max, counts, sc, err,
-                                                                                  p == 0 && n_kept);
+        const auto pass = small ? k_os_pass<kOsThreads, kOsItemsSmall, 3> : k_os_pass<kOsThreads, kOsItems, 3>;
+        pass<<<(unsigned)tiles, kOsThreads, 0, s>>>(ki, vsrc, ko, vo, np, p, tiles_max, counts, sc, err,
+                                                    p == 0 && n_kept);
         std::swap(ki, ko);
         std::swap(vi, vo);
     }
