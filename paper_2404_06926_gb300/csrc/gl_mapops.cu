@@ -27,7 +27,7 @@ namespace gl {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kItems = 4;
+constexpr int kItems = 1;   // points per thread of the expansion
 constexpr int kBlock = kThreads * kItems;
 
 __device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t i)
@@ -229,44 +229,54 @@ __global__ void __launch_bounds__(1024) k_expand_scan(uint64_t* bsum, int nb, ui
     if (threadIdx.x == 1023) *total = sm[1023];
 }
 
+// The kept points' rows.  A CTA's kept points are consecutive rows of the map:
+// they are compacted in shared memory and every array is written element by
+// element, coalesced (a point's SH row alone is 192 bytes at degree 3).  Bound
+// by latency.  Four points a thread, each writing its rows: 19.8 -> 12.5 us
+// (60k points offered, degree 3).
 __global__ void __launch_bounds__(kThreads)
 k_expand_emit(const float* __restrict__ xyz, const float* __restrict__ rgb, int64_t n,
               const uint32_t* __restrict__ flag, const float* __restrict__ depth,
               const uint64_t* __restrict__ bsum, float fx, float logit, int K, GMut dst,
               int64_t off0, int64_t cap)
 {
-    __shared__ uint64_t sm[kThreads];
-    const int64_t base = (int64_t)blockIdx.x * kBlock + threadIdx.x * kItems;
-    uint64_t c = 0;
-    for (int k = 0; k < kItems; k++)
-        if (base + k < n) c += flag[base + k];
-    sm[threadIdx.x] = c;
+    static_assert(kBlock == kThreads, "a point per thread");
+    __shared__ int src[kThreads];        // kept points, in order
+    __shared__ float ls[kThreads];
+    __shared__ int wsum[kThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int64_t i = (int64_t)blockIdx.x * kBlock + tid;
+    const bool keep = i < n && flag[i] != 0u;
+    const unsigned m = __ballot_sync(kFull, keep);
+    if (lane == 0) wsum[w] = __popc(m);
     __syncthreads();
-    for (int off = 1; off < kThreads; off <<= 1) {
-        uint64_t v = threadIdx.x >= off ? sm[threadIdx.x - off] : 0;
-        __syncthreads();
-        sm[threadIdx.x] += v;
-        __syncthreads();
+    int at = __popc(m & ((1u << lane) - 1u)), cnt = 0;
+#pragma unroll
+    for (int v = 0; v < kThreads / 32; v++) {
+        if (v < w) at += wsum[v];
+        cnt += wsum[v];
     }
-    uint64_t pos = bsum[blockIdx.x] + sm[threadIdx.x] - c;
-    for (int k = 0; k < kItems; k++) {
-        const int64_t i = base + k;
-        if (i >= n) break;
-        if (!flag[i]) continue;
-        const int64_t g = off0 + (int64_t)pos++;
-        if (g >= cap) continue;
-        dst.means[3 * g] = xyz[3 * i];
-        dst.means[3 * g + 1] = xyz[3 * i + 1];
-        dst.means[3 * g + 2] = xyz[3 * i + 2];
-        const float ls = logf(depth[i] / fx);
-        dst.log_scales[3 * g] = ls; dst.log_scales[3 * g + 1] = ls; dst.log_scales[3 * g + 2] = ls;
-        reinterpret_cast<float4*>(dst.quats)[g] = make_float4(1.f, 0.f, 0.f, 0.f);
-        dst.logits[g] = logit;
-        float* s = dst.sh + (size_t)g * K * 3;
-        s[0] = (rgb[3 * i] - 0.5f) / kSH0;
-        s[1] = (rgb[3 * i + 1] - 0.5f) / kSH0;
-        s[2] = (rgb[3 * i + 2] - 0.5f) / kSH0;
-        for (int k2 = 3; k2 < K * 3; k2++) s[k2] = 0.0f;
+    if (keep) {
+        src[at] = tid;
+        ls[at] = logf(depth[i] / fx);
+    }
+    __syncthreads();
+    const int64_t g0 = off0 + (int64_t)bsum[blockIdx.x];
+    cnt = (int)min((int64_t)cnt, max((int64_t)0, cap - g0));
+    const int64_t p0 = (int64_t)blockIdx.x * kBlock;
+    for (int e = tid; e < 3 * cnt; e += kThreads) {
+        dst.means[3 * g0 + e] = xyz[3 * (p0 + src[e / 3]) + e % 3];
+        dst.log_scales[3 * g0 + e] = ls[e / 3];
+    }
+    for (int e = tid; e < cnt; e += kThreads) {
+        reinterpret_cast<float4*>(dst.quats)[g0 + e] = make_float4(1.f, 0.f, 0.f, 0.f);
+        dst.logits[g0 + e] = logit;
+    }
+    const int row = 3 * K;
+    float* sh = dst.sh + (size_t)g0 * row;
+    for (int e = tid; e < cnt * row; e += kThreads) {
+        const int r = e / row, c = e - r * row;
+        sh[e] = c < 3 ? (rgb[3 * (p0 + src[r]) + c] - 0.5f) / kSH0 : 0.0f;
     }
 }
 

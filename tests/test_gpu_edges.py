@@ -215,3 +215,50 @@ def test_backward_with_more_blocks_than_warps(n, seg, extra):
         a, ref = gg[name].cpu().numpy().astype(np.float64)[vis].ravel(), np.asarray(g[name], np.float64)[vis].ravel()
         rel = np.abs(a - ref) / np.maximum(np.abs(ref), 1e-4 * np.abs(ref).max())
         assert np.median(rel) < 1e-3 and np.percentile(rel, 99) < 1e-2, (name, np.median(rel), np.percentile(rel, 99))
+
+
+@pytest.mark.parametrize("n", [2047, 2048, 2049, 6145, 799_999, 800_001])   # a tile's keys; the smaller tiles' last count
+def test_sort_tile_sizes(n):
+    """Binning of n Gaussians of one tile each: instances in (tile, depth, index) order."""
+    from paper_2404_06926_gb300 import binding
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    cam = scenes.camera(640, 480, 500.0, 500.0, 320.0, 240.0)
+    z = torch.rand(n, generator=g, device="cuda") * 2 + 1
+    uv = torch.rand(n, 2, generator=g, device="cuda")
+    means = torch.stack([(uv[:, 0] * 600 + 20 - 320) / 500 * z, (uv[:, 1] * 440 + 20 - 240) / 500 * z, z], 1).contiguous()
+    q = torch.zeros(n, 4, device="cuda")
+    q[:, 0] = 1
+    p = dict(means=means, log_scales=torch.full((n, 3), -9.0, device="cuda"), quats=q,
+             logits=torch.full((n,), 2.0, device="cuda"), sh=torch.zeros(n, 1, 3, device="cuda"))
+    ctx = binding.Ctx()
+    ctx.forward(p, cam, 16)
+    keys, vals, ranges = ctx.instances(40 * 30, "cuda")
+    assert len(keys) >= n
+    same = keys[1:] == keys[:-1]
+    assert bool((keys[1:] >= keys[:-1]).all()) and bool((vals[1:][same] > vals[:-1][same]).all())
+    assert int(torch.unique(vals).numel()) == n
+    assert torch.equal(ranges[:, 1] - ranges[:, 0], torch.bincount(keys >> 32, minlength=1200).int())
+
+
+@pytest.mark.parametrize("n", [1, 255, 256, 257, 1000])
+@pytest.mark.parametrize("deg", [0, 3])
+def test_expanded_rows(n, deg):
+    """Points in front of the camera become rows in order, the others none."""
+    from paper_2404_06926_gb300 import binding
+    rng = np.random.default_rng(n)
+    cam = scenes.camera(64, 48, 50.0, 50.0, 32.0, 24.0)
+    xyz = rng.normal(0, 2, (n, 3)).astype(np.float32)
+    rgb = rng.uniform(0, 1, (n, 3)).astype(np.float32)
+    m = binding.Map(binding.default_config(n_sky=0, sh_degree=deg, capacity_hint=16))
+    added = m.add_points(torch.from_numpy(xyz).cuda(), torch.from_numpy(rgb).cuda(), cam, use_mask=False)
+    keep = xyz[:, 2] > np.float32(0.2)
+    assert added == keep.sum() == len(m)
+    if added == 0:
+        return
+    out = {k: torch.as_tensor(v).cpu().numpy() for k, v in m.get_params().items()}
+    assert np.array_equal(out["means"], xyz[keep])
+    assert np.allclose(out["log_scales"], np.log(xyz[keep, 2:] / 50.0), atol=1e-6)
+    assert np.allclose(out["sh"][:, 0], (rgb[keep] - 0.5) / 0.28209479177387814, atol=1e-6)
+    assert not out["sh"][:, 1:].any()
+    assert np.array_equal(out["quats"], np.tile(np.float32([1, 0, 0, 0]), (added, 1)))
