@@ -760,24 +760,28 @@ __device__ __forceinline__ void bwd_turn_over(const RasterArgs& A, const RasterG
     const float2* row = W.sv + h * BW::S + part * BW::PS;
     const float4* pc = W.pix + part * 16;
     const float dya = in.y - (by + (float)(2 * part)), dyb = in.y - (by + (float)(2 * part + 1));
-    float c0 = 0.f, c1 = 0.f, c2 = 0.f, cD = 0.f;
-    float m0a = 0.f, m0b = 0.f, mxa = 0.f, mxb = 0.f, mxx = 0.f;
+    // even and odd columns apart: chains of four terms, then pairs of sums, which
+    // round no worse than a fold of the pixels' terms
+    float c0[2] = {0.f, 0.f}, c1[2] = {0.f, 0.f}, c2[2] = {0.f, 0.f}, cD[2] = {0.f, 0.f}, mxx[2] = {0.f, 0.f};
+    float m0a[2] = {0.f, 0.f}, m0b[2] = {0.f, 0.f}, mxa[2] = {0.f, 0.f}, mxb[2] = {0.f, 0.f};
 #pragma unroll
     for (int x = 0; x < 8; x++) {
+        const int e = x & 1;
         const float2 va = row[x], vb = row[8 + x];
         const float4 ga = pc[x], gb = pc[8 + x];
         const float dx = in.x - (bx + (float)x), dx2 = dx * dx;
-        c0 = fmaf(va.x, ga.x, c0); c1 = fmaf(va.x, ga.y, c1); c2 = fmaf(va.x, ga.z, c2);
-        c0 = fmaf(vb.x, gb.x, c0); c1 = fmaf(vb.x, gb.y, c1); c2 = fmaf(vb.x, gb.z, c2);
-        if (EXTRA) cD = fmaf(vb.x, gb.w, fmaf(va.x, ga.w, cD));
-        m0a += va.y; m0b += vb.y;
-        mxa = fmaf(va.y, dx, mxa); mxb = fmaf(vb.y, dx, mxb);
-        mxx = fmaf(vb.y, dx2, fmaf(va.y, dx2, mxx));
+        c0[e] = fmaf(va.x, ga.x, c0[e]); c1[e] = fmaf(va.x, ga.y, c1[e]); c2[e] = fmaf(va.x, ga.z, c2[e]);
+        c0[e] = fmaf(vb.x, gb.x, c0[e]); c1[e] = fmaf(vb.x, gb.y, c1[e]); c2[e] = fmaf(vb.x, gb.z, c2[e]);
+        if (EXTRA) cD[e] = fmaf(vb.x, gb.w, fmaf(va.x, ga.w, cD[e]));
+        m0a[e] += va.y; m0b[e] += vb.y;
+        mxa[e] = fmaf(va.y, dx, mxa[e]); mxb[e] = fmaf(vb.y, dx, mxb[e]);
+        mxx[e] = fmaf(vb.y, dx2, fmaf(va.y, dx2, mxx[e]));
     }
+    const float ma = m0a[0] + m0a[1], mb = m0b[0] + m0b[1], xa = mxa[0] + mxa[1], xb = mxb[0] + mxb[1];
     // slots 0-3 (lo), 4-7 (hi), 8-9
-    float lo[4] = {c0, c1, c2, m0a + m0b};
-    float hi[4] = {mxa + mxb, fmaf(dya, m0a, dyb * m0b), mxx, fmaf(dya, mxa, dyb * mxb)};
-    float s8 = fmaf(dya * dya, m0a, dyb * dyb * m0b), s9 = cD;
+    float lo[4] = {c0[0] + c0[1], c1[0] + c1[1], c2[0] + c2[1], ma + mb};
+    float hi[4] = {xa + xb, fmaf(dya, ma, dyb * mb), mxx[0] + mxx[1], fmaf(dya, xa, dyb * xb)};
+    float s8 = fmaf(dya * dya, ma, dyb * dyb * mb), s9 = cD[0] + cD[1];
 #pragma unroll
     for (int off = H; off < 16; off <<= 1) {
 #pragma unroll
@@ -1054,20 +1058,22 @@ __device__ __forceinline__ void half_turn_over(const RasterGrad& G, const BwdHal
     const float4 a = R.r0[at + (lane & 15)];
     const float2* row = W.sv + lane * BwdHalf::S;
     const float4* pc = W.pix + half * 16;
-    float c0 = 0.f, c1 = 0.f, c2 = 0.f, cD = 0.f, mxx = 0.f;
+    // chains of four to eight terms, then pairs of sums
+    float c0[2] = {0.f, 0.f}, c1[2] = {0.f, 0.f}, c2[2] = {0.f, 0.f}, cD[2] = {0.f, 0.f}, mxx[2] = {0.f, 0.f};
     float m0[4] = {0.f, 0.f, 0.f, 0.f}, mx[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int x = 0; x < 4; x++) {
         const float dx = a.x - (bx + (float)x), dx2 = dx * dx;
 #pragma unroll
         for (int y = 0; y < 4; y++) {
+            const int e = y & 1;
             const float2 v = row[y * 4 + x];
             const float4 g = pc[y * 4 + x];
-            c0 = fmaf(v.x, g.x, c0); c1 = fmaf(v.x, g.y, c1); c2 = fmaf(v.x, g.z, c2);
-            if (EXTRA) cD = fmaf(v.x, g.w, cD);
+            c0[e] = fmaf(v.x, g.x, c0[e]); c1[e] = fmaf(v.x, g.y, c1[e]); c2[e] = fmaf(v.x, g.z, c2[e]);
+            if (EXTRA) cD[e] = fmaf(v.x, g.w, cD[e]);
             m0[y] += v.y;
             mx[y] = fmaf(v.y, dx, mx[y]);
-            mxx = fmaf(v.y, dx2, mxx);
+            mxx[e] = fmaf(v.y, dx2, mxx[e]);
         }
     }
     float gy = 0.f, gxy = 0.f, gyy = 0.f;
@@ -1081,9 +1087,10 @@ __device__ __forceinline__ void half_turn_over(const RasterGrad& G, const BwdHal
     if (on) {
         const uint32_t id = __float_as_uint(R.r1[at + (lane & 15)].w);
         float* dst = G.g2d + (size_t)id * kGradStride;
-        atomicAdd(reinterpret_cast<float4*>(dst), make_float4(c0, c1, c2, (m0[0] + m0[1]) + (m0[2] + m0[3])));
-        atomicAdd(reinterpret_cast<float4*>(dst + 4), make_float4((mx[0] + mx[1]) + (mx[2] + mx[3]), gy, mxx, gxy));
-        if (EXTRA) atomicAdd(reinterpret_cast<float2*>(dst + 8), make_float2(gyy, cD));
+        atomicAdd(reinterpret_cast<float4*>(dst), make_float4(c0[0] + c0[1], c1[0] + c1[1], c2[0] + c2[1],
+                                                                (m0[0] + m0[1]) + (m0[2] + m0[3])));
+        atomicAdd(reinterpret_cast<float4*>(dst + 4), make_float4((mx[0] + mx[1]) + (mx[2] + mx[3]), gy, mxx[0] + mxx[1], gxy));
+        if (EXTRA) atomicAdd(reinterpret_cast<float2*>(dst + 8), make_float2(gyy, cD[0] + cD[1]));
         else atomicAdd(dst + 8, gyy);
     }
 }
@@ -1785,7 +1792,7 @@ void bwd_pg_launch(const RasterArgs& A, const RasterGrad& G, int64_t units, bool
 
 template <bool EXTRA>
 void bwd_dispatch(int nb, int pd, bool det, bool pg, const RasterArgs& A, const RasterGrad& G, int64_t units,
-                  bool persistent, cudaStream_t s)
+                  int64_t blocks, bool persistent, cudaStream_t s)
 {
     if (pg) {    // per-Gaussian: batch depth 32, one pixel per lane
         if (det) bwd_pg_launch<EXTRA, true>(A, G, units, persistent, s);
@@ -1794,7 +1801,7 @@ void bwd_dispatch(int nb, int pd, bool det, bool pg, const RasterArgs& A, const 
         if (pd == 1) bwd_launch<EXTRA, 1, 1, true>(A, G, units, persistent, s);
         else if (pd == 2) bwd_launch<EXTRA, 1, 2, true>(A, G, units, persistent, s);
         else bwd_launch<EXTRA, 1, 4, true>(A, G, units, persistent, s);
-    } else if (pd == 1 && units >= (int64_t)kMinBlocksHalf * kWpbHalf * sm_count()) {
+    } else if (pd == 1 && blocks >= (int64_t)kMinBlocksHalf * kWpbHalf * sm_count()) {
         // more pixel blocks than resident warps.  Below, a warp has one block
         // and its chain is the time, which the two lists lengthen: 17.8 -> 22.4
         // us on 5k Gaussians at 256x192 (1.5k blocks; the line lies at 3.0k).
@@ -1924,11 +1931,12 @@ gl_status raster_backward(View& v, const float* dL_drgb, const float* dL_ddepth,
         G.part = v.gpart.as<float>();
         G.pmask = v.gmask.as<uint32_t>();
     }
-    const int64_t units = work_items_bound(v) * nblk;
+    // pixel blocks, and the bound on units (a split tile's blocks count once per segment)
+    const int64_t blocks = (int64_t)v.ntiles * nblk, units = work_items_bound(v) * nblk;
     if (dL_ddepth != nullptr || dL_dopac != nullptr)
-        bwd_dispatch<true>(v.nb, v.pd, det, v.pg, A, G, units, v.persistent, s);
+        bwd_dispatch<true>(v.nb, v.pd, det, v.pg, A, G, units, blocks, v.persistent, s);
     else
-        bwd_dispatch<false>(v.nb, v.pd, det, v.pg, A, G, units, v.persistent, s);
+        bwd_dispatch<false>(v.nb, v.pd, det, v.pg, A, G, units, blocks, v.persistent, s);
     count_launches(1);
     if (det) {
         const int blocks = (int)std::min<size_t>(8 * (size_t)sm_count(), (pairs + 31) / 32);
