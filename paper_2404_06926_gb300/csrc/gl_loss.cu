@@ -136,7 +136,7 @@ loss_tile(LossOne one, const ViewDesc* __restrict__ views, int V, const float* _
     float2* hab = hm;                                              // RB rows x HS (reuses hm)
     float* hc = reinterpret_cast<float*>(hab + RB * HS);           // RB rows x HS
     __shared__ float red[kNP][kThreads / 32];
-    __shared__ float chsum[3][2];    // in CTA 0 of the cluster: the channels' sums of |.| and SSIM
+    __shared__ float chsum[2];       // SPLIT: the channel's sums of |.| and SSIM
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int LTX = (W + LT - 1) / LT;
     const int ox = (lt % LTX) * LT, oy = (lt / LTX) * LT;
@@ -361,8 +361,11 @@ loss_tile(LossOne one, const ViewDesc* __restrict__ views, int V, const float* _
             float v = 0.0f;
             for (int ww = 0; ww < kThreads / 32; ww++) v += red[k][ww];
             if (tid < 4) prow[k] = v;
-            else cluster.map_shared_rank(&chsum[0][0], 0)[2 * ch + tid - 4] = v;
+            else chsum[tid - 4] = v;
         }
+        // a CTA's shared memory may be touched from another one only once all
+        // are known to run: sums and gradients are left at home and read after
+        // this barrier
         cluster.sync();
         // component ch of dL/dC = sum over channels k of A[k][ch] dL/dE[C]_k
         const float f0 = E ? E[ch] : (ch == 0 ? 1.0f : 0.0f), f1 = E ? E[4 + ch] : (ch == 1 ? 1.0f : 0.0f);
@@ -376,7 +379,8 @@ loss_tile(LossOne one, const ViewDesc* __restrict__ views, int V, const float* _
             const float v = fmaf(f2, g2[i], fmaf(f1, g1[i], f0 * g0[i]));
             if (gx < W && gy < H) dL_drgb[3 * ((size_t)gy * W + gx) + ch] = v;
         }
-        if (ch == 0 && tid < 2) prow[12 + tid] = chsum[0][tid] + chsum[1][tid] + chsum[2][tid];
+        if (ch == 0 && tid < 2)
+            prow[12 + tid] = chsum[tid] + cluster.map_shared_rank(chsum, 1)[tid] + cluster.map_shared_rank(chsum, 2)[tid];
         cluster.sync();   // the shared memory read by the other CTAs stays until they are done
     } else {
         if (tid < kNP) {
