@@ -627,7 +627,9 @@ struct Jac6 {
 // Sum of the blocks' pose partials in a fixed order (float pairs, df_acc),
 // then J^T g.  One cluster of eight CTAs: thread t of CTA c takes elements
 // 1020 c + t, + 8160, ... (1020 = 170 x 6: always the same component), eight
-// loads in flight; CTA 0 adds the eight CTAs' sums.  Bound by latency.
+// loads in flight; CTA 0 reads and adds the eight CTAs' sums between two
+// cluster barriers (the first shows that all CTAs run, the second keeps their
+// shared memory until it has been read).  Bound by latency.
 // One CTA in double -> this: 34.9 -> 3.5 us (250k Gaussians).
 constexpr int kPoseRows = 170;
 constexpr int kPoseThreads = 1024;
@@ -638,7 +640,7 @@ k_pose_reduce(const float* __restrict__ part, int npart, Jac6 J, float* __restri
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     __shared__ float2 sums[kPoseRows * 6];
-    __shared__ float2 ctas[kPoseCtas][6];   // in CTA 0: every CTA's sums
+    __shared__ float2 mine[6];   // this CTA's sums
     __shared__ double gsum[6];
     const int tid = threadIdx.x;
     constexpr int PER = kPoseRows * 6, STRIDE = PER * kPoseCtas;
@@ -671,20 +673,23 @@ k_pose_reduce(const float* __restrict__ part, int npart, Jac6 J, float* __restri
             df_acc(h, l, oh);
             l += ol;
         }
-        if (lane == 0) cluster.map_shared_rank(&ctas[0][0], 0)[blockIdx.x * 6 + k] = make_float2(h, l);
+        if (lane == 0) mine[k] = make_float2(h, l);
     }
     cluster.sync();
-    if (blockIdx.x != 0) return;
-    if (tid < 6) {
+    if (blockIdx.x == 0 && tid < 6) {
+        float2 v[kPoseCtas];
+#pragma unroll
+        for (int c = 0; c < kPoseCtas; c++) v[c] = cluster.map_shared_rank(mine, c)[tid];
         float h = 0.0f, l = 0.0f;
+#pragma unroll
         for (int c = 0; c < kPoseCtas; c++) {
-            df_acc(h, l, ctas[c][tid].x);
-            l += ctas[c][tid].y;
+            df_acc(h, l, v[c].x);
+            l += v[c].y;
         }
         gsum[tid] = df_value(h, l);
     }
-    __syncthreads();
-    if (tid < 6) {
+    cluster.sync();
+    if (blockIdx.x == 0 && tid < 6) {
         double o = 0.0;
         for (int i = 0; i < 6; i++) o += (double)J.m[i * 6 + tid] * gsum[i];
         out6[tid] = (float)o;

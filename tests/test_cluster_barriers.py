@@ -10,7 +10,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2404_06926_gb300", "csrc")
 
 
-@pytest.mark.parametrize("name", ["gl_loss.cu"])
+@pytest.mark.parametrize("name", ["gl_loss.cu", "gl_params.cu"])
 def test_remote_shared_memory_lies_between_barriers(name):
     src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
     # a kernel's accesses follow the cluster_group it declares
