@@ -234,11 +234,11 @@ def set_exec(m, mode, views, keep_tile, window=None):
     knobs, or graphs with the autotuner's pick for the window `views`;
     explicit --knobs replace the autotuner."""
     if mode == "eager":
-        m.set_exec(use_graphs=0, persistent=0, batch_depth=32, pixels_per_lane=1, tile_size=0, segment=0)
+        m.set_exec(use_graphs=0, persistent=0, batch_depth=32, pixels_per_lane=1, tile_size=0, segment=-1)
         m.set_exec(**KNOBS)
         return m.get_exec(), None
     if mode == "graphs" or KNOBS:
-        m.set_exec(use_graphs=1, persistent=0, batch_depth=32, pixels_per_lane=1, tile_size=0, segment=0)
+        m.set_exec(use_graphs=1, persistent=0, batch_depth=32, pixels_per_lane=1, tile_size=0, segment=-1)
         m.set_exec(**KNOBS)
         return m.get_exec(), None
     best, ms = m.autotune(views, reps=3, keep_tile_size=keep_tile, window=window)

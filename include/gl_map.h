@@ -223,12 +223,17 @@ GL_API gl_status gl_optimize_step(gl_map* map, const gl_keyframe* views, int32_t
  *                    tile, with a 2^-7 slack); renders are bit-identical
  *                    either way, the instance lists (and contributor
  *                    positions) shorter.
- *   segment          0, or a power of two in 64..65536: a tile whose list
- *                    holds at least 2 x segment Gaussians is rendered and
- *                    back-propagated as segments of `segment` consecutive
- *                    Gaussians by separate warps; the transmittance is then
- *                    a product of per-segment products, equal to the
- *                    single running product up to float rounding.
+ *   segment          -1 (default), 0, or a power of two in 64..65536: a tile
+ *                    whose list holds at least 2 x segment Gaussians is
+ *                    rendered and back-propagated as segments of `segment`
+ *                    consecutive Gaussians by separate warps; the
+ *                    transmittance is then a product of products over
+ *                    consecutive parts of the list, equal to the single
+ *                    running product up to float rounding, and the parts'
+ *                    state takes up to 12288 / segment bytes per instance
+ *                    (16 x 16 tiles).  0: no list is split.  -1: the
+ *                    library's choice: segments of 512, and whole lists
+ *                    where the state finds no memory.
  *   per_gaussian     1: per-Gaussian backward (Sec. III-D 1): each lane
  *                    of a warp owns Gaussians of the pixel block's list and
  *                    sums their gradients in its registers while the
@@ -240,7 +245,7 @@ GL_API gl_status gl_optimize_step(gl_map* map, const gl_keyframe* views, int32_t
  *                    batch_depth say (those still drive the forward).
  * Apart from deterministic = 1, results differ between runs only by the
  * order of the backward's float atomics.
- * gl_map_create starts with {0, 0, 32, 1, 0, 0, 0, 1, 0}.  Errors: GL_ERR_INVALID. */
+ * gl_map_create starts with {0, 0, 32, 1, 0, 0, -1, 1, 0}.  Errors: GL_ERR_INVALID. */
 typedef struct {
     int32_t use_graphs;
     int32_t persistent;
@@ -480,7 +485,7 @@ GL_API gl_status gl_ctx_destroy(gl_ctx* ctx);
 
 /* Raster execution of this context's calls: batch_depth, pixels_per_lane,
  * persistent, deterministic, segment, exact_cull and per_gaussian as in
- * gl_exec_config (defaults 32, 1, 0, 0, 0, 1, 0; use_graphs
+ * gl_exec_config (defaults 32, 1, 0, 0, -1, 1, 0; use_graphs
  * and tile_size are ignored: the tile size is each call's argument).  A
  * pixels_per_lane above tile_size / 4 is lowered to it.  Errors:
  * GL_ERR_INVALID. */

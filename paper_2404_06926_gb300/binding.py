@@ -266,7 +266,7 @@ class Ctx:
         return loss, dC, dE.view(3, 4)
 
     # introspection of the last forward
-    def set_exec(self, batch_depth=32, pixels_per_lane=1, persistent=0, deterministic=0, segment=0, exact_cull=1,
+    def set_exec(self, batch_depth=32, pixels_per_lane=1, persistent=0, deterministic=0, segment=-1, exact_cull=1,
                  per_gaussian=0):
         """Raster execution of this context's calls (see gl_ctx_set_exec)."""
         e = ExecConfig(0, int(persistent), int(batch_depth), int(pixels_per_lane), 0, int(deterministic),

@@ -385,6 +385,9 @@ int batch_subs(int batch_depth, bool det)
 
 bool valid_batch_depth(int b) { return b == 32 || b == 64 || b == 128 || b == 256; }
 
+// -1: the library's choice, 0: no splitting
+bool valid_segment(int s) { return s == -1 || s == 0 || (s >= 64 && s <= 65536 && (s & (s - 1)) == 0); }
+
 bool is_device_ptr(const void* p)
 {
     if (!p) return false;
@@ -508,8 +511,8 @@ extern "C" gl_status gl_ctx_set_exec(gl_ctx* ctx, const gl_exec_config* e)
     if (!valid_batch_depth(e->batch_depth) || (e->batch_depth > 64 && e->pixels_per_lane != 1) ||
         (e->deterministic != 0 && e->deterministic != 1) ||
         (e->pixels_per_lane != 1 && e->pixels_per_lane != 2 && e->pixels_per_lane != 4) ||
-        (e->segment != 0 && (e->segment < 64 || e->segment > 65536 || (e->segment & (e->segment - 1)) != 0)) ||
-        (e->exact_cull != 0 && e->exact_cull != 1) || (e->per_gaussian != 0 && e->per_gaussian != 1)) {
+        !valid_segment(e->segment) || (e->exact_cull != 0 && e->exact_cull != 1) ||
+        (e->per_gaussian != 0 && e->per_gaussian != 1)) {
         set_error("invalid execution config");
         return GL_ERR_INVALID;
     }
@@ -688,7 +691,7 @@ struct gl_map {
     std::unordered_map<int64_t, std::unique_ptr<Keyframe>> kfs;
     Prof prof;
     // step execution and the captured step graph
-    gl_exec_config exec{0, 0, 32, 1, 0, 0, 0, 1, 0};
+    gl_exec_config exec{0, 0, 32, 1, 0, 0, -1, 1, 0};
     cudaStream_t gstream = nullptr;      // capture stream (the map's may be the legacy one)
     // caller host images of a step are copied on cstream while the step's
     // first kernels run; the loss waits for stage_ev (ready_ev: the map's
@@ -1494,8 +1497,8 @@ gl_status check_exec_config(const gl_map* m, const gl_exec_config& e)
     if (e.deterministic != 0 && e.deterministic != 1) { set_error("deterministic must be 0 or 1"); return GL_ERR_INVALID; }
     if (e.exact_cull != 0 && e.exact_cull != 1) { set_error("exact_cull must be 0 or 1"); return GL_ERR_INVALID; }
     if (e.per_gaussian != 0 && e.per_gaussian != 1) { set_error("per_gaussian must be 0 or 1"); return GL_ERR_INVALID; }
-    if (e.segment != 0 && (e.segment < 64 || e.segment > 65536 || (e.segment & (e.segment - 1)) != 0)) {
-        set_error("segment must be 0 or a power of two in 64..65536");
+    if (!valid_segment(e.segment)) {
+        set_error("segment must be -1, 0 or a power of two in 64..65536");
         return GL_ERR_INVALID;
     }
     if ((e.pixels_per_lane != 1 && e.pixels_per_lane != 2 && e.pixels_per_lane != 4) || 4 * e.pixels_per_lane > ts) {

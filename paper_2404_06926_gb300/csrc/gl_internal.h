@@ -198,15 +198,16 @@ struct View {
     // into segments of seg records (seg a power of two; 0: never split)
     int seg = 0;
     bool seg_auto = false;    // seg was not asked for: dropped where its state finds no memory
-    // The execution knob: 0 takes kAutoSegment.  Without segments a list is
-    // one warp's serial chain per pixel block, and the deepest tile's chain
-    // is the kernel's time; lists shorter than 2 kAutoSegment stay whole, so
-    // small scenes run as they did.  250k Gaussians at 640x480: forward 423 ->
-    // 140 us, backward 650 -> 91 us.
+    // The execution knob: -1 (what a context starts with) takes kAutoSegment.
+    // Without segments a list is one warp's serial chain per pixel block, and
+    // the deepest tile's chain is the kernel's time; lists shorter than 2
+    // kAutoSegment stay whole, so small scenes run as they did.  250k Gaussians
+    // at 640x480: forward 423 -> 140 us, backward 650 -> 91 us.  0 keeps every
+    // list whole.
     static constexpr int kAutoSegment = 512;
     void set_segment(int knob)
     {
-        seg_auto = knob == 0;
+        seg_auto = knob < 0;
         seg = seg_auto ? kAutoSegment : knob;
     }
     // exact tile culling: only tiles where the Gaussian can reach alpha >=
@@ -233,7 +234,7 @@ struct View {
 struct gl_ctx_impl {
     cudaStream_t stream = nullptr;
     View view;
-    gl_exec_config exec{0, 0, 32, 1, 0, 0, 0, 1, 0};
+    gl_exec_config exec{0, 0, 32, 1, 0, 0, -1, 1, 0};
     DevBuf pose_part;   // per-block pose partials
     DevBuf loss_part;   // per-block loss partials
     float pose_jac[36] = {};   // J_l of the last forward's twist (row-major 6 x 6)

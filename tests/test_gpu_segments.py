@@ -159,3 +159,38 @@ def test_deep_batches_render_and_gradients(scene, bd):
     for name in ("means", "log_scales", "quats", "logits", "sh"):
         med, p99 = _rel(gg[name].cpu().numpy()[vis], g[name][vis])
         assert med < 1e-3 and p99 < 1e-2, (name, med, p99)
+
+
+def test_segment_zero_keeps_lists_whole():
+    """segment = 0 never splits: the images and pixel states of a deep list are
+    those of a segment longer than the list, bit for bit; a context that was
+    told nothing splits at 512; -1 asks for that again; other values are refused."""
+    from paper_2404_06926_gb300 import binding
+    rng = np.random.default_rng(3)
+    n = 3000
+    cam = scenes.camera(20, 13, 100.0, 100.0, 10.0, 6.5)
+    params = dict(means=np.stack([rng.normal(0, 0.05, n), rng.normal(0, 0.05, n), rng.uniform(1, 3, n)], 1),
+                  log_scales=rng.uniform(0.4, 0.8, (n, 3)), quats=rng.normal(size=(n, 4)),
+                  logits=np.full(n, -5.0), sh=rng.normal(0, 0.5, (n, 1, 3)))
+    p = {k: torch.from_numpy(np.ascontiguousarray(v, np.float32)).cuda() for k, v in params.items()}
+
+    def images(seg):
+        ctx = binding.Ctx()
+        if seg is not None:
+            ctx.set_exec(segment=seg)
+        out = list(ctx.forward(p, cam, 16)) + list(ctx.pixel_state(13, 20, "cuda"))
+        return [x.cpu().numpy() for x in out]
+
+    same = lambda a, b: all(np.array_equal(x, y) for x, y in zip(a, b))
+    whole, split = images(65536), images(512)
+    assert not same(whole, split)   # the rounding of the products tells them apart
+    assert same(images(0), whole)
+    assert same(images(None), split) and same(images(-1), split)
+    m = binding.Map(binding.default_config(n_sky=0, sh_degree=0, capacity_hint=n))
+    assert m.get_exec()["segment"] == -1
+    assert m.set_exec(segment=0)["segment"] == 0 and m.get_exec()["segment"] == 0
+    for bad in (-2, 1, 63, 96, 131072):
+        with pytest.raises(binding.GLError, match="INVALID"):
+            m.set_exec(segment=bad)
+        with pytest.raises(binding.GLError, match="INVALID"):
+            binding.Ctx().set_exec(segment=bad)
