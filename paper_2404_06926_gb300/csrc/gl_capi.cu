@@ -1003,32 +1003,30 @@ extern "C" gl_status gl_render(gl_map* m, const gl_pose* pose, const gl_intrinsi
     GL_TRY(make_cam(pose, K, cam));
     if (E34 && !finite_all(E34, 12)) { set_error("exposure contains NaN or Inf"); return GL_ERR_INVALID; }
     // images in the caller's device memory are rendered in place (the colour
-    // only without an exposure)
-    float* depth = is_local_array(out_depth) ? out_depth : nullptr;
-    float* opac = is_local_array(out_opacity) ? out_opacity : nullptr;
-    float* rgb = !E34 && is_local_array(out_rgb) ? out_rgb : nullptr;
-    {
-        const size_t px = (size_t)cam.W * cam.H;
-        if (overlap(rgb, 3 * px, depth, px) || overlap(rgb, 3 * px, opac, px) || overlap(depth, px, opac, px))
-            rgb = depth = opac = nullptr;   // copied out one after the other
-    }
+    // only without an exposure); images that share memory are copied out one
+    // after the other, the later one winning
+    const size_t px = (size_t)cam.W * cam.H;
+    const bool shared = overlap(out_rgb, 3 * px, out_depth, px) || overlap(out_rgb, 3 * px, out_opacity, px) ||
+                        overlap(out_depth, px, out_opacity, px);
+    float* depth = !shared && is_local_array(out_depth) ? out_depth : nullptr;
+    float* opac = !shared && is_local_array(out_opacity) ? out_opacity : nullptr;
+    float* rgb = !shared && !E34 && is_local_array(out_rgb) ? out_rgb : nullptr;
     GL_TRY(render_internal(m, cam, m->cfg.tile_size, rgb, depth, opac));
     View& v = m->ctx.view;
-    const size_t P = (size_t)cam.W * cam.H;
     const float ident[12] = {1, 0, 0, 0, 0, 1, 0, 0, 0, 0, 1, 0};
     if (!rgb && is_device_ptr(out_rgb)) {
-        GL_TRY(apply_exposure(v.rgb.as<float>(), out_rgb, E34 ? E34 : ident, (int64_t)P, m->stream));
+        GL_TRY(apply_exposure(v.rgb.as<float>(), out_rgb, E34 ? E34 : ident, (int64_t)px, m->stream));
     } else if (!rgb) {
         const float* src = v.rgb.as<float>();
         if (E34) {
-            GL_TRY(m->stage_img.reserve(12 * P));
-            GL_TRY(apply_exposure(src, m->stage_img.as<float>(), E34, (int64_t)P, m->stream));
+            GL_TRY(m->stage_img.reserve(12 * px));
+            GL_TRY(apply_exposure(src, m->stage_img.as<float>(), E34, (int64_t)px, m->stream));
             src = m->stage_img.as<float>();
         }
-        GL_CUDA_TRY(cudaMemcpyAsync(out_rgb, src, 12 * P, cudaMemcpyDeviceToHost, m->stream));
+        GL_CUDA_TRY(cudaMemcpyAsync(out_rgb, src, 12 * px, cudaMemcpyDeviceToHost, m->stream));
     }
-    if (out_depth && !depth) GL_TRY(from_device(out_depth, v.depth.as<float>(), P, m->stream));
-    if (out_opacity && !opac) GL_TRY(from_device(out_opacity, v.opac.as<float>(), P, m->stream));
+    if (out_depth && !depth) GL_TRY(from_device(out_depth, v.depth.as<float>(), px, m->stream));
+    if (out_opacity && !opac) GL_TRY(from_device(out_opacity, v.opac.as<float>(), px, m->stream));
     GL_CUDA_TRY(cudaStreamSynchronize(m->stream));
     return sort_wait_status(v, m->stream);
 }

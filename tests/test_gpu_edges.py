@@ -292,3 +292,23 @@ def test_every_band_moves_by_its_own_rate(n, deg, sparse):
     if deg:
         rest = np.abs(got["sh"] - params["sh"])[seen, 1:]
         assert np.allclose(rest[rest > 0], lr["lr_sh_rest"], rtol=1e-3, atol=1e-7)
+
+
+@pytest.mark.parametrize("exposed", [False, True])
+@pytest.mark.parametrize("second", ["out_depth", "out_opacity"])
+def test_render_into_images_that_share_memory(exposed, second):
+    """Colour, depth, opacity are written in that order, whatever the exposure:
+    where two device images share memory the later one stays, as on the host."""
+    from paper_2404_06926_gb300 import binding
+    sc = scenes.small_frustum(n=300)
+    cam = sc["cam"]
+    H, W = cam["height"], cam["width"]
+    m = binding.Map(binding.default_config(n_sky=0, sh_degree=0, capacity_hint=300))
+    m.set_params(_dev(sc["params"]))
+    E = np.concatenate([np.eye(3, dtype=np.float32), np.full((3, 1), 0.25, np.float32)], 1) if exposed else None
+    for at in (0, 2):   # the colour's first and last third
+        want = np.empty((3, H, W), np.float32)
+        m.render(cam, E=E, out_rgb=want.reshape(H, W, 3), **{second: want[at]})
+        got = torch.empty((3, H, W), device="cuda")
+        m.render(cam, E=E, out_rgb=got.view(H, W, 3), **{second: got[at]})
+        assert np.array_equal(got.cpu().numpy(), want), at
