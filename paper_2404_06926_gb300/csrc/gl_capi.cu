@@ -790,15 +790,21 @@ gl_status from_device(float* dst, const float* src, size_t count, cudaStream_t s
 }
 
 // The live rows of five map arrays into the caller's arrays (null: skipped).
+// Arrays that share memory are copied one after the other, the later one
+// winning; the others move in one launch.
 gl_status copy_rows_out(gl_map* m, DevBuf* src, float* const dst[NPARAM])
 {
+    size_t cnt[NPARAM];
+    for (int w = 0; w < NPARAM; w++) cnt[w] = m->row_floats(w) * (size_t)m->n;
+    bool shared = false;
+    for (int w = 1; w < NPARAM; w++)
+        for (int u = 0; u < w; u++) shared = shared || overlap(dst[u], cnt[u], dst[w], cnt[w]);
     ArrayMove mv[NPARAM];
     int k = 0;
     for (int w = 0; w < NPARAM; w++) {
         if (!dst[w] || m->n == 0) continue;
-        const size_t cnt = m->row_floats(w) * (size_t)m->n;
-        if (is_local_array(dst[w])) mv[k++] = {dst[w], src[w].as<float>(), cnt};
-        else GL_TRY(from_device(dst[w], src[w].as<float>(), cnt, m->stream));
+        if (!shared && is_local_array(dst[w])) mv[k++] = {dst[w], src[w].as<float>(), cnt[w]};
+        else GL_TRY(from_device(dst[w], src[w].as<float>(), cnt[w], m->stream));
     }
     return move_arrays(mv, k, m->stream);
 }

@@ -312,3 +312,26 @@ def test_render_into_images_that_share_memory(exposed, second):
         got = torch.empty((3, H, W), device="cuda")
         m.render(cam, E=E, out_rgb=got.view(H, W, 3), **{second: got[at]})
         assert np.array_equal(got.cpu().numpy(), want), at
+
+
+@pytest.mark.parametrize("n", [1, 3000, 100_000])
+def test_arrays_read_back_into_shared_memory(n):
+    """Parameters read back into device arrays that share memory: the arrays are
+    written in their order, the later one winning, as into host memory."""
+    from paper_2404_06926_gb300 import binding
+    rng = np.random.default_rng(n)
+    p = dict(means=rng.normal(size=(n, 3)), log_scales=rng.normal(size=(n, 3)), quats=rng.normal(size=(n, 4)),
+             logits=rng.normal(size=n), sh=rng.normal(size=(n, 1, 3)))
+    m = binding.Map(binding.default_config(n_sky=0, sh_degree=0, capacity_hint=n))
+    m.set_params(_dev(p))
+
+    def read(buf):
+        out = dict(means=buf[:3 * n].reshape(n, 3), log_scales=buf[:3 * n].reshape(n, 3),
+                   quats=buf[2 * n:6 * n].reshape(n, 4), logits=buf[5 * n:6 * n], sh=buf[n:4 * n].reshape(n, 1, 3))
+        g = binding.gaussians(out, n)
+        binding.check(binding.lib().gl_map_get_params(m._h, binding.C.byref(g), None))
+        return buf
+
+    want = read(np.zeros(6 * n, np.float32))
+    for _ in range(5):
+        assert np.array_equal(read(torch.zeros(6 * n, device="cuda")).cpu().numpy(), want)
