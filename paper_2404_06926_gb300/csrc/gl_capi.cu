@@ -1,6 +1,7 @@
 // gl_capi.cu -- host implementation of the C ABI declared in include/gl_map.h:
 // argument validation, device-memory ownership, the keyframe store, and the
 // sequencing of the kernels of one optimisation step on the map's stream.
+#include <cuda.h>   // types only: the driver's entry points are looked up at run time
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -399,8 +400,31 @@ bool is_device_ptr(const void* p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// A float array that a kernel on the current device can read and write.
-bool is_local_array(const void* p)
+// Bytes from p to the end of the device allocation that holds it; 0 if none
+// does (or the driver does not say).
+size_t bytes_left(const void* p)
+{
+    using Range = CUresult(CUDAAPI*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const Range range = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Range>(f);
+    }();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const CUdeviceptr at = (CUdeviceptr)(uintptr_t)p;
+    if (!range || range(&base, &size, at) != CUDA_SUCCESS || at < base || at - base >= size) return 0;
+    return size - (size_t)(at - base);
+}
+
+// `count` floats that a kernel on the current device can read and write: one
+// allocation holds them (a copy looks at that itself, a kernel does not).
+bool is_local_array(const void* p, size_t count)
 {
     cudaPointerAttributes a;
     int dev = -1;
@@ -408,7 +432,20 @@ bool is_local_array(const void* p)
         cudaGetLastError();
         return false;
     }
-    return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev);
+    return (a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev)) &&
+           bytes_left(p) >= 4 * count;
+}
+
+// Refuses device memory that ends before `count` floats with nothing mapped
+// behind it.  (What spans several allocations is left to the copy.)
+gl_status check_extent(const void* p, size_t count)
+{
+    const size_t left = is_device_ptr(p) ? bytes_left(p) : 0;
+    if (left && left < 4 * count && bytes_left(static_cast<const char*>(p) + left) == 0) {
+        set_error("a device array ends before its last row");
+        return GL_ERR_INVALID;
+    }
+    return GL_OK;
 }
 
 bool overlap(const float* a, size_t na, const float* b, size_t nb) { return a && b && a < b + nb && b < a + na; }
@@ -785,6 +822,7 @@ gl_status zero_moments(gl_map* m, int64_t from, int64_t count)
 
 gl_status from_device(float* dst, const float* src, size_t count, cudaStream_t s)
 {
+    GL_TRY(check_extent(dst, count));
     GL_CUDA_TRY(cudaMemcpyAsync(dst, src, 4 * count, is_device_ptr(dst) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     return GL_OK;
 }
@@ -803,7 +841,7 @@ gl_status copy_rows_out(gl_map* m, DevBuf* src, float* const dst[NPARAM])
     int k = 0;
     for (int w = 0; w < NPARAM; w++) {
         if (!dst[w] || m->n == 0) continue;
-        if (!shared && is_local_array(dst[w])) mv[k++] = {dst[w], src[w].as<float>(), cnt[w]};
+        if (!shared && is_local_array(dst[w], cnt[w])) mv[k++] = {dst[w], src[w].as<float>(), cnt[w]};
         else GL_TRY(from_device(dst[w], src[w].as<float>(), cnt[w], m->stream));
     }
     return move_arrays(mv, k, m->stream);
@@ -1014,13 +1052,14 @@ extern "C" gl_status gl_render(gl_map* m, const gl_pose* pose, const gl_intrinsi
     const size_t px = (size_t)cam.W * cam.H;
     const bool shared = overlap(out_rgb, 3 * px, out_depth, px) || overlap(out_rgb, 3 * px, out_opacity, px) ||
                         overlap(out_depth, px, out_opacity, px);
-    float* depth = !shared && is_local_array(out_depth) ? out_depth : nullptr;
-    float* opac = !shared && is_local_array(out_opacity) ? out_opacity : nullptr;
-    float* rgb = !shared && !E34 && is_local_array(out_rgb) ? out_rgb : nullptr;
+    float* depth = !shared && is_local_array(out_depth, px) ? out_depth : nullptr;
+    float* opac = !shared && is_local_array(out_opacity, px) ? out_opacity : nullptr;
+    float* rgb = !shared && !E34 && is_local_array(out_rgb, 3 * px) ? out_rgb : nullptr;
     GL_TRY(render_internal(m, cam, m->cfg.tile_size, rgb, depth, opac));
     View& v = m->ctx.view;
     const float ident[12] = {1, 0, 0, 0, 0, 1, 0, 0, 0, 0, 1, 0};
     if (!rgb && is_device_ptr(out_rgb)) {
+        GL_TRY(check_extent(out_rgb, 3 * px));
         GL_TRY(apply_exposure(v.rgb.as<float>(), out_rgb, E34 ? E34 : ident, (int64_t)px, m->stream));
     } else if (!rgb) {
         const float* src = v.rgb.as<float>();
@@ -1388,10 +1427,14 @@ extern "C" gl_status gl_map_set_params(gl_map* m, const gl_gaussians* in)
     int k = 0;
     for (int w = 0; w < NPARAM; w++) {
         const size_t cnt = m->row_floats(w) * (size_t)in->n;
-        if (is_local_array(src[w])) mv[k++] = {m->prm[w].as<float>(), src[w], cnt};
-        else GL_CUDA_TRY(cudaMemcpyAsync(m->prm[w].p, src[w], 4 * cnt,
-                                         is_device_ptr(src[w]) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                                         m->stream));
+        if (is_local_array(src[w], cnt)) {
+            mv[k++] = {m->prm[w].as<float>(), src[w], cnt};
+        } else {
+            GL_TRY(check_extent(src[w], cnt));
+            GL_CUDA_TRY(cudaMemcpyAsync(m->prm[w].p, src[w], 4 * cnt,
+                                        is_device_ptr(src[w]) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                                        m->stream));
+        }
         mv[k++] = {m->mom1[w].as<float>(), nullptr, cnt};
         mv[k++] = {m->mom2[w].as<float>(), nullptr, cnt};
     }

@@ -335,3 +335,61 @@ def test_arrays_read_back_into_shared_memory(n):
     want = read(np.zeros(6 * n, np.float32))
     for _ in range(5):
         assert np.array_equal(read(torch.zeros(6 * n, device="cuda")).cpu().numpy(), want)
+
+
+class _Raw:
+    """A device allocation of its own, of exactly so many bytes."""
+
+    def __init__(self, nbytes):
+        import ctypes
+        torch.cuda.current_stream().synchronize()   # the primary context exists and is current
+        self.cu, self.p = ctypes.CDLL("libcuda.so.1"), ctypes.c_uint64()
+        assert self.cu.cuMemAlloc_v2(ctypes.byref(self.p), ctypes.c_size_t(nbytes)) == 0
+
+    def free(self):
+        self.cu.cuMemFree_v2(self.p)
+
+
+def test_device_arrays_that_end_early_are_refused():
+    """Arrays that end with their allocation are taken; one that ends 4 MB before
+    its last row is refused on the host, read or written, as a copy would."""
+    from paper_2404_06926_gb300 import binding
+    n = 1_000_000
+    rng = np.random.default_rng(5)
+    rows = dict(means=3, log_scales=3, quats=4, logits=1, sh=3)
+    p = {k: rng.normal(size=n * w).astype(np.float32) for k, w in rows.items()}
+    host = dict(means=p["means"].reshape(n, 3), log_scales=p["log_scales"].reshape(n, 3), quats=p["quats"].reshape(n, 4),
+                logits=p["logits"], sh=p["sh"].reshape(n, 1, 3))
+    m = binding.Map(binding.default_config(n_sky=0, sh_degree=0, capacity_hint=n))
+    m.set_params(host)
+    L, C = binding.lib(), binding.C
+    full = {k: _Raw(4 * n * w) for k, w in rows.items()}
+    short = {k: _Raw(4 * n * w - (4 << 20) + 64) for k, w in rows.items() if 4 * n * w > (4 << 20)}
+
+    def struct(**other):
+        g = binding.gaussians(host)
+        for k in rows:
+            setattr(g, k, other.get(k, full[k]).p.value)
+        return g
+
+    for call in (lambda g: L.gl_map_get_params(m._h, C.byref(g), None), lambda g: L.gl_map_set_params(m._h, C.byref(g))):
+        binding.check(call(struct()))
+        for k, r in short.items():
+            with pytest.raises(binding.GLError, match="INVALID"):
+                binding.check(call(struct(**{k: r})))
+        assert len(m) == n
+    got = m.get_params()   # written to the raw arrays and read back from them
+    assert all(np.array_equal(got[k].ravel(), p[k]) for k in rows)
+    H, W = 1536, 2048
+    cam = scenes.camera(W, H, 1000.0, 1000.0, 1024.0, 768.0)
+    c, d = torch.empty((H, W, 3), device="cuda"), _Raw(4 * H * W)
+    less = _Raw(4 * H * W - (4 << 20) + 64)
+    K, P = binding.intrinsics(cam), binding.pose(cam)
+    small = binding.Map(binding.default_config(n_sky=0, sh_degree=0, capacity_hint=300))
+    small.set_params(_dev(scenes.small_frustum(n=300)["params"]))
+    render = lambda depth: binding.check(L.gl_render(small._h, C.byref(P), C.byref(K), None, c.data_ptr(), depth.p.value, None))
+    render(d)
+    with pytest.raises(binding.GLError, match="INVALID"):
+        render(less)
+    for r in (*full.values(), *short.values(), d, less):
+        r.free()
