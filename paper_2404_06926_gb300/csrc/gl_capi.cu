@@ -1453,9 +1453,11 @@ extern "C" gl_status gl_map_get_exposure(gl_map* m, int64_t id, float* E34_out)
     Keyframe* kf = get_kf(m, id, false, &st);
     if (!kf) return st;
     // through pinned memory: a copy to pageable memory is staged by the driver
-    GL_CUDA_TRY(cudaMemcpyAsync(m->h_expo, kf->expo.p, 48, cudaMemcpyDeviceToHost, m->stream));
+    // (what the host cannot write is left to the driver)
+    const bool host = !is_device_ptr(E34_out);
+    GL_CUDA_TRY(cudaMemcpyAsync(host ? m->h_expo : E34_out, kf->expo.p, 48, cudaMemcpyDeviceToHost, m->stream));
     GL_CUDA_TRY(cudaStreamSynchronize(m->stream));
-    std::memcpy(E34_out, m->h_expo, 48);
+    if (host) std::memcpy(E34_out, m->h_expo, 48);
     return GL_OK;
 }
 

@@ -393,3 +393,17 @@ def test_device_arrays_that_end_early_are_refused():
         render(less)
     for r in (*full.values(), *short.values(), d, less):
         r.free()
+
+
+def test_exposure_into_device_memory_does_not_crash():
+    """An exposure is asked for in host memory; a device pointer is the driver's
+    to take or refuse, not the host's to write to."""
+    from paper_2404_06926_gb300 import binding
+    cam = scenes.camera(32, 16, 30.0, 30.0, 16.0, 8.0)
+    m = binding.Map(binding.default_config(n_sky=0, sh_degree=0, capacity_hint=16))
+    m.add_keyframe(3, cam, np.zeros((16, 32, 3), np.float32))
+    E = torch.full((12,), -1.0, device="cuda")
+    st = binding.lib().gl_map_get_exposure(m._h, 3, E.data_ptr())
+    assert np.array_equal(m.exposure(3), np.eye(3, 4, dtype=np.float32))
+    if st == 0:
+        assert np.array_equal(E.cpu().numpy().reshape(3, 4), np.eye(3, 4, dtype=np.float32))
