@@ -526,22 +526,49 @@ __device__ __forceinline__ void df_div(float ah, float al, float bh, float bl, f
     two_sum(q1, __fdiv_rn(r, bh), qh, ql);
 }
 
-// (h + l) += x, the sum of floats that the reductions of block partials keep:
-// as wide as their double sum was (about 2^-48 relative per addition) without
-// the few FP64 lanes of the chip, which made those sums the reductions' time
-__device__ __forceinline__ void df_acc(float& h, float& l, float x)
-{
-    float s, e;
-    two_sum(h, x, s, e);
-    h = s;
-    l = __fadd_rn(l, e);
-}
+// A sum of floats in three floats: what an addition rounds off goes to m, what
+// that rounds off to l.  Each addition loses about 2^-72 of the sum, so the
+// value is as good as a double sum of the floats (2^-53 an addition), without
+// the few FP64 lanes of the chip, which made those sums the reductions' time.
+struct FloatSum {
+    float h, m, l;
+    __device__ __forceinline__ void add(float x)
+    {
+        float e, r;
+        two_sum(h, x, h, e);
+        two_sum(m, e, m, r);
+        l = __fadd_rn(l, r);
+    }
+    __device__ __forceinline__ void add(const FloatSum& o)
+    {
+        add(o.h);
+        add(o.m);
+        add(o.l);
+    }
+    __device__ __forceinline__ FloatSum xor_lane(int off) const
+    {
+        FloatSum o;
+        o.h = __shfl_xor_sync(kFull, h, off);
+        o.m = __shfl_xor_sync(kFull, m, off);
+        o.l = __shfl_xor_sync(kFull, l, off);
+        return o;
+    }
+    // false where the sum left the range of a float, or met an infinity or a
+    // NaN: then it has to be taken again, in double
+    __device__ __forceinline__ bool finite() const { return fabsf(h) <= 3.4028235e38f && fabsf(m) <= 3.4028235e38f; }
+    __device__ __forceinline__ double value() const { return (double)h + ((double)m + (double)l); }
+};
 
-// its value; an infinite or NaN sum keeps the plain sum's value (the error
-// terms of infinities are NaN)
-__device__ __forceinline__ double df_value(float h, float l)
+// The same over part[k], part[k + stride], ... (count of them) by a warp, in
+// double: the total in every lane.
+__device__ __forceinline__ double warp_double_sum(const float* __restrict__ part, int64_t count, int stride, int lane)
 {
-    return fabsf(l) <= 3.0e38f ? (double)h + (double)l : (double)h;
+    double acc = 0.0;
+#pragma unroll 1
+    for (int64_t i = lane; i < count; i += 32) acc += (double)part[i * stride];
+#pragma unroll 1
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(kFull, acc, off);
+    return acc;
 }
 
 // mu' as (u_hi + u_lo, v_hi + v_lo); z > 0 is known (the decision passed)

@@ -27,7 +27,7 @@
 // One CTA for all three channels -> this: 115.7 -> 104.9 us (1280x1024), 40.6 ->
 // 32.9 (647x481), 24.2 -> 13.8 (256x192: 48 tiles).
 // Per-CTA partial sums of |.|, SSIM and dL/dE are reduced afterwards in a
-// fixed order, in double.
+// fixed order (k_loss_final).
 #include "gl_internal.h"
 
 #include <cooperative_groups.h>
@@ -415,14 +415,15 @@ k_loss(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __re
     loss_tile<false>(one, views, V, rgb_all, dL_all, lambda, part);
 }
 
-// Sums the per-tile partials in a fixed order (float pairs, df_acc).  Single
-// view (views null): block 0 over [0, nblk) -> loss_out, dE_out.  Views: block
-// v over the view's loss tiles -> loss_v[v] (unweighted) and, if the view has
-// Em, one Adam step of its exposure on the (already weighted) gradient.
+// Sums the per-tile partials in a fixed order (in three floats, FloatSum; again
+// in double where that overflows).  Single view (views null): block 0 over
+// [0, nblk) -> loss_out, dE_out.  Views: block v over the view's loss tiles ->
+// loss_v[v] (unweighted) and, if the view has Em, one Adam step of its exposure
+// on the (already weighted) gradient.
 // Bound by latency: one CTA reads nblk x 14 floats in order (thread t takes
 // elements t, t + 1022, ...: 1022 = 73 x 14, so always the same partial),
 // eight loads in flight, then a warp per partial adds the 73 sums.
-// A warp per partial in double -> this: 13.3 -> 4.4 us (1280x1024).
+// A warp per partial in double -> this: 13.3 -> 5.3 us (1280x1024).
 constexpr int kRedBatch = 8;
 constexpr int kRedRows = 73;
 constexpr int kRedThreads = 1024;
@@ -433,8 +434,9 @@ k_loss_final(const float* __restrict__ part, int nblk, int W, int H, float lambd
              const ViewDesc* __restrict__ views, float* __restrict__ loss_v, float b1,
              float b2, float eps, float lr, const uint64_t* __restrict__ abort)
 {
-    __shared__ float2 sums[kRedRows * kNP];
-    __shared__ double tot[kNP];
+    __shared__ FloatSum sums[kRedRows * kNP];
+    __shared__ FloatSum tot[kNP];
+    __shared__ double again[kNP];   // of the sums that overflowed
     __shared__ double s_invN;
     int begin = 0;
     float* Ev = nullptr;
@@ -454,52 +456,49 @@ k_loss_final(const float* __restrict__ part, int nblk, int W, int H, float lambd
     const int tid = threadIdx.x;
     constexpr int STRIDE = kRedRows * kNP;
     if (tid < STRIDE) {
-        const float* src = part + (size_t)begin * kNP;
-        const int64_t total = (int64_t)nblk * kNP;
-        float h = 0.0f, l = 0.0f;
-        for (int64_t i0 = tid; i0 < total; i0 += (int64_t)STRIDE * kRedBatch) {
+        const float* src = part + (size_t)begin * kNP + tid;
+        int left = (nblk * kNP - tid + STRIDE - 1) / STRIDE;   // elements of this thread
+        FloatSum S{};
+        for (; left > 0; left -= kRedBatch, src += STRIDE * kRedBatch) {
             float x[kRedBatch];
 #pragma unroll
-            for (int b = 0; b < kRedBatch; b++) {
-                const int64_t i = i0 + (int64_t)STRIDE * b;
-                x[b] = i < total ? src[i] : 0.0f;
-            }
+            for (int b = 0; b < kRedBatch; b++) x[b] = b < left ? src[STRIDE * b] : 0.0f;
 #pragma unroll
-            for (int b = 0; b < kRedBatch; b++) df_acc(h, l, x[b]);
+            for (int b = 0; b < kRedBatch; b++)
+                if (b < left) S.add(x[b]);
         }
-        sums[tid] = make_float2(h, l);
+        sums[tid] = S;
     } else if (tid == kRedThreads - 1) {
         s_invN = 1.0 / (3.0 * (double)W * (double)H);   // while the others load
     }
     __syncthreads();
     const int k = tid >> 5, lane = tid & 31;
     if (k < kNP) {
-        float h = 0.0f, l = 0.0f;
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            const int r = lane + 32 * j;
-            if (r < kRedRows) {
-                const float2 v = sums[r * kNP + k];
-                df_acc(h, l, v.x);
-                l += v.y;
-            }
+        FloatSum S{};
+        // rolled: the kernel runs once through its code, from a cold
+        // instruction cache
+#pragma unroll 1
+        for (int r = lane; r < kRedRows; r += 32) S.add(sums[r * kNP + k]);
+#pragma unroll 1
+        for (int off = 16; off > 0; off >>= 1) S.add(S.xor_lane(off));
+        if (lane == 0) tot[k] = S;
+        if (__any_sync(kFull, !S.finite())) {
+            const double v = warp_double_sum(part + (size_t)begin * kNP + k, nblk, kNP, lane);
+            if (lane == 0) again[k] = v;
         }
-        for (int off = 16; off > 0; off >>= 1) {
-            const float oh = __shfl_xor_sync(kFull, h, off), ol = __shfl_xor_sync(kFull, l, off);
-            df_acc(h, l, oh);
-            l += ol;
-        }
-        if (lane == 0) tot[k] = df_value(h, l);
     }
     __syncthreads();
+    // (few warps take the sums to double: its lanes are few)
     if (tid == 32) {
-        const double L = (1.0 - lambda) * tot[12] * s_invN + lambda * (1.0 - tot[13] * s_invN);
+        const double l1 = tot[12].finite() ? tot[12].value() : again[12];
+        const double ss = tot[13].finite() ? tot[13].value() : again[13];
+        const double L = (1.0 - lambda) * l1 * s_invN + lambda * (1.0 - ss * s_invN);
         if (views) { if (loss_v) loss_v[blockIdx.x] = (float)L; }
         else if (loss_out) *loss_out = (float)L;
     }
     if (tid < 12) {
         const int i = tid;
-        const float g = (float)tot[i];
+        const float g = (float)(tot[i].finite() ? tot[i].value() : again[i]);
         if (!views && dE_out) dE_out[i] = g;
         if (Ev && Em && !(abort && abort[1])) {
             const float m = b1 * Em[i] + (1.0f - b1) * g;

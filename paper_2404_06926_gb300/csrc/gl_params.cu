@@ -625,13 +625,13 @@ struct Jac6 {
     float m[36];
 };
 
-// Sum of the blocks' pose partials in a fixed order (float pairs, df_acc),
-// then J^T g.  One cluster of eight CTAs: thread t of CTA c takes elements
+// Sum of the blocks' pose partials in a fixed order (in three floats, FloatSum;
+// again in double where that overflows), then J^T g.  One cluster of eight CTAs: thread t of CTA c takes elements
 // 1020 c + t, + 8160, ... (1020 = 170 x 6: always the same component), eight
 // loads in flight; CTA 0 reads and adds the eight CTAs' sums between two
 // cluster barriers (the first shows that all CTAs run, the second keeps their
 // shared memory until it has been read).  Bound by latency.
-// One CTA in double -> this: 34.9 -> 3.5 us (250k Gaussians).
+// One CTA in double -> this: 34.9 -> 4.7 us (250k Gaussians).
 constexpr int kPoseRows = 170;
 constexpr int kPoseThreads = 1024;
 constexpr int kPoseCtas = 8;
@@ -640,59 +640,56 @@ k_pose_reduce(const float* __restrict__ part, int npart, Jac6 J, float* __restri
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    __shared__ float2 sums[kPoseRows * 6];
-    __shared__ float2 mine[6];   // this CTA's sums
-    __shared__ double gsum[6];
+    __shared__ FloatSum sums[kPoseRows * 6];
+    __shared__ FloatSum mine[6];   // this CTA's sums
+    __shared__ FloatSum tot[6];
+    __shared__ double again[6];    // of the sums that overflowed
     const int tid = threadIdx.x;
     constexpr int PER = kPoseRows * 6, STRIDE = PER * kPoseCtas;
     if (tid < PER) {
-        const int64_t total = 6 * (int64_t)npart;
-        float h = 0.0f, l = 0.0f;
-        for (int64_t i0 = (int64_t)blockIdx.x * PER + tid; i0 < total; i0 += (int64_t)STRIDE * 8) {
+        const int first = (int)blockIdx.x * PER + tid;
+        const float* src = part + first;
+        int left = (int)((6 * (int64_t)npart - first + STRIDE - 1) / STRIDE);   // elements of this thread
+        FloatSum S{};
+        for (; left > 0; left -= 8, src += STRIDE * 8) {
             float x[8];
 #pragma unroll
-            for (int b = 0; b < 8; b++) {
-                const int64_t i = i0 + (int64_t)STRIDE * b;
-                x[b] = i < total ? part[i] : 0.0f;
-            }
+            for (int b = 0; b < 8; b++) x[b] = b < left ? src[STRIDE * b] : 0.0f;
 #pragma unroll
-            for (int b = 0; b < 8; b++) df_acc(h, l, x[b]);
+            for (int b = 0; b < 8; b++)
+                if (b < left) S.add(x[b]);
         }
-        sums[tid] = make_float2(h, l);
+        sums[tid] = S;
     }
     __syncthreads();
     const int k = tid >> 5, lane = tid & 31;
     if (k < 6) {
-        float h = 0.0f, l = 0.0f;
-        for (int r = lane; r < kPoseRows; r += 32) {
-            const float2 v = sums[r * 6 + k];
-            df_acc(h, l, v.x);
-            l += v.y;
+        FloatSum S{};
+        // rolled: the kernel runs once through its code, from a cold
+        // instruction cache
+#pragma unroll 1
+        for (int r = lane; r < kPoseRows; r += 32) S.add(sums[r * 6 + k]);
+#pragma unroll 1
+        for (int off = 16; off > 0; off >>= 1) S.add(S.xor_lane(off));
+        if (lane == 0) mine[k] = S;
+    }
+    cluster.sync();
+    if (blockIdx.x == 0 && k < 6) {
+        // lane c < 8 takes CTA c's sums
+        FloatSum S{};
+        if (lane < kPoseCtas) S = cluster.map_shared_rank(mine, lane)[k];
+        for (int off = kPoseCtas / 2; off > 0; off >>= 1) S.add(S.xor_lane(off));
+        if (lane == 0) tot[k] = S;
+        if (__any_sync(kFull, !S.finite())) {
+            const double v = warp_double_sum(part + k, npart, 6, lane);
+            if (lane == 0) again[k] = v;
         }
-        for (int off = 16; off > 0; off >>= 1) {
-            const float oh = __shfl_xor_sync(kFull, h, off), ol = __shfl_xor_sync(kFull, l, off);
-            df_acc(h, l, oh);
-            l += ol;
-        }
-        if (lane == 0) mine[k] = make_float2(h, l);
     }
     cluster.sync();
     if (blockIdx.x == 0 && tid < 6) {
-        float2 v[kPoseCtas];
-#pragma unroll
-        for (int c = 0; c < kPoseCtas; c++) v[c] = cluster.map_shared_rank(mine, c)[tid];
-        float h = 0.0f, l = 0.0f;
-#pragma unroll
-        for (int c = 0; c < kPoseCtas; c++) {
-            df_acc(h, l, v[c].x);
-            l += v[c].y;
-        }
-        gsum[tid] = df_value(h, l);
-    }
-    cluster.sync();
-    if (blockIdx.x == 0 && tid < 6) {
+        const double v = tot[tid].finite() ? tot[tid].value() : again[tid];
         double o = 0.0;
-        for (int i = 0; i < 6; i++) o += (double)J.m[i * 6 + tid] * gsum[i];
+        for (int i = 0; i < 6; i++) o += (double)J.m[i * 6 + tid] * __shfl_sync(0x3fu, v, i);
         out6[tid] = (float)o;
     }
 }
