@@ -1801,11 +1801,16 @@ void bwd_dispatch(int nb, int pd, bool det, bool pg, const RasterArgs& A, const 
         if (pd == 1) bwd_launch<EXTRA, 1, 1, true>(A, G, units, persistent, s);
         else if (pd == 2) bwd_launch<EXTRA, 1, 2, true>(A, G, units, persistent, s);
         else bwd_launch<EXTRA, 1, 4, true>(A, G, units, persistent, s);
-    } else if (pd == 1 && blocks >= (int64_t)kMinBlocksHalf * kWpbHalf * sm_count()) {
+    } else if (pd == 1 && nb == 1 && blocks >= (int64_t)kMinBlocksHalf * kWpbHalf * sm_count()) {
         // more pixel blocks than resident warps.  Below, a warp has one block
         // and its chain is the time, which the two lists lengthen: 17.8 -> 22.4
         // us on 5k Gaussians at 256x192 (1.5k blocks; the line lies at 3.0k).
-        // (Hits wait in a ring, whatever the batch depth.)
+        // Its batches are of 32 records (hits wait in a ring): deeper ones
+        // were asked for and take the kernels that have them.
+        // Whole- and half-warp blocks by footprint, 1280x960, standard
+        // deviation in pixels: 1 (600k Gaussians) 245 and 188 us, 4 (100k) 224
+        // and 193, 10 (30k) 297 and 268, 30 (6k) 482 and 439, 80 (2k) 495 and
+        // 588: only Gaussians as large as the frame's quarter cost more.
         const int grid = grid_for(k_raster_bwd_half<EXTRA>, units, persistent, kWpbHalf);
         k_raster_bwd_half<EXTRA><<<grid, 32 * kWpbHalf, 0, s>>>(A, G);
     } else if (nb == 4) {   // deeper batches: one pixel per lane

@@ -407,3 +407,41 @@ def test_exposure_into_device_memory_does_not_crash():
     assert np.array_equal(m.exposure(3), np.eye(3, 4, dtype=np.float32))
     if st == 0:
         assert np.array_equal(E.cpu().numpy().reshape(3, 4), np.eye(3, 4, dtype=np.float32))
+
+
+@pytest.mark.parametrize("bd", [32, 64, 128, 256])
+def test_batch_depth_reaches_the_backward_of_large_frames(bd):
+    """Frames of more pixel blocks than resident warps (3,192): batches of 32
+    records walk half-warp blocks, deeper ones the kernel that stages them."""
+    from torch.profiler import ProfilerActivity, profile
+    from paper_2404_06926_gb300 import binding
+    rng = np.random.default_rng(60)
+    W, H, n = 331, 300, 60
+    cam = scenes.camera(W, H, 250.0, 250.0, W / 2, H / 2)
+    z = rng.uniform(1.0, 6.0, n)
+    q = rng.normal(size=(n, 4))
+    params = dict(means=np.stack([rng.uniform(-0.6, 0.6, n) * z, rng.uniform(-0.5, 0.5, n) * z, z], 1).astype(np.float32),
+                  log_scales=rng.uniform(-4.0, -2.0, (n, 3)).astype(np.float32),
+                  quats=(q / np.linalg.norm(q, axis=1, keepdims=True)).astype(np.float32),
+                  logits=rng.normal(0, 1, n).astype(np.float32), sh=rng.normal(0, 0.5, (n, 1, 3)).astype(np.float32))
+    pre, bins, _ = oracle.forward(params, cam, 16)
+    dC = (rng.normal(size=(H, W, 3)) * 1e-3).astype(np.float32)
+    g = oracle.backward(params, cam, pre, bins, dC.astype(np.float64))
+    ctx = binding.Ctx()
+    ctx.set_exec(batch_depth=bd)
+    p, d = _dev(params), torch.from_numpy(dC).cuda()
+    ctx.forward(p, cam, 16)
+    names = set()
+    for _ in range(4):   # (a profiler's first window can come back empty)
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            gg, _ = ctx.backward(p, d)
+            torch.cuda.synchronize()
+        names |= {e.name for e in prof.events() if "k_raster_bwd" in e.name}
+        if names:
+            break
+    assert len(names) == 1 and ("k_raster_bwd_half" in names.pop()) == (bd == 32)
+    vis = pre["radius"] > 0
+    for name in NAMES:
+        a, ref = gg[name].cpu().numpy().astype(np.float64)[vis].ravel(), np.asarray(g[name], np.float64)[vis].ravel()
+        rel = np.abs(a - ref) / np.maximum(np.abs(ref), 1e-4 * np.abs(ref).max())
+        assert np.median(rel) < 1e-3 and np.percentile(rel, 99) < 1e-2, (name, np.median(rel), np.percentile(rel, 99))
