@@ -372,6 +372,13 @@ GL_API int64_t gl_kernel_launch_count(void);
  * (null expired), GL_ERR_OOM, GL_ERR_CUDA. */
 GL_API gl_status gl_selftest_bounded_wait(int32_t* expired);
 
+/* Self-test of what the library does when memory runs out: its own device
+ * allocations of more than `bytes` made by the calling thread fail as if there
+ * were none left (0: no limit, as it starts).  *refused (host, nullable)
+ * receives how many failed this way since the last call.  Errors:
+ * GL_ERR_INVALID (negative). */
+GL_API gl_status gl_selftest_alloc_limit(int64_t bytes, int64_t* refused);
+
 /* ---------------------------------------------------------------------- */
 /* Serving loop (not in the paper, which runs the mapping thread of        */
 /* Sec. III-C beside tracking): a request loop over one map that keeps    */

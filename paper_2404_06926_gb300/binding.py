@@ -134,6 +134,7 @@ def lib():
             "gl_map_save": ([P, i32, P, i64], i32),
             "gl_map_load": ([P, P, i64], i32),
             "gl_selftest_bounded_wait": ([P], i32),
+            "gl_selftest_alloc_limit": ([i64, P], i32),
         }
         for name, (args, res) in sigs.items():
             fn = getattr(L, name)
@@ -323,6 +324,14 @@ def photometric_loss_noalloc(rgb, target, E, lam: float = 0.2, stream=None):
 def kernel_launches() -> int:
     """Kernels the library has launched in this process."""
     return int(lib().gl_kernel_launch_count())
+
+
+def selftest_alloc_limit(nbytes: int = 0) -> int:
+    """Make this thread's device allocations of more than nbytes fail as if no
+    memory were left (0: none); returns how many did since the last call."""
+    refused = C.c_int64(0)
+    check(lib().gl_selftest_alloc_limit(int(nbytes), C.byref(refused)))
+    return refused.value
 
 
 def selftest_bounded_wait() -> bool:

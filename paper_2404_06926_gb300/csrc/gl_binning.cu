@@ -899,10 +899,20 @@ int64_t work_items_bound(const View& v)
 
 gl_status build_items(View& v, cudaStream_t s)
 {
-    if (v.seg_auto && v.seg > 0 && reserve_segstate(v) != GL_OK) {
-        if (alloc_frozen()) return GL_ERR_CAPACITY;
-        cudaGetLastError();
-        v.seg = 0;
+    if (v.seg_auto && v.seg > 0) {
+        const size_t need = segstate_bytes(v);
+        if (need > v.segstate.bytes && v.seg_refused && need >= v.seg_refused && v.seg_wait > 0) {
+            v.seg_wait--;
+            v.seg = 0;
+        } else if (reserve_segstate(v) == GL_OK) {
+            v.seg_refused = 0;
+        } else {
+            if (alloc_frozen()) return GL_ERR_CAPACITY;
+            cudaGetLastError();
+            v.seg_refused = need;
+            v.seg_wait = View::kSegWait;
+            v.seg = 0;
+        }
     }
     GL_TRY(v.items.reserve(sizeof(uint2) * (size_t)std::max<int64_t>(work_items_bound(v), 1)));
     GL_TRY(v.tile_order.reserve(4 * (size_t)std::max(v.ntiles, 1)));

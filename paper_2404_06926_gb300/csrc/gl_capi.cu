@@ -162,6 +162,8 @@ void Prof::release()
 
 namespace {
 thread_local int t_freeze = 0;
+// gl_selftest_alloc_limit: allocations above it fail on this thread (0: none)
+thread_local int64_t t_alloc_limit = 0, t_alloc_refused = 0;
 }
 AllocFreeze::AllocFreeze() { t_freeze++; }
 AllocFreeze::~AllocFreeze() { t_freeze--; }
@@ -180,7 +182,9 @@ gl_status DevBuf::reserve(size_t need)
         bytes = 0;
     }
     if (need == 0) need = 16;
-    cudaError_t e = cudaMalloc(&p, need);
+    cudaError_t e = cudaErrorMemoryAllocation;
+    if (t_alloc_limit && need > (size_t)t_alloc_limit) t_alloc_refused++;
+    else e = cudaMalloc(&p, need);
     if (e != cudaSuccess) {
         p = nullptr;
         set_error(std::string("cudaMalloc(") + std::to_string(need) + "): " + cudaGetErrorString(e));
@@ -1524,6 +1528,15 @@ extern "C" gl_status gl_selftest_bounded_wait(int32_t* expired)
     if (!expired) { set_error("null expired"); return GL_ERR_INVALID; }
     *expired = 0;
     return sort_wait_selftest(expired);
+}
+
+extern "C" gl_status gl_selftest_alloc_limit(int64_t bytes, int64_t* refused)
+{
+    if (bytes < 0) { set_error("bytes must not be negative"); return GL_ERR_INVALID; }
+    t_alloc_limit = bytes;
+    if (refused) *refused = t_alloc_refused;
+    t_alloc_refused = 0;
+    return GL_OK;
 }
 
 // ---------------------------------------------------------------------------

@@ -198,6 +198,11 @@ struct View {
     // into segments of seg records (seg a power of two; 0: never split)
     int seg = 0;
     bool seg_auto = false;    // seg was not asked for: dropped where its state finds no memory
+    // what the state last found no memory for, and the binnings until it is
+    // asked for again (a failing allocation costs a step more than it saves)
+    size_t seg_refused = 0;
+    int seg_wait = 0;
+    static constexpr int kSegWait = 64;
     // The execution knob: -1 (what a context starts with) takes kAutoSegment.
     // Without segments a list is one warp's serial chain per pixel block, and
     // the deepest tile's chain is the kernel's time; lists shorter than 2
@@ -272,6 +277,7 @@ gl_status raster_forward(View& v, float* rgb, float* depth, float* opac, cudaStr
 // per seg records of the instance capacity).
 int64_t work_items_bound(const View& v);
 // The split tiles' state for the current capacity.
+size_t segstate_bytes(const View& v);
 gl_status reserve_segstate(View& v);
 // Build the work items of a binned step (after the tile order).
 gl_status build_items(View& v, cudaStream_t s);

@@ -1868,10 +1868,12 @@ void fwd_dispatch(const View& v, const RasterArgs& A, const RasterOut& O, int64_
     }
 }
 
-gl_status reserve_segstate(View& v)
+size_t segstate_bytes(const View& v)
 {
-    return v.segstate.reserve(sizeof(float) * kSegFields * (size_t)(v.Ts * v.Ts) * (size_t)split_items_bound(v));
+    return sizeof(float) * kSegFields * (size_t)(v.Ts * v.Ts) * (size_t)split_items_bound(v);
 }
+
+gl_status reserve_segstate(View& v) { return v.segstate.reserve(segstate_bytes(v)); }
 
 gl_status raster_forward(View& v, float* rgb, float* depth, float* opac, cudaStream_t s, bool extras)
 {

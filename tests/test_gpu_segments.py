@@ -194,3 +194,65 @@ def test_segment_zero_keeps_lists_whole():
             m.set_exec(segment=bad)
         with pytest.raises(binding.GLError, match="INVALID"):
             binding.Ctx().set_exec(segment=bad)
+
+
+def _deep_wide(n=6000, W=320, H=240):
+    """Lists of over a thousand Gaussians in the tiles of 32 pixels around the centre."""
+    rng = np.random.default_rng(11)
+    cam = scenes.camera(W, H, 200.0, 200.0, W / 2, H / 2)
+    params = dict(means=np.stack([rng.normal(0, 0.3, n), rng.normal(0, 0.25, n), rng.uniform(2, 3, n)], 1),
+                  log_scales=rng.uniform(-1.6, -1.0, (n, 3)), quats=rng.normal(size=(n, 4)),
+                  logits=np.full(n, -5.0), sh=rng.normal(0, 0.5, (n, 1, 3)))
+    return cam, {k: np.ascontiguousarray(v, np.float32) for k, v in params.items()}
+
+
+def test_lists_stay_whole_where_the_state_finds_no_memory():
+    """Where the split tiles' state is refused memory, the default execution keeps
+    lists whole, without an error and without asking again for 64 calls; an
+    explicit segment reports it.  Memory that comes back is used again."""
+    from paper_2404_06926_gb300 import binding
+    cam, params = _deep_wide()
+    p = {k: torch.from_numpy(v).cuda() for k, v in params.items()}
+    limit = 2 << 20   # above every other buffer (records 16 bytes an instance), below the state (96 at 32 x 32 tiles)
+
+    def forward(ctx):
+        out = list(ctx.forward(p, cam, 32)) + list(ctx.pixel_state(cam["height"], cam["width"], "cuda"))
+        return [x.cpu().numpy() for x in out]
+
+    same = lambda a, b: all(np.array_equal(x, y) for x, y in zip(a, b))
+    whole, split = binding.Ctx(), binding.Ctx()
+    whole.set_exec(segment=0)
+    ref_whole, ref_split = forward(whole), forward(split)
+    inst = whole.num_instances()
+    assert 16 * 1.25 * inst + 4096 < limit < 96 * inst and not same(ref_whole, ref_split)
+    dC = torch.from_numpy(np.random.default_rng(1).normal(size=(cam["height"], cam["width"], 3)).astype(np.float32)).cuda()
+    ctx, told = binding.Ctx(), binding.Ctx()
+    told.set_exec(segment=512)
+    told.forward(p, cam, 8)   # everything but the state for 32 x 32 tiles
+    m = binding.Map(binding.default_config(n_sky=0, sh_degree=0, tile_size=32, capacity_hint=len(params["logits"])))
+    m.set_params(params)
+    try:
+        binding.selftest_alloc_limit(limit)
+        for _ in range(10):
+            assert same(forward(ctx), ref_whole)
+        grads, _ = ctx.backward(p, dC)
+        assert binding.selftest_alloc_limit(limit) == 1
+        with pytest.raises(binding.GLError, match="OOM"):
+            told.forward(p, cam, 32)
+        binding.selftest_alloc_limit(limit)
+        for graphs in (0, 1):
+            m.set_exec(use_graphs=graphs)
+            losses = [m.optimize_step([(1, cam, np.zeros((cam["height"], cam["width"], 3), np.float32))], want_loss=True)
+                      for _ in range(4)]
+            assert all(np.isfinite(losses)) and losses[3] < losses[0]
+        assert binding.selftest_alloc_limit(limit) == 1
+    finally:
+        binding.selftest_alloc_limit(0)
+    ref, _ = whole.backward(p, dC)
+    for k in grads:   # the order of float atomics
+        a, b = grads[k].double(), ref[k].double()
+        assert float((a - b).norm() / b.norm()) < 1e-3, k
+    # ten calls were made, fewer than 64 more until the state is asked for again
+    for _ in range(64):
+        out = forward(ctx)
+    assert same(out, ref_split)
