@@ -901,10 +901,15 @@ gl_status build_items(View& v, cudaStream_t s)
 {
     if (v.seg_auto && v.seg > 0) {
         const size_t need = segstate_bytes(v);
+        const auto room = [&] {   // beside what has to stay free
+            size_t free = 0, total = 0;
+            if (v.keep_free == 0 || need <= v.segstate.bytes || alloc_frozen()) return true;
+            return cudaMemGetInfo(&free, &total) == cudaSuccess && free + v.segstate.bytes >= need + v.keep_free;
+        };
         if (need > v.segstate.bytes && v.seg_refused && need >= v.seg_refused && v.seg_wait > 0) {
             v.seg_wait--;
             v.seg = 0;
-        } else if (reserve_segstate(v) == GL_OK) {
+        } else if (room() && reserve_segstate(v) == GL_OK) {
             v.seg_refused = 0;
         } else {
             if (alloc_frozen()) return GL_ERR_CAPACITY;

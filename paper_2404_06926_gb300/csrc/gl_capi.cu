@@ -1958,6 +1958,8 @@ void map_exec_knobs(const gl_map* m, View& v, int Ts)
 int map_sh_degree(const gl_map* m) { return m->deg; }
 int map_tile_size(const gl_map* m) { return m->cfg.tile_size; }
 int64_t map_size_now(const gl_map* m) { return m->n; }
+void map_keep_free(gl_map* m, size_t bytes) { m->ctx.view.keep_free = bytes; }
+
 int64_t map_capacity(const gl_map* m) { return m->cap; }
 
 gl_status map_snapshot(gl_map* m, DevBuf* dst, int64_t* n_out, cudaEvent_t done)

@@ -203,6 +203,7 @@ struct View {
     size_t seg_refused = 0;
     int seg_wait = 0;
     static constexpr int kSegWait = 64;
+    size_t keep_free = 0;     // device memory that a state nobody asked for leaves free
     // The execution knob: -1 (what a context starts with) takes kAutoSegment.
     // Without segments a list is one warp's serial chain per pixel block, and
     // the deepest tile's chain is the kernel's time; lists shorter than 2
@@ -375,6 +376,8 @@ gl_status export_instances(const View& v, uint64_t* keys, uint32_t* vals, cudaSt
 // persistence, segment length; pixels per lane capped by the tile size Ts)
 // applied to another view's scratch.
 void map_exec_knobs(const gl_map* m, View& v, int Ts);
+// Device memory that the map's steps leave free where they can do without.
+void map_keep_free(gl_map* m, size_t bytes);
 
 // Validated camera of a pose and intrinsics (finite pose, positive focal
 // lengths, image size 1..16384); GL_ERR_INVALID otherwise.

@@ -139,12 +139,12 @@ double bytes_per_gaussian(int deg)
 }
 
 // Scratch of one step over views of P pixels in total (per-(view, Gaussian)
-// records and binning, per-instance and per-pixel buffers; an instance's share
-// of the split tiles' states is 24 bytes with 16x16 tiles and 512-record
-// segments).
+// records and binning, per-instance and per-pixel buffers).  The split tiles'
+// states of the default execution do not count: a request does without them
+// where they would take from the reserve (View::keep_free).
 double step_scratch(double views, double n, double P, double inst_per_px)
 {
-    return views * n * 170.0 + P * 110.0 + inst_per_px * P * 1.25 * 114.0;
+    return views * n * 170.0 + P * 110.0 + inst_per_px * P * 1.25 * 90.0;
 }
 
 void finish(gl_server* s, Req* q, const gl_result& res)
@@ -460,9 +460,11 @@ extern "C" gl_status gl_server_create(gl_map* map, const gl_server_config* cfg, 
     GL_CUDA_TRY(cudaStreamCreateWithPriority(&s->rstream, cudaStreamNonBlocking, prio_hi));
     for (Snap& sn : s->snap) GL_CUDA_TRY(cudaEventCreateWithFlags(&sn.ready, cudaEventDisableTiming));
     GL_TRY(s->rview.init());
+    s->rview.keep_free = (size_t)c.reserve_bytes;
     GL_TRY(publish(s.get()));
     GL_TRY(record_version(s.get()));
     GL_CUDA_TRY(cudaStreamSynchronize(map_stream(map)));
+    map_keep_free(map, (size_t)c.reserve_bytes);
     gl_server* raw = s.release();
     raw->tm = std::thread(mutation_worker, raw);
     raw->tr = std::thread(render_worker, raw);
@@ -606,6 +608,7 @@ extern "C" gl_status gl_server_destroy(gl_server* s)
     }
     if (s->tm.joinable()) s->tm.join();
     if (s->tr.joinable()) s->tr.join();
+    map_keep_free(s->map, 0);
     cudaStreamSynchronize(s->rstream);
     for (Snap& sn : s->snap) {
         for (DevBuf& b : sn.arr) b.release();

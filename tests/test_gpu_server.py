@@ -175,3 +175,52 @@ def test_map_size_cap():
     st = srv.stats()
     assert st["map_size"] <= cap and st["points_capped"] > 0
     srv.close()
+
+
+def _splitting_map(n, spread, scale, cam):
+    """A map whose lists the default execution splits, and its image with split and with whole lists."""
+    from paper_2404_06926_gb300 import binding
+    rng = np.random.default_rng(2)
+    params = dict(means=np.stack([rng.normal(0, spread, n), rng.normal(0, spread, n), rng.uniform(2, 3, n)], 1),
+                  log_scales=rng.uniform(scale, scale + 0.4, (n, 3)), quats=rng.normal(size=(n, 4)),
+                  logits=np.full(n, -5.0), sh=rng.normal(0, 0.5, (n, 1, 3)))
+    m = binding.Map(binding.default_config(n_sky=0, sh_degree=0, capacity_hint=n))
+    m.set_params({k: np.ascontiguousarray(v, np.float32) for k, v in params.items()})
+    split = m.render(cam).copy()
+    m.set_exec(segment=0)
+    whole = m.render(cam).copy()
+    m.set_exec(segment=-1)
+    assert not np.array_equal(split, whole)
+    torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    return m, split, whole
+
+
+def test_default_splitting_does_not_count_against_a_request():
+    """Free memory between what a render is taken to need (90 bytes an instance)
+    and that plus the split tiles' state (24 more): it is admitted."""
+    from paper_2404_06926_gb300 import binding
+    n, W, H = 4000, 2048, 1536
+    cam = scenes.camera(W, H, 3000.0, 3000.0, W / 2, H / 2)
+    m, split, _ = _splitting_map(n, 0.004, -5.2, cam)
+    P = W * H   # a first render is taken to have two instances a pixel, grown by a quarter
+    need = 170.0 * n + 110.0 * P + 12.0 * P + 2.0 * P * 1.25 * 90.0
+    state = 2.0 * P * 1.25 * 24.0
+    srv = binding.Server(m, reserve_bytes=int(torch.cuda.mem_get_info()[0] - need - state / 2))
+    r, img = srv.wait(srv.render(cam), 120)
+    srv.close()
+    assert r["status"] == 0 and np.array_equal(img, split)
+
+
+def test_default_splitting_leaves_the_reserve_alone():
+    """A render of many more instances than it was taken to have (52 MB of
+    scratch, 16 MB beside the reserve): the split tiles' state, which it can do
+    without, is not taken from the reserve; the image is that of whole lists."""
+    from paper_2404_06926_gb300 import binding
+    cam = scenes.camera(64, 48, 60.0, 60.0, 32.0, 24.0)
+    m, split, whole = _splitting_map(40_000, 0.2, -0.6, cam)
+    srv = binding.Server(m, reserve_bytes=int(torch.cuda.mem_get_info()[0] - (16 << 20)))
+    r, img = srv.wait(srv.render(cam), 120)
+    srv.close()
+    assert r["status"] == 0 and np.array_equal(img, whole)
+    assert np.array_equal(m.render(cam), split)   # the map's own renders split as before
