@@ -531,21 +531,22 @@ int loss_partials_needed(int W, int H)
 }
 
 namespace {
-// Tiles per SM from which a CTA takes all three channels of a tile: two waves
-// of CTAs.  Then no cluster waits for its slowest channel and the channels
-// share the rows in L1; below, a third of the chain per CTA counts more.  A
-// cluster and one CTA per tile: 105 and 97 us (1280x1024, 1,280 tiles), 850 and
-// 656 (12 views, 9.5k); with four CTAs per SM (an earlier form of the moments)
-// 13 and 26 us (256x192, 48), 29 and 36 (647x481, 336), 57 and 62 (957x717, 690);
-// the line lies at 1.2k.
-constexpr int kWholeTilesPerSm = 8;
+// Tiles per two SMs from which a CTA takes all three channels of a tile: one
+// and a half waves of three CTAs per SM.  Then no cluster waits for its slowest
+// channel and the channels share the rows in L1; below, a third of the chain per
+// CTA counts more.  A cluster and one CTA per tile, by tiles: 13 and 25 us (48),
+// 33.2 and 37.3 (336), 44.3 and 38.1 (456, one full wave), 48.9 and 51.2 (525), 56.1
+// and 58.2 (620), 61.7 and 59.4 (690), 67.9 and 67.6 (768), 78.3 and 69.0 (896), 108 and
+// 98 (1,280), 167 and 146 (2,040), 850 and 656 (9.5k, 12 views): from 684 tiles the
+// one CTA is never slower.
+constexpr int kWholeTilesPer2Sms = 9;
 
 gl_status launch_loss(const LossOne& one, const ViewDesc* views, int V, const float* rgb, float* dL, float lambda,
                       float* part, int tiles, cudaStream_t s)
 {
     GL_TRY(ensure_smem_limit(reinterpret_cast<const void*>(&k_loss_split), (int)kSmemBytes));
     GL_TRY(ensure_smem_limit(reinterpret_cast<const void*>(&k_loss), (int)kSmemBytes));
-    if (tiles < kWholeTilesPerSm * sm_count()) {
+    if (2 * (int64_t)tiles < kWholeTilesPer2Sms * (int64_t)sm_count()) {
         k_loss_split<<<3 * tiles, kThreads, kSmemBytes, s>>>(one, views, V, rgb, dL, lambda, part);
     } else {
         k_loss<<<tiles, kThreads, kSmemBytes, s>>>(one, views, V, rgb, dL, lambda, part);

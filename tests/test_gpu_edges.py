@@ -445,3 +445,9 @@ def test_batch_depth_reaches_the_backward_of_large_frames(bd):
         a, ref = gg[name].cpu().numpy().astype(np.float64)[vis].ravel(), np.asarray(g[name], np.float64)[vis].ravel()
         rel = np.abs(a - ref) / np.maximum(np.abs(ref), 1e-4 * np.abs(ref).max())
         assert np.median(rel) < 1e-3 and np.percentile(rel, 99) < 1e-2, (name, np.median(rel), np.percentile(rel, 99))
+
+
+@pytest.mark.parametrize("W,H", [(1151, 575), (1120, 608), (1151, 607)])   # 648, 665 and 684 tiles
+def test_loss_around_the_line_between_its_kernels(W, H):
+    """A cluster per tile below 4.5 tiles per SM (684 on 152 SMs), one CTA from there on."""
+    test_loss_sizes(W, H)
