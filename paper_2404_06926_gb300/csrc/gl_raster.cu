@@ -85,13 +85,15 @@ constexpr int kBackBatch = 4;   // segments whose sums one load round trip bring
 // for; four leave less idle at the rounds' barriers and overshoot the stop by
 // less, which counts once there is far more work than the chip holds
 // (8 and 4 warps: 79 and 112 us on 250k Gaussians at 640x512, 10k pixel
-// blocks; 184 and 216 us at 1280x1024, 41k; 185 and 184 us at 1920x1080, 65k;
-// 3,968 and 3,338 us on 12 views of 2M, 303k; the line lies at 88k).  (The staging and exchange of every
-// variant fit in 48 KB of static shared memory.)
+// blocks; 91 and 132 at 1280x1024, 41k; 1M Gaussians, one view: 241 and 303 us at
+// 65k blocks, 247 and 267 at 88k, 249 and 251 at 93k, 252 and 244 at 102k, 255 and 238
+// at 115k, 359 and 338 at 259k; 300k Gaussians: 115 and 113 at 88k, 125 and 120 at
+// 102k; 3,968 and 3,338 us on 12 views of 2M, 303k; the line lies at 95k).  (The
+// staging and exchange of every variant fit in 48 KB of static shared memory.)
 template <int NB, int D>
 constexpr int wpb_fwd(bool wide) { return D == 4 || NB == 8 ? 2 : (NB == 1 && D == 1 && wide ? 8 : 4); }
 // pixel blocks per resident warp from which CTAs of four warps are taken
-constexpr int kWideUnits = 24;
+constexpr int kWideUnits = 26;
 // registers: 80 a thread (24 warps per SM) at the default shape
 template <int NB, int D>
 constexpr int warps_fwd() { return D == 4 ? 12 : (NB == 1 && D == 1 ? 24 : 16); }
