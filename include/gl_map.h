@@ -214,8 +214,8 @@ GL_API gl_status gl_optimize_step(gl_map* map, const gl_keyframe* views, int32_t
  *                    (Gaussian, tile) instance and adds them per Gaussian
  *                    in a fixed order instead of with float atomics, so a
  *                    step's results are bit-identical from run to run (at
- *                    the cost of one more pass over 40 bytes per instance
- *                    and pixel block); batch_depth is then 32.
+ *                    the cost of one more pass over 48 bytes per instance
+ *                    and pixel block it reaches); batch_depth is then 32.
  *   exact_cull       1 (default): a (Gaussian, tile) pair of the 3-sigma
  *                    rectangle gets an instance only if the Gaussian can
  *                    reach alpha >= 1/255 at a pixel centre of the tile
@@ -239,10 +239,10 @@ GL_API gl_status gl_optimize_step(gl_map* map, const gl_keyframe* views, int32_t
  *                    sums their gradients in its registers while the
  *                    pixels' transmittance and blended colour pass from
  *                    lane to lane; 0: per-pixel backward (lanes own pixels,
- *                    each Gaussian's sums folded across the warp).  The
- *                    per-Gaussian backward works on 8 x 4 pixel blocks with
- *                    32-record batches whatever pixels_per_lane and
- *                    batch_depth say (those still drive the forward).
+ *                    then turn over and own Gaussians to add up their
+ *                    sums).  The per-Gaussian backward works on 8 x 4 pixel
+ *                    blocks with 32-record batches whatever pixels_per_lane
+ *                    and batch_depth say (those still drive the forward).
  * Apart from deterministic = 1, results differ between runs only by the
  * order of the backward's float atomics.
  * gl_map_create starts with {0, 0, 32, 1, 0, 0, -1, 1, 0}.  Errors: GL_ERR_INVALID. */

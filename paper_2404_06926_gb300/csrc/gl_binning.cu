@@ -234,10 +234,13 @@ __global__ void k_set_u64(uint64_t* p, uint64_t v0, uint64_t v1)
 constexpr int kOsThreads = 256;
 constexpr int kOsItems = 15;
 constexpr int kOsTile = kOsThreads * kOsItems;   // 3840 keys per tile
-// Up to kOsSmall keys a tile holds 2048 and a histogram thread 8: with a tile
-// per SM or less, a pass takes as long as one CTA does.  Six passes, tiles of
-// 2048 and 3840 keys: 42.6 and 50.7 us (250k Gaussians), 56 and 60 (500k), 79
-// and 78 (1M), 1,079 and 841 (12 views of 2M).
+// Up to kOsSmall keys a tile holds 2048 and a histogram thread 8: while all of a
+// pass's tiles are resident at once (three per SM) it takes as long as one CTA
+// does, and a smaller one is sooner done.  Both sorts of a view, tiles of 2048 and
+// 3840 keys, by Gaussians (and instances): 54 and 65 us (250k, 336k), 68 and 73
+// (500k, 661k), 73 and 77 (600k, 790k), 80 and 81 (700k, 919k), 88 and 84 (800k,
+// 1.05M), 100 and 92 (1M, 1.30M), 1,079 and 841 (12 views of 2M): they cross where the
+// keys of a sort do the line, which lies at 800k.
 constexpr int kOsItemsSmall = 8;
 constexpr int64_t kOsSmall = 800000;
 constexpr int kOsMaxPasses = 4;

@@ -65,11 +65,6 @@ namespace gl {
 namespace {
 
 constexpr int kWarpsPerBlock = 8;
-// Warps per CTA of the kernels that stage 32 NB records per warp: batches of
-// 128 and 256 records use 4 and 2 warps, so that every variant's staged hits
-// fit in 48 KB of shared memory with the same resident warps per SM.
-template <int NB>
-constexpr int wpb() { return NB <= 2 ? kWarpsPerBlock : 16 / NB; }
 // Prefetch slots (32 records each) of a batch of 32 NB records: the whole
 // next batch up to 64 records, one sub-batch ahead beyond.
 template <int NB>
@@ -94,7 +89,8 @@ template <int NB, int D>
 constexpr int wpb_fwd(bool wide) { return D == 4 || NB == 8 ? 2 : (NB == 1 && D == 1 && wide ? 8 : 4); }
 // pixel blocks per resident warp from which CTAs of four warps are taken
 constexpr int kWideUnits = 26;
-// registers: 80 a thread (24 warps per SM) at the default shape
+// registers: 80 a thread (24 warps per SM) at the default shape, which spill 92 to
+// 128 bytes
 template <int NB, int D>
 constexpr int warps_fwd() { return D == 4 ? 12 : (NB == 1 && D == 1 ? 24 : 16); }
 
@@ -709,7 +705,8 @@ __device__ __forceinline__ float warp_transpose_reduce16(float (&v)[16])
 // every variant's within 48 KB of static shared memory.
 template <int NB>
 constexpr int wpb_bwd() { return NB <= 4 ? 4 : 2; }
-// registers: 96 a thread (20 warps per SM) at the default shape
+// registers: 96 a thread (20 warps per SM) at the default shape (32 bytes spilled
+// without depth gradients)
 template <int NB, int D>
 constexpr int minb_bwd() { return (D > 1 ? 12 : (NB <= 2 ? 20 : 16)) / wpb_bwd<NB>(); }
 
@@ -762,8 +759,12 @@ __device__ __forceinline__ void bwd_turn_over(const RasterArgs& A, const RasterG
     const float2* row = W.sv + h * BW::S + part * BW::PS;
     const float4* pc = W.pix + part * 16;
     const float dya = in.y - (by + (float)(2 * part)), dyb = in.y - (by + (float)(2 * part + 1));
-    // even and odd columns apart: chains of four terms, then pairs of sums, which
-    // round no worse than a fold of the pixels' terms
+    // even and odd columns apart: chains of four terms (the column moments) or
+    // eight fused ones, then pairs of sums.  Against 64 bits the gradients are as
+    // far off as with a fold of the pixels' terms (rms of five gradients, 5k
+    // Gaussians at 256x192: 3.2 3.8 2.6 4.2 3.1e-6, folded 3.3 3.9 2.7 4.1 3.1e-6);
+    // chains of four throughout gain nothing and cost 3 to 11% of the half-warp
+    // kernel.
     float c0[2] = {0.f, 0.f}, c1[2] = {0.f, 0.f}, c2[2] = {0.f, 0.f}, cD[2] = {0.f, 0.f}, mxx[2] = {0.f, 0.f};
     float m0a[2] = {0.f, 0.f}, m0b[2] = {0.f, 0.f}, mxa[2] = {0.f, 0.f}, mxb[2] = {0.f, 0.f};
 #pragma unroll
@@ -994,6 +995,11 @@ __device__ __forceinline__ void bwd_item(int u, const RasterArgs& A, const Raste
 // 220 us (1M, 1280x1024), 92 -> 81 us (300k, 957x717), 3,959 -> 3,772 us (12
 // views of 2M).  The forward has no sums to add up and loses what its two
 // lists cost (185 -> 193 us, 1M; 3,347 -> 3,566 us): it keeps whole warps.
+// A large Gaussian's sums take twice as many additions.  Against 64 bits the
+// gradients of street maps are as far off as with whole warps (within 0.5% in
+// every output; 30k to 250k Gaussians, 400x300 to 640x480); those of 20k
+// Gaussians of tens of pixels at 400x300 a little further (quaternions 4.6e-6
+// instead of 3.9e-6, scales 4.5e-6 instead of 4.1e-6).
 constexpr int kRing = 48;    // three groups of 16: up to 16 waiting, a batch of 32 staged on top
 struct HalfRing {
     float4 r0[kRing], r1[kRing], r2[kRing];
@@ -1060,7 +1066,7 @@ __device__ __forceinline__ void half_turn_over(const RasterGrad& G, const BwdHal
     const float4 a = R.r0[at + (lane & 15)];
     const float2* row = W.sv + lane * BwdHalf::S;
     const float4* pc = W.pix + half * 16;
-    // chains of four to eight terms, then pairs of sums
+    // chains of four to eight terms, then pairs of sums (see bwd_turn_over)
     float c0[2] = {0.f, 0.f}, c1[2] = {0.f, 0.f}, c2[2] = {0.f, 0.f}, cD[2] = {0.f, 0.f}, mxx[2] = {0.f, 0.f};
     float m0[4] = {0.f, 0.f, 0.f, 0.f}, mx[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -1227,8 +1233,9 @@ __device__ __forceinline__ void bwd_half_item(int u, const RasterArgs& A, const 
     }
 }
 
-constexpr int kWpbHalf = 4;       // 43.5 KB of shared memory a CTA
-constexpr int kMinBlocksHalf = 5; // 96 registers, 20 warps per SM
+constexpr int kWpbHalf = 4;       // 37.0 KB of shared memory a CTA
+static_assert(sizeof(BwdHalf) * kWpbHalf == 37888, "five CTAs in an SM's 227 KB");
+constexpr int kMinBlocksHalf = 5; // 96 registers (32 bytes spilled), 20 warps per SM
 
 template <bool EXTRA>
 __global__ void __launch_bounds__(32 * kWpbHalf, kMinBlocksHalf) k_raster_bwd_half(RasterArgs A, RasterGrad G)
