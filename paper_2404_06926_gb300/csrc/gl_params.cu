@@ -237,9 +237,8 @@ __device__ __forceinline__ void mom_load(Mom4& x, const float* __restrict__ Mg, 
 
 // Adam on float4 c of a whole block's span: parameters from the staged rows sP,
 // the gradient from the rows sR (columns from `off`); elements of rows left
-// alone are written back unchanged.  The first three columns take lr0, the rest
-// lr: the DC band and the higher ones on the SH span (which is the DC band
-// alone at degree 0), the same rate twice on the others.
+// alone are written back unchanged.  On the SH span (WIDTH > 4) the first
+// three columns take lr0 (the DC band), the rest lr.
 template <int WIDTH, int NR, bool FULL>
 __device__ __forceinline__ void mom_apply(const Mom4& x, float* __restrict__ P, float* __restrict__ Mg,
                                           float* __restrict__ Vg, size_t base, int c, const float* sP, const float* sR,
@@ -253,7 +252,7 @@ __device__ __forceinline__ void mom_apply(const Mom4& x, float* __restrict__ P, 
 #pragma unroll
     for (int k = 0; k < 4; k++)
         if (FULL || ((upd >> q.rr[k]) & 1u))
-            adam1(pe[k], me[k], ve[k], sR[q.rr[k] * NR + off + q.ww[k]], q.ww[k] < 3 ? lr0 : lr, ad);
+            adam1(pe[k], me[k], ve[k], sR[q.rr[k] * NR + off + q.ww[k]], (WIDTH > 4 && q.ww[k] < 3) ? lr0 : lr, ad);
     __stcs(reinterpret_cast<float4*>(P + base) + c, make_float4(pe[0], pe[1], pe[2], pe[3]));
     __stcs(reinterpret_cast<float4*>(Mg + base) + c, make_float4(me[0], me[1], me[2], me[3]));
     __stcs(reinterpret_cast<float4*>(Vg + base) + c, make_float4(ve[0], ve[1], ve[2], ve[3]));

@@ -264,36 +264,6 @@ def test_expanded_rows(n, deg):
     assert np.array_equal(out["quats"], np.tile(np.float32([1, 0, 0, 0]), (added, 1)))
 
 
-@pytest.mark.parametrize("n", [31, 32, 97])   # a partial block alone, a whole one alone, three and a remainder
-@pytest.mark.parametrize("deg", [0, 1])
-@pytest.mark.parametrize("sparse", [0, 1])
-def test_every_band_moves_by_its_own_rate(n, deg, sparse):
-    """The first step from zero moments moves an entry by its group's learning
-    rate, in whole blocks as in the partial one, at degree 0 too."""
-    from paper_2404_06926_gb300 import binding
-    rng = np.random.default_rng(n + deg)
-    cam = scenes.camera(64, 48, 50.0, 50.0, 32.0, 24.0)
-    K = (deg + 1) ** 2
-    z = rng.uniform(2.0, 4.0, n)
-    params = dict(means=np.stack([rng.uniform(-0.4, 0.4, n) * z, rng.uniform(-0.3, 0.3, n) * z, z], 1).astype(np.float32),
-                  log_scales=rng.uniform(-2.5, -1.5, (n, 3)).astype(np.float32),
-                  quats=np.tile(np.float32([1, 0, 0, 0]), (n, 1)), logits=np.full(n, -1.0, np.float32),
-                  sh=rng.uniform(0.1, 0.3, (n, K, 3)).astype(np.float32))
-    lr = dict(lr_sh_dc=2.5e-3, lr_sh_rest=1e-4, lr_pos=1.6e-4, lr_opacity=0.05)
-    m = binding.Map(binding.default_config(n_sky=0, sh_degree=deg, capacity_hint=n, sparse_adam=sparse, **lr))
-    m.set_params(_dev(params))
-    m.optimize_step([(0, cam, np.zeros((48, 64, 3), np.float32))])
-    got = m.get_params()
-    # a black target: every visible Gaussian's colour has a clear gradient, so |move| = lr up to eps / |gradient|
-    # and the rounding of the stored value (2^-25 of at most 0.3)
-    seen = np.abs(got["sh"] - params["sh"])[:, 0].max(1) > 0
-    assert seen.sum() > 0.9 * n
-    assert np.allclose(np.abs(got["sh"] - params["sh"])[seen, 0], lr["lr_sh_dc"], rtol=1e-3, atol=1e-7)
-    if deg:
-        rest = np.abs(got["sh"] - params["sh"])[seen, 1:]
-        assert np.allclose(rest[rest > 0], lr["lr_sh_rest"], rtol=1e-3, atol=1e-7)
-
-
 @pytest.mark.parametrize("exposed", [False, True])
 @pytest.mark.parametrize("second", ["out_depth", "out_opacity"])
 def test_render_into_images_that_share_memory(exposed, second):
