@@ -541,9 +541,11 @@ struct FloatSum {
     }
     __device__ __forceinline__ void add(const FloatSum& o)
     {
-        add(o.h);
-        add(o.m);
-        add(o.l);
+        float e, r, q;
+        two_sum(h, o.h, h, e);
+        two_sum(m, o.m, m, q);
+        two_sum(m, e, m, r);
+        l = __fadd_rn(__fadd_rn(l, o.l), __fadd_rn(q, r));
     }
     __device__ __forceinline__ FloatSum xor_lane(int off) const
     {
@@ -559,16 +561,15 @@ struct FloatSum {
     __device__ __forceinline__ double value() const { return (double)h + ((double)m + (double)l); }
 };
 
-// The same over part[k], part[k + stride], ... (count of them) by a warp, in
-// double: the total in every lane.
-__device__ __forceinline__ double warp_double_sum(const float* __restrict__ part, int64_t count, int stride, int lane)
+// The value of such a sum of part[0], part[stride], ... (count of them): in
+// double, one after the other, where it left the range of a float.
+__device__ __forceinline__ double sum_value(const FloatSum& S, const float* __restrict__ part, int64_t count, int stride)
 {
-    double acc = 0.0;
+    if (S.finite()) return S.value();
+    double v = 0.0;
 #pragma unroll 1
-    for (int64_t i = lane; i < count; i += 32) acc += (double)part[i * stride];
-#pragma unroll 1
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(kFull, acc, off);
-    return acc;
+    for (int64_t i = 0; i < count; i++) v += (double)part[i * stride];
+    return v;
 }
 
 // mu' as (u_hi + u_lo, v_hi + v_lo); z > 0 is known (the decision passed)

@@ -423,7 +423,7 @@ k_loss(LossOne one, const ViewDesc* __restrict__ views, int V, const float* __re
 // Bound by latency: one CTA reads nblk x 14 floats in order (thread t takes
 // elements t, t + 1022, ...: 1022 = 73 x 14, so always the same partial),
 // eight loads in flight, then a warp per partial adds the 73 sums.
-// A warp per partial in double -> this: 13.3 -> 5.3 us (1280x1024).
+// A warp per partial in double -> this: 13.3 -> 5.2 us (1280x1024).
 constexpr int kRedBatch = 8;
 constexpr int kRedRows = 73;
 constexpr int kRedThreads = 1024;
@@ -436,7 +436,6 @@ k_loss_final(const float* __restrict__ part, int nblk, int W, int H, float lambd
 {
     __shared__ FloatSum sums[kRedRows * kNP];
     __shared__ FloatSum tot[kNP];
-    __shared__ double again[kNP];   // of the sums that overflowed
     __shared__ double s_invN;
     int begin = 0;
     float* Ev = nullptr;
@@ -475,30 +474,27 @@ k_loss_final(const float* __restrict__ part, int nblk, int W, int H, float lambd
     const int k = tid >> 5, lane = tid & 31;
     if (k < kNP) {
         FloatSum S{};
-        // rolled: the kernel runs once through its code, from a cold
-        // instruction cache
-#pragma unroll 1
-        for (int r = lane; r < kRedRows; r += 32) S.add(sums[r * kNP + k]);
-#pragma unroll 1
+        FloatSum q[3];
+#pragma unroll
+        for (int j = 0; j < 3; j++) q[j] = lane + 32 * j < kRedRows ? sums[(lane + 32 * j) * kNP + k] : FloatSum{};
+#pragma unroll
+        for (int j = 0; j < 3; j++) S.add(q[j]);
+#pragma unroll
         for (int off = 16; off > 0; off >>= 1) S.add(S.xor_lane(off));
         if (lane == 0) tot[k] = S;
-        if (__any_sync(kFull, !S.finite())) {
-            const double v = warp_double_sum(part + (size_t)begin * kNP + k, nblk, kNP, lane);
-            if (lane == 0) again[k] = v;
-        }
     }
     __syncthreads();
     // (few warps take the sums to double: its lanes are few)
     if (tid == 32) {
-        const double l1 = tot[12].finite() ? tot[12].value() : again[12];
-        const double ss = tot[13].finite() ? tot[13].value() : again[13];
+        const float* src = part + (size_t)begin * kNP;
+        const double l1 = sum_value(tot[12], src + 12, nblk, kNP), ss = sum_value(tot[13], src + 13, nblk, kNP);
         const double L = (1.0 - lambda) * l1 * s_invN + lambda * (1.0 - ss * s_invN);
         if (views) { if (loss_v) loss_v[blockIdx.x] = (float)L; }
         else if (loss_out) *loss_out = (float)L;
     }
     if (tid < 12) {
         const int i = tid;
-        const float g = (float)(tot[i].finite() ? tot[i].value() : again[i]);
+        const float g = (float)sum_value(tot[i], part + (size_t)begin * kNP + i, nblk, kNP);
         if (!views && dE_out) dE_out[i] = g;
         if (Ev && Em && !(abort && abort[1])) {
             const float m = b1 * Em[i] + (1.0f - b1) * g;

@@ -630,7 +630,7 @@ struct Jac6 {
 // loads in flight; CTA 0 reads and adds the eight CTAs' sums between two
 // cluster barriers (the first shows that all CTAs run, the second keeps their
 // shared memory until it has been read).  Bound by latency.
-// One CTA in double -> this: 34.9 -> 4.7 us (250k Gaussians).
+// One CTA in double -> this: 34.9 -> 4.2 us (250k Gaussians).
 constexpr int kPoseRows = 170;
 constexpr int kPoseThreads = 1024;
 constexpr int kPoseCtas = 8;
@@ -642,7 +642,6 @@ k_pose_reduce(const float* __restrict__ part, int npart, Jac6 J, float* __restri
     __shared__ FloatSum sums[kPoseRows * 6];
     __shared__ FloatSum mine[6];   // this CTA's sums
     __shared__ FloatSum tot[6];
-    __shared__ double again[6];    // of the sums that overflowed
     const int tid = threadIdx.x;
     constexpr int PER = kPoseRows * 6, STRIDE = PER * kPoseCtas;
     if (tid < PER) {
@@ -664,11 +663,10 @@ k_pose_reduce(const float* __restrict__ part, int npart, Jac6 J, float* __restri
     const int k = tid >> 5, lane = tid & 31;
     if (k < 6) {
         FloatSum S{};
-        // rolled: the kernel runs once through its code, from a cold
-        // instruction cache
-#pragma unroll 1
-        for (int r = lane; r < kPoseRows; r += 32) S.add(sums[r * 6 + k]);
-#pragma unroll 1
+#pragma unroll
+        for (int j = 0; j < (kPoseRows + 31) / 32; j++)
+            if (lane + 32 * j < kPoseRows) S.add(sums[(lane + 32 * j) * 6 + k]);
+#pragma unroll
         for (int off = 16; off > 0; off >>= 1) S.add(S.xor_lane(off));
         if (lane == 0) mine[k] = S;
     }
@@ -679,14 +677,10 @@ k_pose_reduce(const float* __restrict__ part, int npart, Jac6 J, float* __restri
         if (lane < kPoseCtas) S = cluster.map_shared_rank(mine, lane)[k];
         for (int off = kPoseCtas / 2; off > 0; off >>= 1) S.add(S.xor_lane(off));
         if (lane == 0) tot[k] = S;
-        if (__any_sync(kFull, !S.finite())) {
-            const double v = warp_double_sum(part + k, npart, 6, lane);
-            if (lane == 0) again[k] = v;
-        }
     }
     cluster.sync();
     if (blockIdx.x == 0 && tid < 6) {
-        const double v = tot[tid].finite() ? tot[tid].value() : again[tid];
+        const double v = sum_value(tot[tid], part + tid, npart, 6);
         double o = 0.0;
         for (int i = 0; i < 6; i++) o += (double)J.m[i * 6 + tid] * __shfl_sync(0x3fu, v, i);
         out6[tid] = (float)o;
