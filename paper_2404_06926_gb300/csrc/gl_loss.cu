@@ -373,14 +373,18 @@ loss_tile(LossOne one, const ViewDesc* __restrict__ views, int V, const float* _
         const float* g0 = cluster.map_shared_rank(gout, 0);
         const float* g1 = cluster.map_shared_rank(gout, 1);
         const float* g2 = cluster.map_shared_rank(gout, 2);
+        float s1 = 0.0f, s2 = 0.0f;   // on their way while the gradients are added
+        if (ch == 0 && tid < 2) {
+            s1 = cluster.map_shared_rank(chsum, 1)[tid];
+            s2 = cluster.map_shared_rank(chsum, 2)[tid];
+        }
 #pragma unroll
         for (int o = 0; o < AVR; o++) {
             const int gx = ox + c, gy = oy + r0 + o, i = (r0 + o) * LT + c;
             const float v = fmaf(f2, g2[i], fmaf(f1, g1[i], f0 * g0[i]));
             if (gx < W && gy < H) dL_drgb[3 * ((size_t)gy * W + gx) + ch] = v;
         }
-        if (ch == 0 && tid < 2)
-            prow[12 + tid] = chsum[tid] + cluster.map_shared_rank(chsum, 1)[tid] + cluster.map_shared_rank(chsum, 2)[tid];
+        if (ch == 0 && tid < 2) prow[12 + tid] = chsum[tid] + s1 + s2;
         cluster.sync();   // the shared memory read by the other CTAs stays until they are done
     } else {
         if (tid < kNP) {
