@@ -995,11 +995,6 @@ __device__ __forceinline__ void bwd_item(int u, const RasterArgs& A, const Raste
 // 220 us (1M, 1280x1024), 92 -> 81 us (300k, 957x717), 3,959 -> 3,772 us (12
 // views of 2M).  The forward has no sums to add up and loses what its two
 // lists cost (185 -> 193 us, 1M; 3,347 -> 3,566 us): it keeps whole warps.
-// A large Gaussian's sums take twice as many additions.  Against 64 bits the
-// gradients of street maps are as far off as with whole warps (within 0.5% in
-// every output; 30k to 250k Gaussians, 400x300 to 640x480); those of 20k
-// Gaussians of tens of pixels at 400x300 a little further (quaternions 4.6e-6
-// instead of 3.9e-6, scales 4.5e-6 instead of 4.1e-6).
 constexpr int kRing = 48;    // three groups of 16: up to 16 waiting, a batch of 32 staged on top
 struct HalfRing {
     float4 r0[kRing], r1[kRing], r2[kRing];
@@ -1235,20 +1230,49 @@ __device__ __forceinline__ void bwd_half_item(int u, const RasterArgs& A, const 
 
 constexpr int kWpbHalf = 4;       // 37.0 KB of shared memory a CTA
 static_assert(sizeof(BwdHalf) * kWpbHalf == 37888, "five CTAs in an SM's 227 KB");
-constexpr int kMinBlocksHalf = 5; // 96 registers (32 bytes spilled), 20 warps per SM
+// Instances per visible (view, Gaussian) pair up to which blocks are half-warps
+// (street maps have 1.3 to 1.5).  A half-warp block adds a row of its own, so a
+// large Gaussian's sums take twice as many additions: against 64 bits the
+// gradients are as far off with either block up to 28 instances a Gaussian, 2 to
+// 4% further with half-warps at 240, and on 20k Gaussians of 4 to 84 pixels (64
+// instances) the quaternions' 4.6e-6 instead of 3.9e-6, the scales' 4.5e-6 instead
+// of 4.1e-6.  Whole-warp blocks' times there, 1280x960: 440 -> 485 us (63 instances), 442
+// -> 482 (219), 574 -> 495 (1,150).  The counts are on the device, so the choice is made
+// there; the whole-warp item is a call, which leaves the half-warp loop's registers
+// as they are (inlined, the loop took 3% longer).
+constexpr uint64_t kHalfInstances = 32;
+constexpr int kMinBlocksHalf = 5; // 96 registers (at most 8 bytes spilled), 20 warps per SM
 
 template <bool EXTRA>
-__global__ void __launch_bounds__(32 * kWpbHalf, kMinBlocksHalf) k_raster_bwd_half(RasterArgs A, RasterGrad G)
+__device__ __noinline__ void bwd_item_call(int u, const RasterArgs& A, const RasterGrad& G, BwdWarp<1, 1>& W, int lane)
 {
-    __shared__ BwdHalf sw[kWpbHalf];
+    bwd_item<EXTRA, 1, 1, false>(u, A, G, W, lane);
+}
+
+template <bool EXTRA>
+__global__ void __launch_bounds__(32 * kWpbHalf, kMinBlocksHalf)
+k_raster_bwd_half(const __grid_constant__ RasterArgs A, const __grid_constant__ RasterGrad G)
+{
+    __shared__ union {
+        BwdHalf half;
+        BwdWarp<1, 1> whole;
+    } sw[kWpbHalf];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int nunits = (int)A.ctl[6] * A.nblk;
     int u = A.work ? next_unit(A.work, lane) : blockIdx.x * kWpbHalf + w;
-    while (u < nunits) {
-        bwd_half_item<EXTRA>(u, A, G, sw[w], lane);
-        __syncwarp();
-        if (!A.work) break;
-        u = next_unit(A.work, lane);
+    if (A.ctl[0] <= kHalfInstances * A.ctl[9]) {
+        while (u < nunits) {
+            bwd_half_item<EXTRA>(u, A, G, sw[w].half, lane);
+            __syncwarp();
+            if (!A.work) break;
+            u = next_unit(A.work, lane);
+        }
+    } else {
+        while (u < nunits) {
+            bwd_item_call<EXTRA>(u, A, G, sw[w].whole, lane);
+            if (!A.work) break;
+            u = next_unit(A.work, lane);
+        }
     }
 }
 
@@ -1818,8 +1842,8 @@ void bwd_dispatch(int nb, int pd, bool det, bool pg, const RasterArgs& A, const 
         // were asked for and take the kernels that have them.
         // Whole- and half-warp blocks by footprint, 1280x960, standard
         // deviation in pixels: 1 (600k Gaussians) 245 and 188 us, 4 (100k) 224
-        // and 193, 10 (30k) 297 and 268, 30 (6k) 482 and 439, 80 (2k) 495 and
-        // 588: only Gaussians as large as the frame's quarter cost more.
+        // and 193, 10 (30k) 297 and 268.  (Maps of much larger Gaussians take
+        // whole-warp blocks within the kernel, see kHalfInstances.)
         const int grid = grid_for(k_raster_bwd_half<EXTRA>, units, persistent, kWpbHalf);
         k_raster_bwd_half<EXTRA><<<grid, 32 * kWpbHalf, 0, s>>>(A, G);
     } else if (nb == 4) {   // deeper batches: one pixel per lane

@@ -421,3 +421,37 @@ def test_batch_depth_reaches_the_backward_of_large_frames(bd):
 def test_loss_around_the_line_between_its_kernels(W, H):
     """A cluster per tile below 4.5 tiles per SM (684 on 152 SMs), one CTA from there on."""
     test_loss_sizes(W, H)
+
+
+@pytest.mark.parametrize("scale,small", [(-4.5, True), (-3.2, True), (-1.5, False)])
+@pytest.mark.parametrize("seg,persistent", [(0, 0), (64, 1)])
+@pytest.mark.parametrize("extra", [False, True])
+def test_blocks_by_footprint(scale, small, seg, persistent, extra):
+    """Frames of more pixel blocks than resident warps: Gaussians of up to 32
+    instances each take half-warp blocks, larger ones whole-warp blocks.  Either
+    way the gradients are those of the kernel that has whole-warp blocks only
+    (batches of 64): the terms are the same, the sums' order is not (2-norm 1e-4)."""
+    from paper_2404_06926_gb300 import binding
+    rng = np.random.default_rng(7)
+    W, H, n = 331, 300, 900
+    cam = scenes.camera(W, H, 250.0, 250.0, W / 2, H / 2)
+    z = rng.uniform(1.0, 6.0, n)
+    q = rng.normal(size=(n, 4))
+    params = dict(means=np.stack([rng.uniform(-0.6, 0.6, n) * z, rng.uniform(-0.5, 0.5, n) * z, z], 1).astype(np.float32),
+                  log_scales=rng.uniform(scale - 0.3, scale + 0.3, (n, 3)).astype(np.float32),
+                  quats=(q / np.linalg.norm(q, axis=1, keepdims=True)).astype(np.float32),
+                  logits=rng.normal(0, 1, n).astype(np.float32), sh=rng.normal(0, 0.5, (n, 1, 3)).astype(np.float32))
+    p = _dev(params)
+    t = lambda *s: torch.from_numpy(rng.normal(size=s).astype(np.float32)).cuda() * 1e-3
+    d = [t(H, W, 3), t(H, W) if extra else None, t(H, W) if extra else None]
+    res = []
+    for bd in (32, 64):
+        ctx = binding.Ctx()
+        ctx.set_exec(batch_depth=bd, segment=seg, persistent=persistent)
+        ctx.forward(p, cam, 16)
+        visible = int((ctx.preprocess(n, "cuda")["radius"] > 0).sum())
+        assert (ctx.num_instances() <= 32 * visible) == small
+        res.append(ctx.backward(p, *d)[0])
+    for k in NAMES:
+        a, b = res[0][k].double(), res[1][k].double()
+        assert float((a - b).norm()) <= 1e-4 * float(b.norm()), k
